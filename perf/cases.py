@@ -294,11 +294,12 @@ class _Form:
         M, D, lam = _reference(d, N, d == 3)
         to = lambda a: torch.tensor(np.asarray(a, dtype=np.float64), device=dev)  # noqa: E731
         self.M, self.D, self.Mf = to(M), [to(x) for x in D], to(_reference(d - 1, N, d == 3)[0])
-        V = torch.tensor(X[E], device=dev)                                    # K, d+1, d
+        V = X[E]                                                              # K, d+1, d
         T = V[:, 1:] - V[:, :1]
-        self.vol = torch.linalg.det(T).abs() / math.factorial(d)
-        g = torch.linalg.inv(T).transpose(1, 2)                               # grad lambda_1..d
+        self.vol = to(np.abs(np.linalg.det(T)) / math.factorial(d))
+        g = to(np.linalg.inv(T).transpose(0, 2, 1))                           # grad lambda_1..d
         self.g = torch.cat([-g.sum(1, keepdim=True), g], 1)
+        V = to(V)
         self.x = torch.einsum("nv,kvd->knd", to(lam), V)
         ex = _lattice(d, N)
         of = {a: i for i, a in enumerate(_lattice(d - 1, N))}
