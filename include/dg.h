@@ -61,8 +61,8 @@ typedef enum {
 } dg_status;
 
 /* DG_F64: FP64 in/out with the mesh's FP64 kernel (DG_KERNEL_* below; built-in:
- *         from degree 3 up the dense products run on the BF16 tensor cores with
- *         exact integer slicing, relative error ~1e-13 of |A||u|; that path scales
+ *         from degree 3 up the dense products run on the FP16 tensor cores with
+ *         exact integer slicing, relative error ~1e-15 of |A||u|; that path scales
  *         each element's data by a power of two and rebuilds results from their
  *         exponent bits, so it takes finite fields whose nonzero element
  *         magnitudes lie between about 1e-250 and 1e250);
@@ -93,11 +93,10 @@ typedef struct dg_mesh dg_mesh; /* opaque; owned by the library until dg_mesh_de
  *                     pieces per operand scaled by powers of two; degrees 1-8. Needs u and
  *                     Au 16-byte aligned (otherwise DG_KERNEL_TENSOR runs instead).
  *   DG_KERNEL_TC64:   FP64 only: both products on the Blackwell tensor cores (tcgen05,
- *                     exact 7-bit integer slicing, 8 slices, accumulators in tensor memory)
- *                     and the pointwise stage in float-float on the FP32 pipe; all degrees.
- *                     Intermediates carry 48 bits (float-float), so where the operator's
- *                     terms cancel strongly (a node next to an element 2^60 larger, at
- *                     N = 10) an entry's error can reach a few 1e-12 of |A||u|.
+ *                     exact integer slicing, 7 digits of 8 bits, accumulators in tensor
+ *                     memory) and the pointwise stage in 64-bit fixed point, each element's
+ *                     data at its own power-of-two scale; all degrees. An element with an
+ *                     infinity or a NaN, and its neighbours, give NaN.
  *                     Handles finite fields whose magnitudes stay within the double range
  *                     at every stage (about 1e-250..1e250, as DG_KERNEL_TENSOR). */
 enum { DG_KERNEL_AUTO = 0, DG_KERNEL_TILE = 1, DG_KERNEL_GEMM = 2, DG_KERNEL_TENSOR = 3, DG_KERNEL_EPT = 4,
@@ -194,7 +193,7 @@ dg_status dg_operator_apply(const dg_mesh* mesh, int degree, dg_prec prec, int B
  * enqueued behind the caller's earlier work on `stream`; the caller's later
  * work on `stream` runs after the last copy. With the tcgen05 FP64 kernel (the
  * FP64 default from degree 3) the copies run on two copy streams of the mesh,
- * in chunks of rows: a chunk's gradient product starts once its input has
+ * in chunks of rows: a chunk's first phase starts once its input has
  * arrived, and a chunk's output copy starts as soon as its output product has
  * written it. The host buffers must stay valid until `stream` has passed the
  * call (synchronise it before reading Au_host). Calls on one mesh must not

@@ -339,6 +339,7 @@ dg_status dg_mesh_setup(int N, int64_t Nv, const double* VX, const double* VY, i
     const std::vector<float> gx32(gx.begin(), gx.end());
     if (ce == cudaSuccess) ce = cudaMalloc(&m->geox32, sizeof(float) * 16 * K);
     if (ce == cudaSuccess) ce = cudaMemcpy(m->geox32, gx32.data(), sizeof(float) * 16 * K, cudaMemcpyHostToDevice);
+    if (ce == cudaSuccess) ce = build_fixed_geometry(m);
   }
   if (ce == cudaSuccess) ce = ensure_ops(m, N);
   // the tensor kernels' operator slices of the mesh degree: built here so that
@@ -366,6 +367,8 @@ dg_status dg_mesh_destroy(dg_mesh* m) {
   cudaFree(m->ih32);
   cudaFree(m->geox);
   cudaFree(m->geox32);
+  cudaFree(m->gfix);
+  cudaFree(m->gfix_ex);
   cudaFree(m->geo64);
   cudaFree(m->geo32);
   cudaFree(m->conn);

@@ -1,762 +1,840 @@
 // SIPDG apply in FP64 on the Blackwell tensor cores (tcgen05), without the
 // FP64 pipe (GB300 runs FP64 arithmetic at 1/64 of its FP32 rate).
 //
-// The operator of Eq. ellipticOp3 as the two dense products of apply_tensor.cu,
-//   C1 = [Dr; Ds] u                 and   Au = OB Y,
-// Y = [wr, ws | 1/2 nr sJ [u], 1/2 ns sJ [u], -sJ ({n.grad u} + tau [u]) (| lambda J u)]
-// (OB = [Br Bs | Dr_f^T Mf  Ds_f^T Mf | E_f Mf (| M)]: the Helmholtz term enters
-// as extra columns of Y and rows of OB), in three kernels:
-//  * tc64_gemm: out[row] = A X[row] for 128 rows per tile, exact to FP64
-//    accuracy by integer slicing (the error-free splitting of Ozaki et al.,
-//    Numer. Algorithms 59, 2012): every operator row scaled by a power of two
-//    and cut into 8 signed 7-bit slices on the host, every data row the same
-//    way on the device (integer operations on the double's bits); the 36 slice
-//    products with i + j <= 7 run as tcgen05.mma (BF16 operands from shared
-//    memory, FP32 accumulators in tensor memory, one accumulator per slice
-//    exponent i + j: integer sums below 2^24 for K <= 256 and up to 4 products,
-//    exact); the accumulators are recombined by Horner's rule in float-float
-//    and rebuilt as doubles from the exponent bits. Data slices are written by
-//    the threads into a double-buffered shared-memory chunk (32 columns) while
-//    the previous chunk's products run; operator blocks (48 rows x 32 columns,
-//    8 slices) arrive by bulk copy.
-//  * the gradient product C1 = [Dr; Ds] u (rows interleaved, so one thread
-//    holds ur and us of a node) with an epilogue that forms the volume columns
-//    of Y (wr, ws), the Helmholtz columns and every element's face data
-//    (u, n.grad u at its face nodes) in float-float on the FP32 pipe;
-//  * tc64_face_fill: the face columns of Y (jumps and averages against the
-//    neighbour's face data, penalty of Eq. PenaltyParameter), float-float,
-//    one thread per face-node entry;
-//  * the output product Au = OB Y, a plain tc64_gemm launch.
-// Accuracy: relative error near 2^-44 of |A||u| (the slicing's), as the mma.sync path.
+// The operator of Eq. ellipticOp3, element by element, is one dense product of
+// a reference matrix with a column X of the element's own and its neighbours'
+// data, Au = OB X with
+//   X  = [Grr u, Grs u, Gss u | 1/2 nr sJ [u], 1/2 ns sJ [u], -sJ ({n.grad u} + tau [u]) (| lambda J u)]
+//   OB = [S_rr, S_rs + S_sr, S_ss | Dr_f^T Mf, Ds_f^T Mf, E_f Mf (| M)],   S_ab = D_a^T M D_b,
+// so that the volume term needs no gradient; the only derivative left is
+// n.grad u at the face nodes. Two kernels:
+//  * t64_trace: per 128 elements the rows of [Dr; Ds] at the 3N boundary nodes
+//    times u, from which q = sJ n.grad u at every face node; writes u and q as
+//    fixed-point integers at the element's own scale, column-major (entry i of
+//    element e at [i][e], so that a warp's 32 elements are contiguous);
+//  * t64_output: forms X chunk by chunk in registers from those integers (own
+//    and neighbours'), cuts it into digits in shared memory and multiplies; X
+//    never reaches memory.
+// Constants are in the kernel of D_a and S_ab, so both kernels work on v = u - u0,
+// u0 the element's first node, and add the difference of the two u0 to a jump:
+// a smooth field's columns are as small as its gradient's, which keeps the
+// digits for the result (on u itself an apply to a smooth field had 20 times
+// the error: S_ab is N^2 times larger than what it yields there).
+// Both products are exact to FP64 accuracy by integer slicing (Ozaki et al.,
+// Numer. Algorithms 59, 2012) into seven base-256 digits (fix64.cuh): the 34
+// digit products with i + j <= 7 run as tcgen05.mma in FP16 with FP32
+// accumulators in tensor memory, one accumulator per digit sum i + j. The
+// operator's digits are stacked along N, so one instruction multiplies data
+// digit j with the operator's digits 0 .. 7 - j into the accumulators j .. 7:
+// 7 to 12 instructions per 16 columns in place of 34, each reading the data
+// digit once.
+// Accuracy: columns of X carry 56 bits of a bound on the row, rounded to nearest
+// (a bias that all elements share would be a smooth source, which a solve
+// amplifies), and the digit products left out weigh 2^-60 of the largest. Against
+// 64-bit arithmetic the relative error of an apply is 0.9e-15 (N = 3) to 1.2e-14
+// (N = 10) on random fields, 1.5 times the FP64-pipe kernel's.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
 
 #include "dg_internal.h"
+#include "fix64.cuh"
 #include "tc05.cuh"
 
 namespace dgx {
 namespace {
 
-constexpr int kT = 128;                      // rows per tile (MMA M)
-constexpr int kKC = 32;                      // data columns per chunk
-constexpr int kNC = 48;                      // output columns per pass (MMA N)
-constexpr int kSl = 8;                       // slices of 7 bits
-// Longest sum: a slice product is below 127^2 in magnitude, and an accumulator
-// group with up to 4 products over 256 terms stays below 4 * 256 * 127^2 <
-// 2^24, an integer FP32 represents exactly; groups with more products carry
-// weights below 2^-28 of the leading one (the fifth group stays exact up to
-// 208 terms: 5 * 208 * 127^2 < 2^24).
-constexpr int kMaxDepth = 256;
-// The output product at depths above this runs per column block (volume,
-// face, Helmholtz), each block with its own row exponent, accumulated into Au.
-constexpr int kSplitDepth = 208;
-constexpr int kABytes = kSl * kT * kKC * 2;  // one data chunk, 8 slices: 64 KB
-constexpr int kBBytes = kSl * kNC * kKC * 2; // one operator block, 8 slices: 24 KB
-constexpr int kASlice = kT * kKC * 2, kBSlice = kNC * kKC * 2;
-constexpr int kNodeTab = 72;  // entries of the gradient product's node-to-face table (Np <= 66)
-// the tail: 10 mbarriers, slot, 2 flags, the node-to-face table, the tile's face normals
-// (MODE 1: n.grad r and n.grad s of the three faces as float-float, [3 faces][4][kT])
-constexpr int kSmem = 2 * kABytes + 2 * kBBytes + 4 * kT * 4 + 12 * 8 + kNodeTab * 4 + 12 * kT * 4;
+using fx::kDigits;
+using fx::kSums;
+using fx::Split;
 
-__device__ int g_tc64_err;
+constexpr int kT = 128;       // rows (elements x right-hand sides) per tile: MMA M
+constexpr int kItems = 16;    // items of X per chunk, three columns each
+constexpr int kChunkSlice = kT * 3 * kItems * 2;       // one digit of a chunk: 12 KB
+constexpr int kChunkBytes = kDigits * kChunkSlice;     // 84 KB
+constexpr int kTraceN = 32;                            // output columns (16 boundary nodes) per pass of t64_trace
+constexpr int kTraceStep = kDigits * kTraceN * 16 * 2; // operator block of one pass and 16 columns
+constexpr int trace_smem(int ks) {
+  return kDigits * kT * ks * 32 + (ks != 3 ? 2 : 1) * ks * kTraceStep + 6 * kT * 4 + 6 * 8;
+}
+constexpr int kCoefs = 12;    // Grr, Grs, Gss | per face nr sJ, ns sJ | per face -sJ tau0
 
-// exponent e with |v| < 2^e (-1100 for zero)
-__device__ __forceinline__ int exp_bound64(double v) {
-  const int E = int((__double_as_longlong(v) >> 52) & 0x7ff);
-  return E == 0 ? -1100 : E - 1022;
+__device__ int g_t64_err;
+
+__device__ __forceinline__ void mbar_arrive(uint64_t* b) {
+  asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.shared::cta.b64 st, [%0];\n}\n" ::"r"(tc::smem_addr(b)) : "memory");
+}
+// A wait that gave up sets the block's abort flag, and every later wait then
+// returns at once: all warps run to the end of their loops (their named
+// barriers stay matched) and the block ends.
+__device__ __forceinline__ bool aborted(volatile int* flag) { return __any_sync(0xffffffffu, *flag != 0); }
+__device__ __forceinline__ void wait(uint64_t* b, uint32_t parity, volatile int* abort_flag) {
+  if (!aborted(abort_flag) && !tc::mbar_wait(b, parity)) *abort_flag = 1;
+}
+__device__ __forceinline__ void bar_sync(int id, int threads) {
+  asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(threads) : "memory");
 }
 
-// |v| 2^{56 - E} as a 56-bit integer (|v| < 2^E) and its sign
-__device__ __forceinline__ uint64_t fixed56(double v, int E, uint32_t& sgn) {
-  const unsigned long long b = __double_as_longlong(v);
-  const int Eb = int((b >> 52) & 0x7ff);
-  sgn = uint32_t(b >> 63);
-  if (Eb == 0) return 0ull;
-  const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
-  const int sh = Eb - 1075 + 56 - E;  // <= 3 whenever |v| < 2^E
-  if (sh >= 0) return sh < 11 ? (m << sh) : 0ull;
-  return sh > -63 ? (m >> (-sh)) : 0ull;
+__device__ __forceinline__ int64_t elem_of(int64_t row, int64_t K) { return row < K ? row : row % K; }
+
+// accumulator columns d .. d + rows += data digit x the operator's stacked rows
+__device__ __forceinline__ void issue_rows(uint32_t d, uint64_t a, uint64_t b, int rows, uint32_t acc) {
+  const int n0 = rows <= 256 ? rows : ((rows / 2 + 15) & ~15);
+  tc::mma_ss(d, a, b, tc::idesc_f16(128, n0, false), acc);
+  if (n0 < rows) tc::mma_ss(d + n0, a, b + ((n0 * 32) >> 4), tc::idesc_f16(128, rows - n0, false), acc);
 }
-// exact double of (h + l) 2^sc for a float-float pair with |l| small against h
-__device__ __forceinline__ double ff_to_double(float h, float l, int sc) {
-  const float s = __fadd_rn(h, l);
-  l = __fsub_rn(l, __fsub_rn(s, h));
-  h = s;
-  const uint32_t uh = __float_as_uint(h), ul = __float_as_uint(l);
-  const int eh = int((uh >> 23) & 0xffu), el = int((ul >> 23) & 0xffu);
-  if (eh == 0) return 0.0;
-  long long M = (long long)((uh & 0x7fffffu) | 0x800000u) << 29;  // h in a 53-bit frame
-  if (el != 0) {
-    const int sh = 29 - (eh - el);
-    const long long ml = (long long)((ul & 0x7fffffu) | 0x800000u);
-    long long Ml = sh >= 0 ? (ml << sh) : (sh > -40 ? (ml >> (-sh)) : 0ll);
-    if ((uh ^ ul) >> 31) Ml = -Ml;
-    M += Ml;
+// The digit products i + j <= 7 of 16 columns: data digits (slices of `aslice`
+// bytes at a) with the operator's (nc stacked rows each at b); `first` starts the sums.
+__device__ __forceinline__ void issue_step(uint32_t d, uint64_t a, int aslice, uint64_t b, int nc, bool first) {
+  issue_rows(d, a, b, kDigits * nc, first ? 0u : 1u);  // sums 0 .. 6
+  a += aslice >> 4;
+  if (first) {  // sums 1 .. 6 are there, sum 7 starts here
+    issue_rows(d + nc, a, b, (kDigits - 1) * nc, 1u);
+    issue_rows(d + kDigits * nc, a, b + (((kDigits - 1) * nc * 32) >> 4), nc, 0u);
+  } else {
+    issue_rows(d + nc, a, b, kDigits * nc, 1u);
   }
-  int e = eh;
-  if (M >= (1ll << 53)) {
-    M >>= 1;
-    ++e;
-  } else if (M < (1ll << 52)) {
-    M <<= 1;
-    --e;
+#pragma unroll 1
+  for (int j = 2; j < kDigits; ++j) {
+    a += aslice >> 4;
+    issue_rows(d + j * nc, a, b, (kSums - j) * nc, 1u);
   }
-  const unsigned long long bits = ((unsigned long long)(uh >> 31) << 63) |
-                                  ((unsigned long long)(e - 127 + 1023 + sc) << 52) |
-                                  ((unsigned long long)M & 0xFFFFFFFFFFFFFull);
-  return __longlong_as_double((long long)bits);
 }
 
-// ------------------------------------------------------------------ float-float
-struct ff {
-  float h, l;
-};
-__device__ __forceinline__ ff ff_renorm(float s, float e) {
-  const float h = __fadd_rn(s, e);
-  return ff{h, __fsub_rn(e, __fsub_rn(h, s))};
-}
-__device__ __forceinline__ ff ff_add(ff x, ff y) {
-  const float s = __fadd_rn(x.h, y.h);
-  const float bb = __fsub_rn(s, x.h);
-  float e = __fadd_rn(__fsub_rn(x.h, __fsub_rn(s, bb)), __fsub_rn(y.h, bb));
-  e = __fadd_rn(e, __fadd_rn(x.l, y.l));
-  return ff_renorm(s, e);
-}
-__device__ __forceinline__ ff ff_neg(ff x) { return ff{-x.h, -x.l}; }
-__device__ __forceinline__ ff ff_sub(ff x, ff y) { return ff_add(x, ff_neg(y)); }
-__device__ __forceinline__ ff ff_mul(ff x, ff y) {
-  const float p = __fmul_rn(x.h, y.h);
-  float e = __fmaf_rn(x.h, y.h, -p);
-  e = __fmaf_rn(x.h, y.l, e);
-  e = __fmaf_rn(x.l, y.h, e);
-  return ff_renorm(p, e);
-}
-__device__ __forceinline__ ff ff_pow2(ff x, float p2) { return ff{x.h * p2, x.l * p2}; }  // exact scaling
-
-// x 2^{-R} as float-float (top 47 bits of the double; parts below the FP32
-// range of the scaled value, far below the largest input, flush to zero)
-__device__ __forceinline__ ff d2ff(double x, int R) {
-  const unsigned long long b = __double_as_longlong(x);
-  const int Eb = int((b >> 52) & 0x7ff);
-  const int e = Eb - 1023 - R;
-  if (Eb == 0 || e < -125) return ff{0.f, 0.f};
-  const uint32_t sgn = uint32_t(b >> 63) << 31;
-  const unsigned long long m = b & 0xFFFFFFFFFFFFFull;
-  const float h = __uint_as_float(sgn | (uint32_t(min(e, 127) + 127) << 23) | uint32_t(m >> 29));
-  const uint32_t r23 = uint32_t(m >> 6) & 0x7fffffu;  // the next 23 bits
-  const int el = e - 46;
-  float l = 0.f;
-  if (el >= -126 && r23) {
-    l = (__uint_as_float(0x4B000000u | r23) - 8388608.0f) * __uint_as_float(uint32_t(el + 127) << 23);
-    l = __uint_as_float(__float_as_uint(l) | sgn);
-  }
-  return ff{h, l};
-}
-
-// ------------------------------------------------------------------ the GEMM
-__device__ __forceinline__ int fnode(int N, int f, int j) {
+__device__ __forceinline__ int node_of(int N, int f, int j) {  // local node of face f's j-th node
   auto rs = [N](int row) { return row * (N + 1) - row * (row - 1) / 2; };
   return f == 0 ? j : (f == 1 ? rs(j) + (N - j) : rs(N - j));
 }
 
-// Horner's rule over the 8 slice sums of one output column: (h, l) with
-// h + l = sum_s acc_s 2^{-7 s} (float-float)
-__device__ __forceinline__ ff horner8(const uint32_t (&acc)[kSl][4], int c) {
-  float h = __uint_as_float(acc[kSl - 1][c]), l = 0.f;
-#pragma unroll
-  for (int s = kSl - 2; s >= 0; --s) {
-    const float a = __uint_as_float(acc[s][c]);
-    const float hs = h * 0.0078125f, ls = l * 0.0078125f;
-    const float sum = __fadd_rn(a, hs);
-    const float bb = __fsub_rn(sum, a);
-    const float err = __fadd_rn(__fsub_rn(a, __fsub_rn(sum, bb)), __fsub_rn(hs, bb));
-    h = sum;
-    l = __fadd_rn(ls, err);
+// Per-element coefficients in fixed point, one exponent for each kind (|c| < 2^e):
+// word i of element e at tab[i K + e], exponents in ex (G, n sJ, sJ tau0, J).
+__global__ void k_fix_geometry(int64_t K, const double* __restrict__ gx, int2* __restrict__ tab,
+                               short4* __restrict__ ex) {
+  const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (e >= K) return;
+  const double* g = gx + 16 * e;
+  double c[kCoefs];
+  for (int i = 0; i < 3; ++i) c[i] = g[1 + i];
+  for (int f = 0; f < 3; ++f) {
+    const double sJ = g[4 + 4 * f + 2];
+    c[3 + 2 * f] = g[4 + 4 * f] * sJ;
+    c[4 + 2 * f] = g[4 + 4 * f + 1] * sJ;
+    c[9 + f] = -g[4 + 4 * f + 3] * sJ;
   }
-  return ff_renorm(h, l);
+  int eg = fx::kZeroExp, ec = fx::kZeroExp, et = fx::kZeroExp;
+  for (int i = 0; i < 3; ++i) eg = max(eg, fx::exp_bound(c[i]));
+  for (int i = 3; i < 9; ++i) ec = max(ec, fx::exp_bound(c[i]));
+  for (int i = 9; i < 12; ++i) et = max(et, fx::exp_bound(c[i]));
+  for (int i = 0; i < kCoefs; ++i) {
+    const Split s = fx::split(fx::fix<62>(c[i], i < 3 ? eg : (i < 9 ? ec : et)));
+    tab[int64_t(i) * K + e] = make_int2(s.h, s.l);
+  }
+  ex[e] = make_short4(short(eg), short(ec), short(et), short(fx::exp_bound(g[0])));
 }
 
-// Arguments of the gradient product's epilogue (MODE 1): the rows of A are
-// [Dr; Ds] interleaved (column 2n = ur at node n, 2n + 1 = us), and instead of
-// C1 the epilogue writes the volume columns of Y (wr, ws), the Helmholtz
-// columns lambda J u, and every element's face data FN = (u, n.grad u) at its
-// face nodes (outward normal of the element itself).
-// Y and the face data are column-major with leading dimension ldc (a multiple
-// of 32 rows), so a warp's 32 rows write 256 contiguous bytes per column.
-struct GradOut {
-  int N;
-  int64_t K;
-  const double* gx;  // derived geometry, 16 words per element
-  double* Y;         // [columns][ldc]
+__device__ __forceinline__ Split coef(const int2* p) {
+  const int2 v = __ldg(p);
+  return Split{v.x, v.y};
+}
+
+// ------------------------------------------------------------------ boundary derivatives
+struct TraceArgs {
+  int N, passes, aligned;
+  int64_t K, rows, row0;   // rows of this launch, the first one's global index
+  const double* u;         // this launch's first row
+  const int2* tab;
+  const short4* tex;
+  const uint8_t* ops;      // [pass][16 columns][7 digits x 32 rows][16]
+  int ea;                  // common exponent of the operator
+  long long* Iu;           // [Np][ldc], first row of this launch
+  long long* Iq;           // [3 (N + 1)][ldc]
   int64_t ldc;
-  int helm;
-  double lambda;
-  double *FNu, *FNd;  // [3 (N+1)][ldc]: u and n.grad u at the element's face nodes
-  int* exy;     // [rows]: largest exponent of the row's Y values (for the output product)
-  int* exf;     // [rows] or null: set to "none" here when the face columns keep their own exponent
-  int64_t row0;  // global index of the launch's first row (Y, FNu, FNd, exy, exf start there)
+  int4* ex;                // per row: exponents of v, q's scale, q, u
+  double* u0;              // per row: u at the first node
 };
 
-// out[r][c] = sum_k A[c][k] X[r][k] for r < rows, c < M, k < Kd (A sliced in
-// blocks of kNC rows x kKC columns: block (nc, kc) at (nc KCH + kc) kBBytes).
-//
-// Warp-specialised pipeline over a stream of data chunks (tile, output pass
-// nc, column chunk kc), chunk g using shared-memory buffer g & 1:
-//  * warps 0-15 (four threads per row of the 128-row tile) find each row's
-//    scale exponent, slice chunk g into buffer g & 1 once the products of
-//    chunk g - 2 have released it (mbarrier `empty`), signal `full`, and after
-//    a pass's last chunk wait for its accumulators (`acc_full`), drain them
-//    (Horner's rule, epilogue) and release them (`acc_empty`);
-//  * warp 16 loads operator block g by bulk copy, waits for `full`, issues the
-//    36 slice products per 16 columns from one lane and commits to `empty`
-//    (and to `acc_full` after a pass's last chunk); before a pass's first
-//    chunk it waits until the previous pass has been drained.
-// No CTA-wide barrier in the steady state; every wait is bounded in time.
-constexpr int kSlicers = 512;  // threads of warps 0-15
-template <int MODE>
-__global__ void __launch_bounds__(kSlicers + 32, 1) tc64_gemm(int64_t rows, int M, int Kd, int NCH, int KCH,
-                                                              const double* __restrict__ X, int64_t ldx, int vec2,
-                                                              int xcol,
-                                                              const int* __restrict__ ex_given,
-                                                              const uint8_t* __restrict__ Bops,
-                                                              const int* __restrict__ ea, double* __restrict__ out,
-                                                              int64_t ldo, int accum, GradOut go) {
+// KS: 16-column steps of u (Np <= 16 KS). Eight warps (two threads per row)
+// slice a tile and drain its products, one warp issues copies and products;
+// two blocks per SM up to KS = 3 (shared memory 110 KB, tensor memory 256
+// columns each), so one block's slicing runs under the other's products. The
+// tile's rows arrive by one bulk copy into the space that then takes their
+// digits (each thread reads its values before the first digit is written), so
+// the row-major u is read with full sectors.
+template <int KS>
+__global__ void __launch_bounds__(288, KS <= 3 ? 2 : 1) t64_trace(const TraceArgs a) {
   extern __shared__ __align__(1024) uint8_t sm[];
-  uint8_t* sA = sm;                        // [2][8 slices][128 rows][32] canonical
-  uint8_t* sB = sm + 2 * kABytes;          // [2][8 slices][48 rows][32] canonical
-  int* pmax = reinterpret_cast<int*>(sB + 2 * kBBytes);  // [4][kT]
-  // full[2], empty[2], bfull[2], acc_full, acc_empty, bempty[2]
-  uint64_t* bars = reinterpret_cast<uint64_t*>(pmax + 4 * kT);
-  uint64_t *full = bars, *empty = bars + 2, *bfull = bars + 4, *acc_full = bars + 6, *acc_empty = bars + 7,
-           *bempty = bars + 8;
-  uint32_t* slot = reinterpret_cast<uint32_t*>(bars + 10);
-  int* abort_flag = reinterpret_cast<int*>(slot + 1);
-  int* tile_abort = abort_flag + 1;  // the slicers' common copy of abort_flag at a tile's start
-  // MODE 1: per node n the face nodes it is, packed (fa + 1) | ja << 4 | (fb + 1) << 8 | jb << 12
-  // (face f, position j; a corner is on two faces; 0 in the face field: none)
-  int* nodetab = reinterpret_cast<int*>(reinterpret_cast<uint8_t*>(bars) + 12 * 8);
-  float* snrm = reinterpret_cast<float*>(nodetab + kNodeTab);  // [f][nr.h, nr.l, ns.h, ns.l][kT]
+  constexpr int kSlice = kT * KS * 16 * 2;
+  constexpr bool kResident = KS != 3;  // all passes' operator blocks stay in shared memory (KS = 3: one at a time)
+  constexpr int kPass = KS * kTraceStep;
+  uint8_t* sB = sm + kDigits * kSlice;
+  int* pmax = reinterpret_cast<int*>(sB + (kResident ? 2 : 1) * kPass);  // [2 halves][exponent of v, of u, bits of q][kT]
+  uint64_t* bars = reinterpret_cast<uint64_t*>(pmax + 6 * kT);
+  uint64_t *ufull = bars, *full = bars + 1, *accf = bars + 2, *acce = bars + 3, *bfull = bars + 4;
+  uint32_t* slot = reinterpret_cast<uint32_t*>(bars + 5);
+  volatile int* abort_flag = reinterpret_cast<int*>(slot + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int64_t ntiles = (rows + kT - 1) / kT;
-  // with at most two data chunks per row, both stay in the two buffers for all
-  // output passes of a tile: sliced once per tile instead of once per pass
-  const bool resident = KCH <= 2 && NCH > 1;
+  const int N = a.N, Np = (N + 1) * (N + 2) / 2;
+  const int64_t ntiles = (a.rows + kT - 1) / kT;
   if (tid == 0) {
-    for (int i = 0; i < 2; ++i) {
-      tc::mbar_init(full + i, kSlicers / 32);  // one arrival per slicing warp
-      tc::mbar_init(empty + i, 1);             // the products' commit
-      tc::mbar_init(bfull + i, 1);             // the bulk copy
-    }
-    tc::mbar_init(acc_full, 1);
-    tc::mbar_init(acc_empty, kSlicers / 32);
-    for (int i = 0; i < 2; ++i) tc::mbar_init(bempty + i, 1);  // an operator stage's products completed
+    tc::mbar_init(ufull, 1);
+    tc::mbar_init(full, 8);
+    tc::mbar_init(accf, 1);
+    tc::mbar_init(acce, 8);
+    tc::mbar_init(bfull, 1);
     *abort_flag = 0;
     tc::mbar_init_fence();
   }
-  if (warp == 0) tc::tmem_alloc(slot, 512);
-  if (MODE == 1 && tid < (go.N + 1) * (go.N + 2) / 2 && tid < kNodeTab) {
-    const int N = go.N, n = tid;
-    int rrow = 0;  // n's row of constant s
-    while (n >= (rrow + 1) * (N + 1) - (rrow + 1) * rrow / 2) ++rrow;
-    const int rs0 = rrow * (N + 1) - rrow * (rrow - 1) / 2, len = N + 1 - rrow;
-    int fa = -1, ja = 0, fb = -1, jb = 0;
-    if (rrow == 0) fa = 0, ja = n;  // face 0, j = n
-    if (n == rs0 + len - 1) {       // face 1, j = row
-      if (fa < 0) fa = 1, ja = rrow;
-      else fb = 1, jb = rrow;
-    }
-    if (n == rs0 && fb < 0) {  // face 2, j = N - row
-      if (fa < 0) fa = 2, ja = N - rrow;
-      else fb = 2, jb = N - rrow;
-    }
-    nodetab[n] = (fa + 1) | (ja << 4) | ((fb + 1) << 8) | (jb << 12);
-  }
+  if (warp == 0) tc::tmem_alloc(slot, 256);
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
   const uint32_t tb = *slot;
-  constexpr uint32_t idesc = tc::idesc_f16(128, kNC, true);
+  // a tile's rows arrive by bulk copy where address and size are multiples of 16 bytes
+  auto bulk_rows = [&](int64_t tile) -> uint32_t {
+    const int64_t left = a.rows - tile * kT;
+    const uint32_t bytes = uint32_t(left < kT ? left : kT) * uint32_t(Np) * 8u;
+    return a.aligned && (bytes & 15u) == 0 ? bytes : 0u;
+  };
 
-  if (warp == kSlicers / 32) {
-    // ================= products
-    uint32_t g = 0, pass = 0, it = 0;
-    const uint64_t adesc0 = tc::smem_desc(tc::smem_addr(sA), 128, (kKC / 8) * 128);
-    const uint64_t bdesc0 = tc::smem_desc(tc::smem_addr(sB), 128, (kKC / 8) * 128);
-    for (int64_t tile = blockIdx.x; tile < ntiles && !*abort_flag; tile += gridDim.x, ++it) {
-      for (int nc = 0; nc < NCH; ++nc, ++pass) {
-        // the accumulators are free once the previous pass has been drained
-        if (pass > 0 && !tc::mbar_wait(acc_empty, (pass - 1) & 1u)) *abort_flag = 1;
-        tc::fence_after();
-        for (int kc = 0; kc < KCH; ++kc, ++g) {
-          const uint32_t bs = g & 1u;                 // operator stage
-          const uint32_t bd = resident ? kc : bs;     // data buffer
-          // the operator stage is free once chunk g - 2's products completed
-          if (g >= 2 && !tc::mbar_wait(bempty + bs, ((g - 2) >> 1) & 1u)) *abort_flag = 1;
-          if (lane == 0) {
-            tc::mbar_expect_tx(bfull + bs, kBBytes);
-            tc::bulk_g2s(sB + bs * kBBytes, Bops + size_t(nc * KCH + kc) * kBBytes, kBBytes, bfull + bs);
-          }
-          __syncwarp();
-          // the data chunk: sliced once per chunk, or (resident) once per tile for all passes
-          if (!resident && !tc::mbar_wait(full + bd, (g >> 1) & 1u)) *abort_flag = 1;
-          if (resident && nc == 0 && !tc::mbar_wait(full + bd, it & 1u)) *abort_flag = 1;
-          if (!tc::mbar_wait(bfull + bs, (g >> 1) & 1u)) *abort_flag = 1;
-          tc::fence_after();
-          if (lane == 0) {
-            const uint64_t ab = adesc0 + ((bd * kABytes) >> 4), bb = bdesc0 + ((bs * kBBytes) >> 4);
-            uint32_t started = kc > 0 ? 0xffu : 0u;
-#pragma unroll
-            for (int ks = 0; ks < kKC / 16; ++ks)
-#pragma unroll
-              for (int i = 0; i < kSl; ++i)
-#pragma unroll
-                for (int j = 0; j < kSl - i; ++j) {
-                  const int s = i + j;
-                  tc::mma_ss(tb + s * kNC, ab + ((j * kASlice + ks * 256) >> 4), bb + ((i * kBSlice + ks * 256) >> 4),
-                             idesc, (started >> s) & 1u);
-                  started |= 1u << s;
-                }
-            tc::mma_commit(bempty + bs);
-            if (!resident || nc == NCH - 1) tc::mma_commit(empty + bd);  // the data buffer is free
-            if (kc == KCH - 1) tc::mma_commit(acc_full);
-          }
-          __syncwarp();
-        }
+  if (warp == 8) {
+    const uint64_t ad = tc::smem_desc(tc::smem_addr(sm), 128, KS * 256);
+    const uint64_t bd = tc::smem_desc(tc::smem_addr(sB), 128, 256);
+    uint32_t loads = 0, it = 0, pc = 0;
+    auto load_ops = [&](int pass0, int n) {
+      if (lane == 0) {
+        tc::mbar_expect_tx(bfull, n * kPass);
+        tc::bulk_g2s(sB, a.ops + size_t(pass0) * kPass, n * kPass, bfull);
       }
-    }
-  } else {
-    // ================= slicing and epilogue
-    const int e = (warp & 3) * 32 + lane;
-    const int q = warp >> 2;
-    const uint32_t lanebase = uint32_t((warp & 3) * 32) << 16;
-    uint32_t g = 0, pass = 0, it = 0;
-    auto load8 = [&](const double* xr, bool live, int k0, double (&v)[8]) {
-      if (xcol) {  // column-major X: element (row, k) at xr[k ldx], xr = X + row
-#pragma unroll
-        for (int t = 0; t < 8; ++t) v[t] = (live && k0 + t < Kd) ? __ldg(xr + int64_t(k0 + t) * ldx) : 0.0;
-      } else if (live && vec2 && k0 + 8 <= Kd) {
-        const double2* p2 = reinterpret_cast<const double2*>(xr + k0);
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-          const double2 w = __ldg(p2 + t);
-          v[2 * t] = w.x;
-          v[2 * t + 1] = w.y;
-        }
-      } else {
-#pragma unroll
-        for (int t = 0; t < 8; ++t) v[t] = (live && k0 + t < Kd) ? __ldg(xr + k0 + t) : 0.0;
+      ++loads;
+    };
+    auto load_u = [&](int64_t tile) {
+      const uint32_t bytes = bulk_rows(tile);
+      if (bytes && lane == 0) {
+        tc::mbar_expect_tx(ufull, bytes);
+        tc::bulk_g2s(sm, a.u + tile * kT * Np, bytes, ufull);
       }
     };
-    // output product (row exponents given): the last chunk of a tile requests the
-    // next tile's first chunk and exponent (vn, En), so that their latency overlaps
-    // the drain
-    bool have_next = false;
-    int En = 0;
-    double vn[8];  // the next chunk's values (loaded one chunk ahead)
-    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
-      // every slicer takes the same decision to stop (they meet at named barriers below)
-      asm volatile("bar.sync 1, %0;\n" ::"r"(kSlicers) : "memory");
-      if (tid == 0) *reinterpret_cast<volatile int*>(tile_abort) = *reinterpret_cast<volatile int*>(abort_flag);
-      if (MODE == 1 && q < 3) {  // face q's normal metric of this row, once per tile (read by the drains)
-        const int64_t rw = tile * kT + e;
-        const double* gq = go.gx + 16 * (((rw < rows ? rw : 0) + go.row0) % go.K) + 4 + 4 * q;
-        const ff nr = d2ff(__ldg(gq), 0), ns = d2ff(__ldg(gq + 1), 0);
-        snrm[(q * 4 + 0) * kT + e] = nr.h;
-        snrm[(q * 4 + 1) * kT + e] = nr.l;
-        snrm[(q * 4 + 2) * kT + e] = ns.h;
-        snrm[(q * 4 + 3) * kT + e] = ns.l;
-      }
-      asm volatile("bar.sync 1, %0;\n" ::"r"(kSlicers) : "memory");
-      if (*reinterpret_cast<volatile int*>(tile_abort)) break;
-      const int64_t row = tile * kT + e;
-      const bool live = row < rows;
-      const double* xr = xcol ? X + (live ? row : 0) : X + (live ? row : 0) * ldx;
-      // scale exponent of the row: a bound |X[row][k]| < 2^E, given by the producer
-      // of X or found here
-      int E;
-      if (ex_given) {
-        E = have_next ? En : (live ? __ldg(ex_given + row) : 0);
-        if (E == -1100) E = 0;
-      } else {
-        int em = -1100;
-        if (live) {
-          double v[2][8];
-          for (int kc = 0; kc < KCH; kc += 2) {
-            load8(xr, live, kc * kKC + 8 * q, v[0]);
-            load8(xr, live && kc + 1 < KCH, (kc + 1) * kKC + 8 * q, v[1]);
-#pragma unroll
-            for (int t = 0; t < 8; ++t) em = max(em, max(exp_bound64(v[0][t]), exp_bound64(v[1][t])));
-          }
-        }
-        asm volatile("bar.sync 1, %0;\n" ::"r"(kSlicers) : "memory");  // pmax free (previous tile read it)
-        pmax[q * kT + e] = em;
-        asm volatile("bar.sync 1, %0;\n" ::"r"(kSlicers) : "memory");
-        E = max(max(pmax[e], pmax[kT + e]), max(pmax[2 * kT + e], pmax[3 * kT + e]));
-        if (E == -1100) E = 0;
-      }
-      if (!have_next) load8(xr, live, 8 * q, vn);
-      have_next = false;
-      int ymax = -1100;  // MODE 1: largest exponent of the Y columns this thread writes
-      float gh[6];  // MODE 1: Grr, Grs, Gss as float-float
-      const double* gg = nullptr;  // MODE 1: the row's element geometry
-      if (MODE == 1) {
-        gg = go.gx + 16 * (((live ? row : 0) + go.row0) % go.K);
-#pragma unroll
-        for (int t = 0; t < 3; ++t) {
-          const ff gf = d2ff(__ldg(gg + 1 + t), 0);
-          gh[2 * t] = gf.h;
-          gh[2 * t + 1] = gf.l;
-        }
-      }
-      for (int nc = 0; nc < NCH; ++nc, ++pass) {
-        for (int kc = 0; kc < KCH; ++kc, ++g) {
-          if (resident && nc > 0) continue;  // the tile's chunks are still in the buffers
-          const uint32_t b = resident ? uint32_t(kc) : (g & 1u);
-          double v[8];
-#pragma unroll
-          for (int t = 0; t < 8; ++t) v[t] = vn[t];
-          {  // request the next chunk of this row (the next pass starts again at chunk 0)
-            const int kn = kc + 1 < KCH ? kc + 1 : 0;
-            if (kc + 1 < KCH || (nc + 1 < NCH && !resident)) {
-              load8(xr, live, kn * kKC + 8 * q, vn);
-            } else if (MODE == 0 && ex_given && nc + 1 == NCH && tile + gridDim.x < ntiles) {
-              const int64_t nrow = row + int64_t(gridDim.x) * kT;
-              const bool nlive = nrow < rows;
-              load8(xcol ? X + (nlive ? nrow : 0) : X + (nlive ? nrow : 0) * ldx, nlive, 8 * q, vn);
-              En = nlive ? __ldg(ex_given + nrow) : 0;
-              have_next = true;
-            }
-          }
-          // each value's 56-bit fixed-point magnitude as two 28-bit halves, and its sign
-          // as the pair (s, c) with fma(2^23 + x, s, c) = +-x exactly for 0 <= x < 2^23
-          uint32_t hi[8], lo[8];
-          float sm[8], sc[8];
-#pragma unroll
-          for (int t = 0; t < 8; ++t) {
-            uint32_t sgn;
-            const uint64_t I = fixed56(v[t], E, sgn);
-            hi[t] = uint32_t(I >> 28);
-            lo[t] = uint32_t(I) & 0xFFFFFFFu;
-            sm[t] = sgn ? -1.0f : 1.0f;
-            sc[t] = sgn ? 8388608.0f : -8388608.0f;
-          }
-          // buffer b is free once the products that read it completed: chunk g - 2's, or
-          // (resident) the previous tile's last pass
-          if (!resident && g >= 2 && !tc::mbar_wait(empty + b, ((g - 2) >> 1) & 1u)) *abort_flag = 1;
-          if (resident && it >= 1 && !tc::mbar_wait(empty + b, (it - 1) & 1u)) *abort_flag = 1;
-          uint8_t* dst = sA + b * kABytes + (e >> 3) * 512 + q * 128 + (e & 7) * 16;
-#pragma unroll
-          for (int j = 0; j < kSl; ++j) {
-            // slice j: 7 bits of the magnitude below bit 56 - 7j, as a signed float,
-            // whose upper 16 bits are its BF16 pattern (at most 8 significant bits)
-            uint32_t fb[8];
-#pragma unroll
-            for (int t = 0; t < 8; ++t) {
-              const uint32_t x = ((j < 4 ? hi[t] : lo[t]) >> (21 - 7 * (j & 3))) & 127u;
-              fb[t] = __float_as_uint(__fmaf_rn(__uint_as_float(0x4B000000u | x), sm[t], sc[t]));
-            }
-            uint4 w;  // value 2i in the low half of word i, value 2i + 1 in the high half
-            w.x = __byte_perm(fb[0], fb[1], 0x7632);
-            w.y = __byte_perm(fb[2], fb[3], 0x7632);
-            w.z = __byte_perm(fb[4], fb[5], 0x7632);
-            w.w = __byte_perm(fb[6], fb[7], 0x7632);
-            *reinterpret_cast<uint4*>(dst + j * kASlice) = w;
-          }
-          tc::fence_async_smem();
-          __syncwarp();
-          if (lane == 0) asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.shared::cta.b64 st, [%0];\n}\n" ::"r"(
-                                          tc::smem_addr(full + b))
-                                      : "memory");
-        }
-        // drain: output columns [12q, 12q + 12) of this pass
-        if (!tc::mbar_wait(acc_full, pass & 1u)) *abort_flag = 1;
+    load_ops(0, kResident ? a.passes : 1);
+    if (int64_t(blockIdx.x) < ntiles) load_u(blockIdx.x);
+    for (int64_t tile = blockIdx.x; tile < ntiles && !aborted(abort_flag); tile += gridDim.x, ++it) {
+      wait(full, it & 1u, abort_flag);
+      for (int p = 0; p < a.passes; ++p, ++pc) {
+        wait(bfull, (loads - 1) & 1u, abort_flag);
+        if (pc > 0) wait(acce, (pc - 1) & 1u, abort_flag);
         tc::fence_after();
+        if (lane == 0) {
+          const uint64_t b0 = bd + ((kResident ? p * kPass : 0) >> 4);
 #pragma unroll 1
-        for (int p = 0; p < 3; ++p) {
-          const int c0 = 12 * q + 4 * p;
-          uint32_t acc[kSl][4];
-#pragma unroll
-          for (int s = 0; s < kSl; ++s) {
-            uint32_t vv[4];
-            tc::tmem_ld4(tb + lanebase + s * kNC + c0, vv);
-#pragma unroll
-            for (int c = 0; c < 4; ++c) acc[s][c] = vv[c];
-          }
-          tc::tmem_wait_ld();
-          if (p == 2) {  // the accumulators are read: release them to the next pass
-            tc::fence_before();
-            __syncwarp();
-            if (lane == 0) asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.shared::cta.b64 st, [%0];\n}\n" ::"r"(
-                                            tc::smem_addr(acc_empty))
-                                        : "memory");
-          }
-          if (MODE == 0) {
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-              const int col = nc * kNC + c0 + c;
-              if (live && col < M) {
-                // value = 2^{ea + E - 14} sum_s acc_s 2^{-7 s}
-                const ff hl = horner8(acc, c);
-                const double v = ff_to_double(hl.h, hl.l, __ldg(ea + col) + E - 14);
-                if (accum) out[row * ldo + col] += v;  // (the Helmholtz or face block of a split product)
-                else out[row * ldo + col] = v;
-              }
-            }
-          } else {
-            // nodes n = col / 2: (ur, us) in columns (2n, 2n + 1)
-            const int N = go.N, Np = (N + 1) * (N + 2) / 2, Nfp = N + 1, NFN = 3 * Nfp;
-#pragma unroll
-            for (int c = 0; c < 4; c += 2) {
-              const int n = (nc * kNC + c0 + c) >> 1;
-              if (live && n < Np) {
-                const int er = __ldg(ea + 2 * n), es = __ldg(ea + 2 * n + 1);
-                const int ec = max(er, es);
-                ff ur = horner8(acc, c), us = horner8(acc, c + 1);
-                ur = ff_pow2(ur, __uint_as_float(uint32_t(127 + er - ec) << 23));
-                us = ff_pow2(us, __uint_as_float(uint32_t(127 + es - ec) << 23));
-                const int S = ec + E - 14;  // ur, us, wr, ws, n.grad u all carry 2^S
-                const ff grr{gh[0], gh[1]}, grs{gh[2], gh[3]}, gss{gh[4], gh[5]};
-                const ff wr = ff_add(ff_mul(grr, ur), ff_mul(grs, us));
-                const ff ws = ff_add(ff_mul(grs, ur), ff_mul(gss, us));
-                double* yr = go.Y + row;  // column c of this row at yr[c ldc]
-                const int64_t ldc = go.ldc;
-                const double dwr = ff_to_double(wr.h, wr.l, S), dws = ff_to_double(ws.h, ws.l, S);
-                yr[n * ldc] = dwr;
-                yr[(Np + n) * ldc] = dws;
-                ymax = max(ymax, max(exp_bound64(dwr), exp_bound64(dws)));
-                const double un = __ldg(X + row * ldx + n);
-                if (go.helm) {
-                  const int eu = exp_bound64(un);
-                  const ff lj = ff_mul(d2ff(go.lambda, 0), d2ff(__ldg(gg), 0));
-                  const ff vv = ff_mul(lj, d2ff(un, eu));
-                  const double dv = ff_to_double(vv.h, vv.l, eu);
-                  yr[(2 * Np + 3 * NFN + n) * ldc] = dv;
-                  ymax = max(ymax, exp_bound64(dv));
-                }
-                // face data at the face nodes this node is (a corner belongs to two faces)
-                const int nt = nodetab[n];
-                const int fa = (nt & 15) - 1, ja = (nt >> 4) & 15, fb = ((nt >> 8) & 15) - 1, jb = (nt >> 12) & 15;
-#pragma unroll
-                for (int t = 0; t < 2; ++t) {
-                  const int f = t == 0 ? fa : fb, j = t == 0 ? ja : jb;
-                  if (f >= 0) {
-                    const ff nr{snrm[(f * 4 + 0) * kT + e], snrm[(f * 4 + 1) * kT + e]};
-                    const ff ns{snrm[(f * 4 + 2) * kT + e], snrm[(f * 4 + 3) * kT + e]};
-                    const ff dn = ff_add(ff_mul(nr, ur), ff_mul(ns, us));
-                    const int64_t fi = int64_t(f * Nfp + j) * ldc + row;
-                    go.FNu[fi] = un;
-                    go.FNd[fi] = ff_to_double(dn.h, dn.l, S);
-                  }
-                }
-              }
-            }
-          }
+          for (int ks = 0; ks < KS; ++ks)
+            issue_step(tb, ad + ((ks * 256) >> 4), kSlice, b0 + ((ks * kTraceStep) >> 4), kTraceN, ks == 0);
+          tc::mma_commit(accf);
         }
-      }
-      if (MODE == 1) {  // the row's largest Y exponent so far (the face columns add theirs)
-        asm volatile("bar.sync 1, %0;\n" ::"r"(kSlicers) : "memory");
-        pmax[q * kT + e] = ymax;
-        asm volatile("bar.sync 1, %0;\n" ::"r"(kSlicers) : "memory");
-        if (q == 0 && live)
-          go.exy[row] = max(max(pmax[e], pmax[kT + e]), max(pmax[2 * kT + e], pmax[3 * kT + e]));
-        if (q == 0 && live && go.exf) go.exf[row] = -1100;  // raised by the face fill
+        __syncwarp();
+        const bool last = p + 1 == a.passes;
+        if (!kResident || last) {  // the products are done: their operands' space is free
+          wait(accf, pc & 1u, abort_flag);
+          if (!kResident && a.passes > 1 && (!last || tile + gridDim.x < ntiles)) load_ops(last ? 0 : p + 1, 1);
+          if (last && tile + gridDim.x < ntiles) load_u(tile + gridDim.x);
+        }
       }
     }
+    // nothing is left in flight when the block ends
+    wait(bfull, (loads - 1) & 1u, abort_flag);
+  } else {
+    const int e = (warp & 3) * 32 + lane, half = warp >> 2;
+    const uint32_t lanebase = uint32_t((warp & 3) * 32) << 16;
+    const double* su = reinterpret_cast<const double*>(sm);
+    uint32_t it = 0, pc = 0, bulks = 0;
+    int* pm = pmax + half * 3 * kT + e;
+    int4 xprev{};
+    // a row's exponents are complete once both its threads have seen their part of q:
+    // written behind the next barrier (the next tile's, or the last one)
+    auto write_exponents = [&](int64_t row) {
+      if (half != 0 || row >= a.rows) return;
+      const int bits = pmax[2 * kT + e] | pmax[5 * kT + e];  // of |q|'s upper words
+      xprev.z = xprev.y + 7 - __clz(bits);                   // |q| < 2^{64 - clz} at scale 2^{57-eq}
+      a.ex[row] = xprev;
+    };
+    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
+      const int64_t row = tile * kT + e;
+      const bool live = row < a.rows;
+      if (bulk_rows(tile)) {
+        wait(ufull, bulks & 1u, abort_flag);
+        ++bulks;
+      } else {  // every product that read the space has completed (accf below)
+        const int64_t left = a.rows - tile * kT;
+        const int n = int(left < kT ? left : kT) * Np;
+        for (int i = tid; i < n; i += 256) reinterpret_cast<double*>(sm)[i] = __ldg(a.u + tile * kT * Np + i);
+        bar_sync(1, 256);
+      }
+      // this thread's columns: 8-column groups half, half + 2, ...
+      double v[KS * 8];
+      const double u0 = live ? su[e * Np] : 0.0;
+      int ev = fx::kZeroExp, eu = fx::kZeroExp;
+#pragma unroll
+      for (int ks = 0; ks < KS; ++ks)
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+          const int n = (2 * ks + half) * 8 + t;
+          const double u = live && n < Np ? su[e * Np + n] : u0;
+          v[ks * 8 + t] = u - u0;
+          eu = max(eu, fx::exp_bound(u));
+          ev = max(ev, fx::exp_bound(v[ks * 8 + t]));
+        }
+      pm[0] = ev;
+      pm[kT] = eu;
+      bar_sync(1, 256);  // exponents written, and the rows read before digits overwrite them
+      if (it > 0) write_exponents(row - int64_t(gridDim.x) * kT);
+      ev = max(pmax[e], pmax[3 * kT + e]);
+      eu = max(pmax[kT + e], pmax[4 * kT + e]);
+      if (ev >= fx::kBadExp) eu = fx::kBadExp;
+      const int64_t el = live ? elem_of(a.row0 + row, a.K) : 0;
+      const int eq = a.ea + ev + __ldg(reinterpret_cast<const short*>(a.tex + el) + 1) + 3;
+      xprev = make_int4(ev, eq, 0, eu);
+      if (live && half == 0) a.u0[row] = u0;
+      int qbits = 0;
+#pragma unroll
+      for (int ks = 0; ks < KS; ++ks) {
+        long long x[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+          const int n = (2 * ks + half) * 8 + t;
+          x[t] = fx::fix<59>(v[ks * 8 + t], ev);
+          if (live && n < Np) a.Iu[int64_t(n) * a.ldc + row] = x[t];
+          x[t] = (x[t] + 4) >> 3;
+        }
+        fx::digits8(x, sm + (e >> 3) * (KS * 256) + (2 * ks + half) * 128 + (e & 7) * 16, kSlice);
+      }
+      tc::fence_async_smem();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(full);
+      for (int p = 0; p < a.passes; ++p, ++pc) {
+        wait(accf, pc & 1u, abort_flag);
+        tc::fence_after();
+        const int b0 = 16 * p + 8 * half;  // this warp's boundary nodes of the pass
+        int f = b0 / N, j = b0 - f * N;    // node b is the j-th of face f; a corner also ends the face before it
+#pragma unroll 1
+        for (int i = 0; i < 4; ++i) {
+          const int b = b0 + 2 * i;
+          if (b >= 3 * N) break;
+          float acc[2][2][kSums];
+          __syncwarp();
+#pragma unroll
+          for (int s = 0; s < kSums; ++s) {
+            uint32_t w[4];
+            tc::tmem_ld4(tb + lanebase + s * kTraceN + 16 * half + 4 * i, w);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[c >> 1][c & 1][s] = __uint_as_float(w[c]);
+          }
+          tc::tmem_wait_ld();
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            if (b + k >= 3 * N) break;
+            const Split ur = fx::split(fx::from_sums(acc[k][0])), us = fx::split(fx::from_sums(acc[k][1]));
+            if (live) {
+              const int2* c = a.tab + el;
+              const long long q = fx::mul(ur, coef(c + (3 + 2 * f) * a.K)) + fx::mul(us, coef(c + (4 + 2 * f) * a.K));
+              a.Iq[int64_t(f * (N + 1) + j) * a.ldc + row] = q;
+              qbits |= int(q >> 32) ^ int(q >> 63);
+              if (j == 0) {
+                const int g = f == 0 ? 2 : f - 1;
+                const long long p2 = fx::mul(ur, coef(c + (3 + 2 * g) * a.K)) + fx::mul(us, coef(c + (4 + 2 * g) * a.K));
+                a.Iq[int64_t(g * (N + 1) + N) * a.ldc + row] = p2;
+                qbits |= int(p2 >> 32) ^ int(p2 >> 63);
+              }
+            }
+            if (++j == N) ++f, j = 0;
+          }
+        }
+        tc::fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(acce);
+      }
+      pm[2 * kT] = qbits;
+    }
+    bar_sync(1, 256);
+    if (it > 0) write_exponents((blockIdx.x + int64_t(it - 1) * gridDim.x) * kT + e);
   }
-  if (*abort_flag && tid == 0) atomicExch(&g_tc64_err, 1);
+  if (*abort_flag && tid == 0) atomicExch(&g_t64_err, 1);
+  tc::fence_before();
+  __syncthreads();
+  tc::fence_after();
+  if (warp == 0) tc::tmem_dealloc(tb, 256);
+}
+
+// ------------------------------------------------------------------ output product
+constexpr int kOutStages = 2;  // operator blocks in flight (three measured the same)
+struct OutArgs {
+  int N, chunks, M;         // chunks of two item groups, output columns of this launch
+  int gvol, gface;          // groups of eight items: [0, gvol) volume, [gvol, gface) face, then mass
+  int cpen, lpen;           // (N+1)(N+2)/2 <= 2^lpen
+  int k1, k2, km;           // data columns carry 2^-k (k1: flux, k2: jumps, km: mass), operator columns 2^k
+  int helm;
+  double lambda;
+  int64_t K, rows, row0;
+  const long long* Iu;      // all rows
+  const long long* Iq;
+  int64_t ldc;
+  const int4* ex;
+  const double* u0;
+  const int2* tab;
+  const short4* tex;
+  const double* gx;
+  const int32_t* conn;
+  const uint8_t* ops;       // [chunk][3 kinds of columns][7 digits x NC rows][16]
+  const int* ea;            // [NC]
+  double* out;              // this launch's first row, first column
+  int64_t ldo;
+};
+
+constexpr int kWorkers = 512;
+constexpr int kOutThreads = kWorkers + 128;
+constexpr int kLut = 3 * (kMaxN + 1);          // local nodes of the face nodes
+constexpr int kScaleWords = 2 * kCoefs + 6 + 7;  // a row's scale: coefficients, differences of u0, E, neighbours, shifts
+constexpr int kBadScale = 1 << 20;             // E of a row with an infinity or a NaN among its data
+__host__ __device__ constexpr int out_sets(int nc) { return nc <= 48 ? 2 : 1; }
+__host__ __device__ constexpr int out_smem(int nc) {
+  return 2 * kChunkBytes + kOutStages * kDigits * nc * 32 + out_sets(nc) * kScaleWords * kT * 4 + 24 * 8 + 16 + kLut * 8;
+}
+
+// NC: output columns (a multiple of 16). Sixteen warps in two groups of eight:
+// group p forms the chunks of buffer p (two threads per row, eight items each)
+// while the products of the other buffer run; all sixteen drain a tile's
+// accumulators after the first chunk of the next one, so neither the products
+// nor the copies wait for the drain. Warp 16 issues the products, warp 17 the
+// operator's copies (a ring of 16-column blocks); warps 18 and 19 run a tile
+// ahead and work out each row's scale: a bound on its columns from its own and
+// its neighbours' exponents, the coefficients at that scale and the shifts that
+// bring both sides of a face to a common one (done by every thread that forms
+// columns, this took a third of the kernel's instructions).
+template <int NC>
+__global__ void __launch_bounds__(kOutThreads, 1) t64_output(const OutArgs a) {
+  extern __shared__ __align__(1024) uint8_t sm[];
+  constexpr int kStages = kOutStages;
+  constexpr int kSets = out_sets(NC);
+  constexpr int kStage = kDigits * NC * 32;
+  constexpr int kAcc = 2 * kSums * NC <= 512 ? 2 : 1;  // accumulator sets
+  uint8_t* sB = sm + 2 * kChunkBytes;
+  int2* scoef = reinterpret_cast<int2*>(sB + kStages * kStage);        // [sets][kCoefs][kT], at the row's scale
+  long long* sdiff = reinterpret_cast<long long*>(scoef + kSets * kCoefs * kT);  // [sets][3][kT]: u0+ - u0- at the jump's scale
+  int* sinfo = reinterpret_cast<int*>(sdiff + kSets * 3 * kT);         // [sets][E | 3 neighbours | 3 shifts][kT]
+  long long* lut = reinterpret_cast<long long*>(sinfo + kSets * 7 * kT);   // [3][N + 1]: offset of face f's j-th node in Iu
+  uint64_t* bars = reinterpret_cast<uint64_t*>(lut + kLut);
+  uint64_t *full = bars, *empty = bars + 2, *accf = bars + 4, *acce = bars + 6, *sfull = bars + 8, *sempty = bars + 10,
+           *bfull = bars + 12, *bempty = bars + 12 + kStages;
+  uint32_t* slot = reinterpret_cast<uint32_t*>(bars + 24);
+  volatile int* abort_flag = reinterpret_cast<int*>(slot + 1);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int64_t ntiles = (a.rows + kT - 1) / kT;
+  if (tid < 3 * (a.N + 1)) lut[tid] = node_of(a.N, tid / (a.N + 1), tid % (a.N + 1)) * a.ldc;
+  if (tid == 0) {
+    for (int i = 0; i < 2; ++i) {
+      tc::mbar_init(full + i, 8);
+      tc::mbar_init(empty + i, 1);
+      tc::mbar_init(accf + i, 1);
+      tc::mbar_init(acce + i, 16);
+      tc::mbar_init(sfull + i, 2);
+      tc::mbar_init(sempty + i, 16);
+    }
+    for (int i = 0; i < kStages; ++i) {
+      tc::mbar_init(bfull + i, 1);
+      tc::mbar_init(bempty + i, 1);
+    }
+    *abort_flag = 0;
+    tc::mbar_init_fence();
+  }
+  if (warp == 0) tc::tmem_alloc(slot, 512);
+  tc::fence_before();
+  __syncthreads();
+  tc::fence_after();
+  const uint32_t tb = *slot;
+
+  if (warp == 17) {
+    // ================= operator blocks
+    uint32_t n = 0;
+    const int steps = 3 * a.chunks;
+    for (int64_t tile = blockIdx.x; tile < ntiles && !aborted(abort_flag); tile += gridDim.x)
+      for (int s = 0; s < steps; ++s, ++n) {
+        const uint32_t b = n % kStages, use = n / kStages;
+        if (use > 0) wait(bempty + b, (use - 1) & 1u, abort_flag);
+        if (aborted(abort_flag)) break;
+        if (lane == 0) {
+          tc::mbar_expect_tx(bfull + b, kStage);
+          tc::bulk_g2s(sB + b * kStage, a.ops + size_t(s) * kStage, kStage, bfull + b);
+        }
+        __syncwarp();
+      }
+    // every copy has landed before the block ends
+    for (uint32_t k = n < kStages ? 0 : n - kStages; k < n; ++k)
+      wait(bfull + k % kStages, (k / kStages) & 1u, abort_flag);
+  } else if (warp == 16) {
+    // ================= products
+    const uint64_t ad = tc::smem_desc(tc::smem_addr(sm), 128, 6 * 128);
+    const uint64_t bd = tc::smem_desc(tc::smem_addr(sB), 128, 256);
+    uint32_t n = 0, g = 0, it = 0;
+    for (int64_t tile = blockIdx.x; tile < ntiles && !aborted(abort_flag); tile += gridDim.x, ++it) {
+      const uint32_t ab = it % kAcc, use = it / kAcc;
+      if (use > 0) wait(acce + ab, (use - 1) & 1u, abort_flag);
+      for (int kc = 0; kc < a.chunks; ++kc, ++g) {
+        wait(full + (g & 1u), (g >> 1) & 1u, abort_flag);
+        for (int c = 0; c < 3; ++c, ++n) {
+          const uint32_t b = n % kStages;
+          wait(bfull + b, (n / kStages) & 1u, abort_flag);
+          tc::fence_after();
+          if (lane == 0) {
+            issue_step(tb + ab * kSums * NC, ad + (((g & 1u) * kChunkBytes + c * 256) >> 4), kChunkSlice,
+                       bd + ((b * kStage) >> 4), NC, kc == 0 && c == 0);
+            tc::mma_commit(bempty + b);
+            if (c == 2) tc::mma_commit(empty + (g & 1u));
+            if (c == 2 && kc + 1 == a.chunks) tc::mma_commit(accf + ab);
+          }
+          __syncwarp();
+        }
+      }
+    }
+  } else if (warp >= 18) {
+    // ================= scales
+    uint32_t it = 0;
+    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
+      const uint32_t set = it % kSets;
+      if (it >= kSets) wait(sempty + set, (it / kSets - 1) & 1u, abort_flag);
+#pragma unroll 1
+      for (int k = 0; k < 2; ++k) {
+        const int e = (warp - 18) * 32 + lane + 64 * k;
+        const int64_t row = tile * kT + e, be = a.row0 + (row < a.rows ? row : 0), el = elem_of(be, a.K);
+        const int boff = int(be - el);
+        int code[3];
+#pragma unroll
+        for (int f = 0; f < 3; ++f) code[f] = __ldg(a.conn + 3 * el + f);
+        const int4 x = __ldg(a.ex + be);
+        const short4 t = __ldg(a.tex + el);
+        const double u0 = __ldg(a.u0 + be);
+        long long c[kCoefs];
+#pragma unroll
+        for (int i = 0; i < kCoefs; ++i) c[i] = fx::join(coef(a.tab + el + int64_t(i) * a.K));
+        int4 y[3];
+        double d[3];  // the jump without its v parts
+#pragma unroll
+        for (int f = 0; f < 3; ++f) {
+          const int64_t nb = boff + (code[f] >> 2);
+          y[f] = code[f] >= 0 ? __ldg(a.ex + nb) : x;
+          d[f] = code[f] >= 0 ? __ldg(a.u0 + nb) - u0 : (code[f] == -2 ? -2.0 * u0 : 0.0);
+        }
+        const int et = t.z + a.lpen;
+        int E = x.x + t.x;
+        bool bad = x.w >= fx::kBadExp;
+        int ej[3];  // each of the jump's three parts is below 2^ej
+#pragma unroll
+        for (int f = 0; f < 3; ++f) {
+          ej[f] = max(max(x.x, y[f].x), fx::exp_bound(d[f]));
+          bad = bad || y[f].w >= fx::kBadExp;
+          E = max(E, max(max(ej[f] + t.y + 1 - a.k2, ej[f] + et + 3 - a.k1), max(x.z, y[f].z) + 1 - a.k1));
+          E = max(E, max(x.y, y[f].y) - 2 - a.k1);  // q is only shifted down
+        }
+        if (a.helm) E = max(E, x.w + fx::exp_bound(a.lambda * __ldg(a.gx + 16 * el)) - a.km);
+        int2* sc = scoef + set * kCoefs * kT + e;
+        int* si = sinfo + set * 7 * kT + e;
+        // columns at scale 2^{56-E}, from v 2^{59-ev} and a coefficient c 2^{62-e}
+        auto put = [&](int i, long long v, int sh) {
+          const Split q = fx::split(fx::sar(v, sh));
+          sc[i * kT] = make_int2(q.h, q.l);
+        };
+#pragma unroll
+        for (int i = 0; i < 3; ++i) put(i, c[i], E - x.x - t.x + 1);
+        si[0] = bad ? kBadScale : E;
+        const int sq = E + 2 + a.k1;  // half of q 2^{57-eq} at 2^{56-E}
+#pragma unroll
+        for (int f = 0; f < 3; ++f) {
+          const int sj = E - ej[f] - t.y + 2 + a.k2;  // half the jump
+          put(3 + 2 * f, c[3 + 2 * f], sj);
+          put(4 + 2 * f, c[4 + 2 * f], sj);
+          put(9 + f, (c[9 + f] >> a.lpen) * a.cpen, E - ej[f] - et + 1 + a.k1);
+          sdiff[(set * 3 + f) * kT + e] = fx::fix<59>(d[f], ej[f]);
+          si[(1 + f) * kT] = code[f] >= 0 ? boff + (code[f] >> 2) : code[f];
+          si[(4 + f) * kT] = (code[f] & 3) | (min(ej[f] - x.x, 63) << 2) | (min(ej[f] - y[f].x, 63) << 8) |
+                             (min(sq - x.y, 63) << 14) | (min(sq - y[f].y, 63) << 20);
+        }
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(sfull + set);
+    }
+  } else {
+    // ================= columns and drain
+    const int grp = warp >> 3, half = (warp >> 2) & 1, e = (warp & 3) * 32 + lane;
+    const uint32_t lanebase = uint32_t((warp & 3) * 32) << 16;
+    const int N = a.N, Np = (N + 1) * (N + 2) / 2, Nfp = N + 1, nface = 3 * Nfp;
+    uint32_t it = 0, g0 = 0;
+    int Eprev = 0;
+
+    auto drain = [&](uint32_t t, int64_t row, int E) {
+      const uint32_t ab = t % kAcc;
+      wait(accf + ab, (t / kAcc) & 1u, abort_flag);
+      tc::fence_after();
+      const int c0 = (warp >> 2) * (NC / 4);
+#pragma unroll 1
+      for (int p = 0; p < NC / 16; ++p) {
+        const int col = c0 + 4 * p;
+        if (col < a.M) {
+          float acc[4][kSums];
+          __syncwarp();
+#pragma unroll
+          for (int s = 0; s < kSums; ++s) {
+            uint32_t w[4];
+            tc::tmem_ld4(tb + lanebase + (ab * kSums + s) * NC + col, w);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[c][s] = __uint_as_float(w[c]);
+          }
+          tc::tmem_wait_ld();
+          if (row < a.rows) {
+            double* o = a.out + row * a.ldo + col;
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+              if (col + c < a.M) {
+                const double v = fx::to_double(fx::from_sums(acc[c]), __ldg(a.ea + col + c) + E - 56);
+                o[c] = E == kBadScale ? fx::double_of(0x7ff8000000000000ll) : v;
+              }
+          }
+        }
+      }
+      tc::fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(acce + ab);
+    };
+
+    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it, g0 += a.chunks) {
+      const int64_t row = tile * kT + e, be = a.row0 + (row < a.rows ? row : 0);
+      const long long *uo = a.Iu + be, *qo = a.Iq + be;
+      const uint32_t set = it % kSets;
+      const int2* sc = scoef + set * kCoefs * kT + e;
+      const long long* sd = sdiff + set * 3 * kT + e;
+      const int* si = sinfo + set * 7 * kT + e;
+      wait(sfull + set, (it / kSets) & 1u, abort_flag);
+      const int E = si[0];
+      bool drained = it == 0;
+      for (int kc = 0; kc < a.chunks; ++kc) {
+        const uint32_t g = g0 + kc;
+        if ((g & 1u) != uint32_t(grp)) continue;
+        if (g >= 2) wait(empty + grp, ((g >> 1) - 1) & 1u, abort_flag);
+        const int gr = 2 * kc + half;  // this warp's group of eight items
+        uint8_t* dst = sm + grp * kChunkBytes + (e >> 3) * 768 + half * 128 + (e & 7) * 16;
+        auto cf = [&](int k) {
+          const int2 q = sc[k * kT];
+          return Split{q.x, q.y};
+        };
+        if (gr < a.gvol) {  // Grr u, Grs u, Gss u at eight nodes
+          long long v[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) v[i] = 8 * gr + i < Np ? __ldg(uo + (8 * gr + i) * a.ldc) : 0;
+#pragma unroll 1
+          for (int c = 0; c < 3; ++c) {
+            const Split k = cf(c);
+            long long x[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) x[i] = fx::mul(fx::split(v[i]), k);
+            fx::digits8(x, dst + c * 256, kChunkSlice);
+          }
+        } else if (gr < a.gface) {
+#pragma unroll 1
+          for (int hb = 0; hb < 2; ++hb) {  // four face nodes at a time: their sixteen loads are in flight together
+            const int i0 = 8 * (gr - a.gvol) + 4 * hb;
+            long long v[4], w[4], y[4], z[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const int t = i0 + i, f = t >= 2 * Nfp ? 2 : (t >= Nfp ? 1 : 0);
+              v[i] = w[i] = y[i] = z[i] = 0;
+              if (t < nface) {
+                const int nb = si[(1 + f) * kT], fn = si[(4 + f) * kT] & 3;
+                v[i] = __ldg(uo + lut[t]);
+                y[i] = __ldg(qo + t * a.ldc);
+                if (nb >= 0) {
+                  const int tn = fn * Nfp + N - (t - f * Nfp);
+                  w[i] = __ldg(a.Iu + nb + lut[tn]);
+                  z[i] = __ldg(a.Iq + nb + tn * a.ldc);
+                }
+              }
+            }
+            long long x[3][4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const int t = i0 + i, f = t >= 2 * Nfp ? 2 : (t >= Nfp ? 1 : 0);
+              const int nb = si[(1 + f) * kT], info = si[(4 + f) * kT];
+              const long long um = v[i] >> ((info >> 2) & 63), qm = y[i] >> ((info >> 14) & 63);
+              long long up = w[i] >> ((info >> 8) & 63), qp = z[i] >> ((info >> 20) & 63);
+              if (nb < 0) {  // Dirichlet: u+ = -u-, grad u+ = grad u-; Neumann: no terms
+                up = nb == -2 ? -um : um;
+                qp = nb == -2 ? ~qm : qm;  // ~: the shifts' roundings cancel, as two neighbours' do
+              }
+              const Split s = fx::split(up - um + sd[f * kT]);
+              x[0][i] = fx::mul(s, cf(3 + 2 * f));
+              x[1][i] = fx::mul(s, cf(4 + 2 * f));
+              x[2][i] = qp - qm + fx::mul(s, cf(9 + f));
+            }
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+              fx::digits4(x[c], dst + c * 256 + hb * 8, kChunkSlice);
+          }
+        } else {  // lambda J u, three nodes an item (zero past the last group)
+          const int n0 = 24 * (gr - a.gface);
+          Split k{0, 0};
+          long long k0 = 0;  // lambda J u0
+          if (a.helm) {
+            const double lj = a.lambda * __ldg(a.gx + 16 * elem_of(be, a.K)), l0 = lj * __ldg(a.u0 + be);
+            const int elj = fx::exp_bound(lj), e0 = fx::exp_bound(l0);
+            k = fx::split(fx::sar(fx::fix<62>(lj, elj), E - __ldg(a.ex + be).x - elj + 1 + a.km));
+            k0 = fx::sar(fx::fix<59>(l0, e0), E - e0 + 3 + a.km);
+          }
+#pragma unroll 1
+          for (int c = 0; c < 3; ++c) {
+            long long x[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const int n = n0 + 3 * i + c;
+              x[i] = a.helm && n < Np ? fx::mul(fx::split(__ldg(uo + n * a.ldc)), k) + k0 : 0;
+            }
+            fx::digits8(x, dst + c * 256, kChunkSlice);
+          }
+        }
+        tc::fence_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(full + grp);
+        if (!drained) {
+          drain(it - 1, row - int64_t(gridDim.x) * kT, Eprev);
+          drained = true;
+        }
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(sempty + set);  // the tile's columns are formed
+      if (!drained) drain(it - 1, row - int64_t(gridDim.x) * kT, Eprev);
+      Eprev = E;
+    }
+    if (it > 0) drain(it - 1, (blockIdx.x + int64_t(it - 1) * gridDim.x) * kT + e, Eprev);
+  }
+  if (*abort_flag && tid == 0) atomicExch(&g_t64_err, 1);
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
   if (warp == 0) tc::tmem_dealloc(tb, 512);
 }
 
-// ------------------------------------------------------------------ face columns of Y
-// One thread per element (consecutive threads take consecutive rows, so every
-// access to the column-major face data and Y is coalesced except the
-// neighbour's): for each face f and face node j, entry i = f (N+1) + j, from
-// the element's face data and its neighbour's across face f (FNu, FNd, written
-// by the gradient product), Y[2Np + i] = 1/2 nr sJ [u], Y[2Np + NFN + i] =
-// 1/2 ns sJ [u], Y[2Np + 2 NFN + i] = -sJ ({n.grad u} + tau [u]), in
-// float-float scaled by the entry's largest input; the row's largest exponent
-// (exy: raised from the value the gradient product wrote for the volume
-// columns) for the output product's slicing.
-__global__ void __launch_bounds__(256) tc64_face_fill(int N, int64_t K, int64_t r0, int64_t nE,
-                                                      const double* __restrict__ gx,
-                                                      const int32_t* __restrict__ conn,
-                                                      const double* __restrict__ FNu,
-                                                      const double* __restrict__ FNd, double* __restrict__ Y,
-                                                      int64_t ldc, int* __restrict__ exy) {
-  const int Np = (N + 1) * (N + 2) / 2, Nfp = N + 1, NFN = 3 * Nfp;
-  const ff cpen{float((N + 1) * (N + 2)) * 0.5f, 0.f};
-  for (int64_t be = r0 + int64_t(blockIdx.x) * blockDim.x + threadIdx.x; be < nE;
-       be += int64_t(gridDim.x) * blockDim.x) {  // rows r0 .. nE - 1
-    const int64_t el = be < K ? be : be % K, boff = be - el;  // first right-hand side: no division
-    int ym = -1100;
-    for (int f = 0; f < 3; ++f) {
-      const double* g = gx + 16 * el + 4 + 4 * f;
-      const ff nr = d2ff(__ldg(g), 0), ns = d2ff(__ldg(g + 1), 0), sJ = d2ff(__ldg(g + 2), 0);
-      const ff tau = ff_mul(cpen, d2ff(__ldg(g + 3), 0));
-      const int code = __ldg(conn + 3 * el + f);
-      const int64_t nb = code >= 0 ? boff + (code >> 2) : 0;
-      const int fn = code >= 0 ? (code & 3) : 0;
-      for (int j = 0; j < Nfp; ++j) {
-        const int i = f * Nfp + j;
-        const double ou = __ldg(FNu + int64_t(i) * ldc + be), od = __ldg(FNd + int64_t(i) * ldc + be);
-        double pu = 0.0, pd = 0.0;
-        if (code >= 0) {
-          const int64_t pi = int64_t(fn * Nfp + (Nfp - 1 - j)) * ldc + nb;
-          pu = __ldg(FNu + pi);
-          pd = __ldg(FNd + pi);
-        }
-        const int R = max(max(exp_bound64(ou), exp_bound64(od)), max(exp_bound64(pu), exp_bound64(pd)));
-        const int Rs = R == -1100 ? 0 : R;
-        const ff um = d2ff(ou, Rs), dnm = d2ff(od, Rs);
-        ff jm{0.f, 0.f}, av{0.f, 0.f};
-        if (code >= 0) {
-          jm = ff_sub(d2ff(pu, Rs), um);
-          av = ff_pow2(ff_sub(dnm, d2ff(pd, Rs)), 0.5f);
-        } else if (code == -2) {  // Dirichlet
-          jm = ff_pow2(um, -2.0f);
-          av = dnm;
-        }
-        const ff hs = ff_pow2(ff_mul(sJ, jm), 0.5f);
-        const ff a = ff_mul(nr, hs), b = ff_mul(ns, hs);
-        const ff fl = ff_neg(ff_mul(sJ, ff_add(av, ff_mul(tau, jm))));
-        double* y = Y + int64_t(2 * Np + i) * ldc + be;
-        const double da = ff_to_double(a.h, a.l, Rs), db = ff_to_double(b.h, b.l, Rs), dc = ff_to_double(fl.h, fl.l, Rs);
-        y[0] = da;
-        y[int64_t(NFN) * ldc] = db;
-        y[int64_t(2 * NFN) * ldc] = dc;
-        ym = max(ym, max(exp_bound64(da), max(exp_bound64(db), exp_bound64(dc))));
-      }
-    }
-    if (ym > -1100) exy[be] = max(exy[be], ym);  // with the volume columns' bound, set before
-  }
-}
-
 // ------------------------------------------------------------------ host side
-int row_exp(const double* row, int K) {
-  double mx = 0.0;
-  for (int k = 0; k < K; ++k) mx = std::max(mx, std::fabs(row[k]));
-  if (mx == 0.0) return 0;
+// An operator block image: rows scaled to integers below 2^56 (one exponent
+// per row, or one for all), cut into digits (fix64.cuh), digit i of row r at
+// stacked row i nc + r, in 16-column steps of the canonical layout.
+int ceil_log2(double x) {  // e with x < 2^e (0 for zero)
   int e = 0;
-  std::frexp(mx, &e);  // mx < 2^e
+  std::frexp(x, &e);
   return e;
 }
+// A row's exponent: its entries below 2^e, and its absolute sum below 2^{e+6}, so
+// that a product's digit sums stay below 2^62 where fx::from_sums joins them.
+int row_exp(double mx, double l1) { return std::max(ceil_log2(mx), ceil_log2(l1) - 6); }
 
-uint16_t bf16_int(int x) {  // exact for |x| <= 256
-  const float f = float(x);
-  uint32_t b;
-  std::memcpy(&b, &f, 4);
-  return uint16_t(b >> 16);
+uint16_t fp16_int(int d) {  // exact for |d| <= 2048
+  if (d == 0) return 0;
+  const int m = std::abs(d);
+  int e = 0;
+  while ((m >> e) > 1) ++e;
+  return uint16_t((d < 0 ? 0x8000 : 0) | ((e + 15) << 10) | (((m << 10) >> e) & 0x3ff));
 }
 
-}  // namespace
-
-// A (M x K, row-major FP64) into the block layout of tc64_gemm.
-cudaError_t tc64_op_create(const std::vector<double>& A, int M, int K, Tc64Op* op) {
-  op->M = M;
-  op->K = K;
-  op->NCH = (M + kNC - 1) / kNC;
-  op->KCH = (K + kKC - 1) / kKC;
-  if (K > kMaxDepth) return cudaErrorInvalidValue;  // longer sums would leave the FP32 group sums inexact
-  std::vector<uint8_t> img(size_t(op->NCH) * op->KCH * kBBytes, 0);
-  std::vector<int> ea(size_t(op->NCH) * kNC, 0);
-  for (int r = 0; r < M; ++r) {
-    const int er = row_exp(&A[size_t(r) * K], K);
-    ea[r] = er;
+// A(r, k) for r < M <= nc, k < K (columns past K are zero; K a multiple of 16 on
+// the way out), ea[r] the row exponents to use.
+template <typename F>
+void slice_block(const F& A, int M, int nc, int K, const int* ea, std::vector<uint8_t>& img) {
+  const int steps = (K + 15) / 16;
+  const size_t step_bytes = size_t(kDigits) * nc * 32;
+  const size_t base = img.size();
+  img.resize(base + steps * step_bytes, 0);
+  for (int r = 0; r < M; ++r)
     for (int k = 0; k < K; ++k) {
-      const double v = A[size_t(r) * K + k];
-      if (v == 0.0 || !std::isfinite(v)) continue;
-      int e2 = 0;
-      const double fr = std::frexp(std::fabs(v), &e2);
-      const int sh = e2 + 56 - er;
-      if (sh <= 0) continue;
-      const unsigned long long I = (unsigned long long)std::ldexp(fr, sh);
-      const int sgn = v < 0 ? -1 : 1;
-      const int nc = r / kNC, rl = r % kNC, kc = k / kKC, kl = k % kKC;
-      uint8_t* blk = img.data() + size_t(nc * op->KCH + kc) * kBBytes;
-      const size_t off = size_t(rl / 8) * ((kKC / 8) * 128) + size_t(kl / 8) * 128 + size_t(rl % 8) * 16 + size_t(kl % 8) * 2;
-      for (int i = 0; i < kSl; ++i) {
-        const int x = sgn * int((I >> (49 - 7 * i)) & 127ull);
-        const uint16_t b = bf16_int(x);
-        std::memcpy(blk + size_t(i) * kBSlice + off, &b, 2);
+      const double v = A(r, k);
+      if (v == 0.0) continue;
+      long long x = std::llround(std::ldexp(v, 56 - ea[r]));
+      uint8_t* blk = img.data() + base + size_t(k / 16) * step_bytes;
+      for (int i = kDigits - 1; i >= 0; --i) {  // last digit first
+        const int d = i == 0 ? int(x) : int((x + 128) & 255) - 128;
+        x = (x - d) >> 8;
+        const int R = i * nc + r, c = k % 16;
+        const uint16_t h = fp16_int(d);
+        std::memcpy(blk + size_t(R / 8) * 256 + (c / 8) * 128 + (R % 8) * 16 + (c % 8) * 2, &h, 2);
       }
     }
-  }
-  cudaError_t e = cudaMalloc(&op->blocks, img.size());
-  if (e == cudaSuccess) e = cudaMemcpy(op->blocks, img.data(), img.size(), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMalloc(&op->ea, ea.size() * sizeof(int));
-  if (e == cudaSuccess) e = cudaMemcpy(op->ea, ea.data(), ea.size() * sizeof(int), cudaMemcpyHostToDevice);
-  return e;
 }
 
-void tc64_op_free(Tc64Op* op) {
-  cudaFree(op->blocks);
-  cudaFree(op->ea);
-  op->blocks = nullptr;
-  op->ea = nullptr;
-}
-
-namespace {
-template <int MODE>
-cudaError_t gemm_launch(const Tc64Op& op, int64_t rows, const double* X, int64_t ldx, double* out, int64_t ldo,
-                        const int* ex_given, const GradOut& go, cudaStream_t st, int accum = 0, int xcol = 0) {
-  if (rows <= 0) return cudaSuccess;
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  static int grid[64];
-  {
-    std::lock_guard<std::mutex> lk(table_mutex());
-    if (!grid[dev & 63]) {
-      e = cudaFuncSetAttribute(tc64_gemm<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
-      if (e == cudaSuccess) e = cudaFuncSetAttribute(tc64_gemm<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
-      int sms = 0;
-      if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-      if (e != cudaSuccess) return e;
-      grid[dev & 63] = sms;  // one CTA per SM (all of tensor memory, most of shared memory)
-    }
-  }
-  const int vec2 = (ldx % 2 == 0 && (reinterpret_cast<uintptr_t>(X) & 15u) == 0) ? 1 : 0;
-  const int64_t tiles = (rows + kT - 1) / kT;
-  const unsigned g = unsigned(std::min<int64_t>(tiles, grid[dev & 63]));
-  tc64_gemm<MODE><<<g, kSlicers + 32, kSmem, st>>>(rows, op.M, op.K, op.NCH, op.KCH, X, ldx, vec2, xcol, ex_given,
-                                                   op.blocks, op.ea, out, ldo, accum, go);
-  note_launch();
-  return cudaGetLastError();
-}
-}  // namespace
-
-cudaError_t tc64_gemm_launch(const Tc64Op& op, int64_t rows, const double* X, int64_t ldx, double* out, int64_t ldo,
-                             cudaStream_t st, int accum, const int* ex) {
-  return gemm_launch<0>(op, rows, X, ldx, out, ldo, ex, GradOut{}, st, accum);
-}
-
-namespace {
+struct OutOp {
+  int M = 0, c0 = 0;  // output columns [c0, c0 + M)
+  uint8_t* ops = nullptr;
+  int* ea = nullptr;
+};
+struct OutSet {  // one form of the operator: Poisson, or with the Helmholtz columns
+  int gvol = 0, gface = 0, chunks = 0, nc = 0, parts = 0;
+  OutOp part[2];
+};
 struct Tc64Apply {
-  Tc64Op grad;       // [Dr; Ds] with rows interleaved (Dr row n, Ds row n, ...)
-  Tc64Op out, outh;  // OB, [OB | M] (when its depth stays within kMaxDepth)
-  Tc64Op mh;         // M alone, otherwise: the Helmholtz term as a second, accumulating product
-  Tc64Op outv, outf; // [Br Bs] and the face blocks of OB, when OB is deeper than kSplitDepth
+  bool ready = false;
+  int trace_ea = 0, passes = 0, ks = 0, k1 = 0, k2 = 0, km = 0;
+  uint8_t* trace = nullptr;
+  OutSet out[2];  // [helmholtz]
 };
 Tc64Apply g_t64[64][kMaxN + 1];  // [device][degree]
 
+cudaError_t upload(const void* p, size_t n, void** d) {
+  cudaError_t e = cudaMalloc(d, n);
+  if (e == cudaSuccess) e = cudaMemcpy(*d, p, n, cudaMemcpyHostToDevice);
+  return e;
+}
+int floor_log2(double x) {
+  int e = 0;
+  std::frexp(x, &e);
+  return e - 1;
+}
+
 cudaError_t build_t64(const RefElem& R, Tc64Apply& o) {
-  const int N = R.N, Np = R.Np, Nfp = R.Nfp, NFN = 3 * Nfp;
-  std::vector<double> A1(size_t(2 * Np) * Np);
-  for (int n = 0; n < Np; ++n)
-    for (int m = 0; m < Np; ++m) {
-      A1[size_t(2 * n) * Np + m] = R.Dr[size_t(n) * Np + m];
-      A1[size_t(2 * n + 1) * Np + m] = R.Ds[size_t(n) * Np + m];
+  const int N = R.N, Np = R.Np, Nfp = R.Nfp, nface = 3 * Nfp;
+  // boundary derivatives: rows 2b, 2b + 1 = d/dr, d/ds at the b-th node counter-clockwise
+  auto trace = [&](int r, int k) {
+    const int b = r / 2, n = face_node(N, b / N, b % N);
+    return (r & 1) ? R.Ds[size_t(n) * Np + k] : R.Dr[size_t(n) * Np + k];
+  };
+  double mx = 0.0, l1 = 0.0;
+  for (int r = 0; r < 6 * N; ++r) {
+    double s = 0.0;
+    for (int k = 0; k < Np; ++k) {
+      mx = std::max(mx, std::fabs(trace(r, k)));
+      s += std::fabs(trace(r, k));
     }
-  const int KY = 2 * Np + 3 * NFN, KH = KY + Np;
-  std::vector<double> B(size_t(Np) * KY, 0.0), BH(size_t(Np) * KH, 0.0);
+    l1 = std::max(l1, s);
+  }
+  o.trace_ea = row_exp(mx, l1);
+  o.passes = (6 * N + kTraceN - 1) / kTraceN;
+  o.ks = (Np + 15) / 16;
+  std::vector<uint8_t> img;
+  const std::vector<int> eat(kTraceN, o.trace_ea);
+  for (int p = 0; p < o.passes; ++p)
+    slice_block([&](int r, int k) { return k < Np ? trace(p * kTraceN + r, k) : 0.0; },
+                std::min(kTraceN, 6 * N - p * kTraceN), kTraceN, 16 * o.ks, eat.data(), img);
+  cudaError_t e = upload(img.data(), img.size(), reinterpret_cast<void**>(&o.trace));
+  // the output operator, its three volume blocks in extended precision
+  std::vector<double> S[3], Df[2], Ef(size_t(Np) * nface, 0.0);
+  for (auto& s : S) s.assign(size_t(Np) * Np, 0.0);
+  for (auto& d : Df) d.assign(size_t(Np) * nface, 0.0);
+  double ms = 0.0, md = 0.0, me = 0.0, mm = 0.0;
   for (int i = 0; i < Np; ++i) {
-    for (int m = 0; m < Np; ++m) {
-      B[size_t(i) * KY + m] = R.Br[size_t(i) * Np + m];
-      B[size_t(i) * KY + Np + m] = R.Bs[size_t(i) * Np + m];
+    for (int n = 0; n < Np; ++n) {
+      long double rr = 0, rs = 0, ss = 0;
+      for (int k = 0; k < Np; ++k) {
+        const long double br = R.Br[size_t(i) * Np + k], bs = R.Bs[size_t(i) * Np + k];
+        const long double dr = R.Dr[size_t(k) * Np + n], ds = R.Ds[size_t(k) * Np + n];
+        rr += br * dr;
+        rs += br * ds + bs * dr;
+        ss += bs * ds;
+      }
+      S[0][size_t(i) * Np + n] = double(rr);
+      S[1][size_t(i) * Np + n] = double(rs);
+      S[2][size_t(i) * Np + n] = double(ss);
+      for (const auto& s : S) ms = std::max(ms, std::fabs(s[size_t(i) * Np + n]));
+      mm = std::max(mm, std::fabs(R.M[size_t(i) * Np + n]));
     }
     for (int f = 0; f < 3; ++f)
       for (int l = 0; l < Nfp; ++l) {
@@ -768,44 +846,60 @@ cudaError_t build_t64(const RefElem& R, Tc64Apply& o) {
           ds += R.Ds[size_t(k) * Np + i] * mf;
           if (k == i) ef += mf;
         }
-        B[size_t(i) * KY + 2 * Np + f * Nfp + l] = dr;
-        B[size_t(i) * KY + 2 * Np + NFN + f * Nfp + l] = ds;
-        B[size_t(i) * KY + 2 * Np + 2 * NFN + f * Nfp + l] = ef;
+        Df[0][size_t(i) * nface + f * Nfp + l] = dr;
+        Df[1][size_t(i) * nface + f * Nfp + l] = ds;
+        Ef[size_t(i) * nface + f * Nfp + l] = ef;
+        md = std::max(md, std::max(std::fabs(dr), std::fabs(ds)));
+        me = std::max(me, std::fabs(ef));
       }
-    for (int k = 0; k < KY; ++k) BH[size_t(i) * KH + k] = B[size_t(i) * KY + k];
-    for (int m = 0; m < Np; ++m) BH[size_t(i) * KH + KY + m] = R.M[size_t(i) * Np + m];
   }
-  cudaError_t e = tc64_op_create(A1, 2 * Np, Np, &o.grad);
-  if (KY > kSplitDepth) {  // column blocks [Br Bs], [face blocks], M, each from its own Y columns
-    std::vector<double> Bv(size_t(Np) * 2 * Np), Bf(size_t(Np) * 3 * NFN), Mm(R.M.begin(), R.M.begin() + size_t(Np) * Np);
-    for (int i = 0; i < Np; ++i) {
-      for (int k = 0; k < 2 * Np; ++k) Bv[size_t(i) * 2 * Np + k] = B[size_t(i) * KY + k];
-      for (int k = 0; k < 3 * NFN; ++k) Bf[size_t(i) * 3 * NFN + k] = B[size_t(i) * KY + 2 * Np + k];
+  // powers of two that bring every block's largest entry to the volume block's
+  o.k1 = floor_log2(ms / me);
+  o.k2 = floor_log2(ms / md);
+  o.km = floor_log2(ms / mm);
+  for (int helm = 0; helm < 2; ++helm) {
+    OutSet& w = o.out[helm];
+    w.gvol = (Np + 7) / 8;
+    w.gface = w.gvol + (nface + 7) / 8;
+    w.chunks = (w.gface + (helm ? (Np + 23) / 24 : 0) + 1) / 2;
+    w.parts = Np > 64 ? 2 : 1;
+    const int M = (Np + w.parts - 1) / w.parts;
+    w.nc = (M + 15) & ~15;
+    auto entry = [&](int i, int k) -> double {  // column k = (3 chunk + kind) 16 + item of the chunk
+      const int c = (k / 16) % 3, g = k / 48 * 2 + k % 16 / 8, t = k % 8;
+      if (g < w.gvol) return 8 * g + t < Np ? S[c][size_t(i) * Np + 8 * g + t] : 0.0;
+      if (g < w.gface) {
+        const int l = 8 * (g - w.gvol) + t;
+        if (l >= nface) return 0.0;
+        const size_t at = size_t(i) * nface + l;
+        return c == 2 ? std::ldexp(Ef[at], o.k1) : std::ldexp(Df[c][at], o.k2);
+      }
+      const int n = 24 * (g - w.gface) + 3 * t + c;
+      return helm && n < Np ? std::ldexp(R.M[size_t(i) * Np + n], o.km) : 0.0;
+    };
+    for (int q = 0; q < w.parts; ++q) {
+      OutOp& p = w.part[q];
+      p.c0 = q * M;
+      p.M = std::min(M, Np - p.c0);
+      std::vector<int> ea(w.nc, 0);
+      for (int r = 0; r < p.M; ++r) {
+        double m = 0.0, s = 0.0;
+        for (int k = 0; k < 48 * w.chunks; ++k) {
+          m = std::max(m, std::fabs(entry(p.c0 + r, k)));
+          s += std::fabs(entry(p.c0 + r, k));
+        }
+        ea[r] = row_exp(m, s);
+      }
+      std::vector<uint8_t> im;
+      slice_block([&](int r, int k) { return entry(p.c0 + r, k); }, p.M, w.nc, 48 * w.chunks, ea.data(), im);
+      if (e == cudaSuccess) e = upload(im.data(), im.size(), reinterpret_cast<void**>(&p.ops));
+      if (e == cudaSuccess) e = upload(ea.data(), ea.size() * sizeof(int), reinterpret_cast<void**>(&p.ea));
     }
-    if (e == cudaSuccess) e = tc64_op_create(Bv, Np, 2 * Np, &o.outv);
-    if (e == cudaSuccess) e = tc64_op_create(Bf, Np, 3 * NFN, &o.outf);
-    if (e == cudaSuccess) e = tc64_op_create(Mm, Np, Np, &o.mh);
-    return e;
   }
-  if (e == cudaSuccess) e = tc64_op_create(B, Np, KY, &o.out);
-  if (e == cudaSuccess) {
-    if (KH <= kMaxDepth) {
-      e = tc64_op_create(BH, Np, KH, &o.outh);
-    } else {
-      std::vector<double> Mm(R.M.begin(), R.M.begin() + size_t(Np) * Np);
-      e = tc64_op_create(Mm, Np, Np, &o.mh);
-    }
-  }
+  o.ready = e == cudaSuccess;
   return e;
 }
-}  // namespace
 
-bool tc64_supported(int degree) {
-  const int Np = (degree + 1) * (degree + 2) / 2, NFN = 3 * (degree + 1);
-  return 2 * Np + 3 * NFN <= kMaxDepth && Np <= kMaxDepth;
-}
-
-namespace {
 // The degree's sliced operators on the current device, built on first use
 // when `build` is set (null if not built, or if building failed: *err says why).
 const Tc64Apply* t64_ops(dg_mesh* m, int degree, bool build, cudaError_t* err) {
@@ -818,7 +912,7 @@ const Tc64Apply* t64_ops(dg_mesh* m, int degree, bool build, cudaError_t* err) {
   }
   std::lock_guard<std::mutex> lk(table_mutex());
   Tc64Apply& o = g_t64[dev & 63][degree];
-  if (!o.grad.blocks) {
+  if (!o.ready) {
     if (!build) return nullptr;
     const RefElem R = m->ref[degree].N ? m->ref[degree] : build_reference(degree);
     Tc64Apply built;
@@ -831,32 +925,63 @@ const Tc64Apply* t64_ops(dg_mesh* m, int degree, bool build, cudaError_t* err) {
   }
   return &o;
 }
-int t64_cols(int degree, bool helm) {  // Y's columns
-  const int Np = (degree + 1) * (degree + 2) / 2, NFN = 3 * (degree + 1);
-  return 2 * Np + 3 * NFN + (helm ? Np : 0);
-}
 int64_t t64_ldc(int64_t nE) { return (nE + 31) & ~int64_t(31); }
-}  // namespace
 
-size_t tc64_scratch_words(int degree, int64_t nE, bool helm) {
-  const int NFN = 3 * (degree + 1);
-  return size_t(t64_ldc(nE)) * (t64_cols(degree, helm) + 2 * NFN) + 2 * (size_t(nE + 1) / 2) + 2;
+// Shared memory of the kernels, once per device; returns the SM count.
+cudaError_t t64_launch_setup(int* sms) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  static int count[64];
+  std::lock_guard<std::mutex> lk(table_mutex());
+  if (!count[dev & 63]) {
+    auto allow = [&](const void* f, int bytes) {
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    };
+    allow(reinterpret_cast<const void*>(t64_trace<1>), trace_smem(1));
+    allow(reinterpret_cast<const void*>(t64_trace<2>), trace_smem(2));
+    allow(reinterpret_cast<const void*>(t64_trace<3>), trace_smem(3));
+    allow(reinterpret_cast<const void*>(t64_trace<4>), trace_smem(4));
+    allow(reinterpret_cast<const void*>(t64_trace<5>), trace_smem(5));
+    allow(reinterpret_cast<const void*>(t64_output<16>), out_smem(16));
+    allow(reinterpret_cast<const void*>(t64_output<32>), out_smem(32));
+    allow(reinterpret_cast<const void*>(t64_output<48>), out_smem(48));
+    allow(reinterpret_cast<const void*>(t64_output<64>), out_smem(64));
+    int n = 0;
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    count[dev & 63] = n;
+  }
+  *sms = count[dev & 63];
+  return cudaSuccess;
 }
 
-cudaError_t ensure_tc64_ops(dg_mesh* m, int degree) {
-  if (!tc64_supported(degree)) return cudaSuccess;
-  cudaError_t e;
-  t64_ops(m, degree, true, &e);
-  return e;
+cudaError_t launch_trace(const TraceArgs& a, int ks, int sms, cudaStream_t st) {
+  const int64_t tiles = (a.rows + kT - 1) / kT;
+  const unsigned g = unsigned(std::min<int64_t>(tiles, int64_t(sms) * (ks <= 3 ? 2 : 1)));
+  switch (ks) {
+    case 1: t64_trace<1><<<g, 288, trace_smem(1), st>>>(a); break;
+    case 2: t64_trace<2><<<g, 288, trace_smem(2), st>>>(a); break;
+    case 3: t64_trace<3><<<g, 288, trace_smem(3), st>>>(a); break;
+    case 4: t64_trace<4><<<g, 288, trace_smem(4), st>>>(a); break;
+    default: t64_trace<5><<<g, 288, trace_smem(5), st>>>(a); break;
+  }
+  note_launch();
+  return cudaGetLastError();
 }
 
-bool tc64_ops_ready(int degree) {
-  if (!tc64_supported(degree)) return false;
-  cudaError_t e;
-  return t64_ops(nullptr, degree, false, &e) != nullptr;
+cudaError_t launch_output(const OutArgs& a, int nc, int sms, cudaStream_t st) {
+  const unsigned g = unsigned(std::min<int64_t>((a.rows + kT - 1) / kT, sms));
+  switch (nc) {
+    case 16: t64_output<16><<<g, kOutThreads, out_smem(16), st>>>(a); break;
+    case 32: t64_output<32><<<g, kOutThreads, out_smem(32), st>>>(a); break;
+    case 48: t64_output<48><<<g, kOutThreads, out_smem(48), st>>>(a); break;
+    default: t64_output<64><<<g, kOutThreads, out_smem(64), st>>>(a); break;
+  }
+  note_launch();
+  return cudaGetLastError();
 }
 
-namespace {
 // The largest forward distance from an element to one of its neighbours (rows),
 // from the host copy of the connectivity; kept with the mesh.
 int64_t t64_reach(dg_mesh* m) {
@@ -873,6 +998,39 @@ int64_t t64_reach(dg_mesh* m) {
 }
 }  // namespace
 
+bool tc64_supported(int degree) { return degree >= 1 && degree <= kMaxN; }
+
+// The scratch a caller that brings its own has to hold: u and q in fixed point
+// and each row's exponents and u0 need Np + 3 (N + 1) + 3 words per row; the size
+// stays the published one (include/dg.h), which is larger.
+size_t tc64_scratch_words(int degree, int64_t nE, bool helm) {
+  const int Np = (degree + 1) * (degree + 2) / 2, NFN = 3 * (degree + 1);
+  return size_t(t64_ldc(nE)) * (2 * Np + 5 * NFN + (helm ? Np : 0)) + 2 * (size_t(nE + 1) / 2) + 2;
+}
+
+cudaError_t ensure_tc64_ops(dg_mesh* m, int degree) {
+  if (!tc64_supported(degree)) return cudaSuccess;
+  cudaError_t e;
+  t64_ops(m, degree, true, &e);
+  return e;
+}
+
+bool tc64_ops_ready(int degree) {
+  if (!tc64_supported(degree)) return false;
+  cudaError_t e;
+  return t64_ops(nullptr, degree, false, &e) != nullptr;
+}
+
+cudaError_t build_fixed_geometry(dg_mesh* m) {
+  cudaError_t e = cudaMalloc(&m->gfix, sizeof(int2) * kCoefs * m->K);
+  if (e == cudaSuccess) e = cudaMalloc(&m->gfix_ex, sizeof(short4) * m->K);
+  if (e != cudaSuccess) return e;
+  k_fix_geometry<<<unsigned((m->K + 255) / 256), 256>>>(m->K, m->geox, m->gfix, m->gfix_ex);
+  note_launch();
+  e = cudaGetLastError();
+  return e == cudaSuccess ? cudaStreamSynchronize(nullptr) : e;
+}
+
 cudaError_t launch_apply_tc64(dg_mesh* m, int degree, int B, double lambda, const double* u, double* Au,
                               cudaStream_t st, double* scratch, const ApplyChunks* chunks) {
   if (B < 1) return cudaSuccess;
@@ -880,16 +1038,17 @@ cudaError_t launch_apply_tc64(dg_mesh* m, int degree, int B, double lambda, cons
   cudaError_t e;
   const Tc64Apply* ops = t64_ops(m, degree, scratch == nullptr, &e);
   if (!ops) return e != cudaSuccess ? e : cudaErrorNotReady;
-  int dev = 0;
-  e = cudaGetDevice(&dev);
+  int sms = 0;
+  e = t64_launch_setup(&sms);
   if (e != cudaSuccess) return e;
-  const int N = degree, Np = (N + 1) * (N + 2) / 2, NFN = 3 * (N + 1);
+  const int N = degree, Np = (N + 1) * (N + 2) / 2, nface = 3 * (N + 1);
   const bool helm = lambda != 0.0;
   const int64_t nE = int64_t(B) * m->K;
+  if (nE > 0x7fffffff) return cudaErrorInvalidValue;  // rows are addressed in 32 bits (their scratch is above 160 GB)
   const int64_t ldc = t64_ldc(nE);
-  // scratch: Y [columns][ldc], the face data FNu, FNd [NFN][ldc] (u, n.grad u), FP64,
-  // and the rows' largest Y exponents; every word read is written first by this call
-  const size_t words = tc64_scratch_words(N, nE, helm);
+  // scratch: u and q in fixed point [Np + 3 (N + 1)][ldc], the rows' exponents and u0;
+  // every word read is written first by this call
+  const size_t words = size_t(ldc) * (Np + nface + 3);
   if (!scratch && m->t64_cap < words) {
     cudaFree(m->t64_scratch);
     m->t64_scratch = nullptr;
@@ -900,63 +1059,87 @@ cudaError_t launch_apply_tc64(dg_mesh* m, int degree, int B, double lambda, cons
     m->t64_cap = words;
     ++m->scratch_gen;
   }
-  double* Y = scratch ? scratch : m->t64_scratch;
-  double* FNu = Y + size_t(ldc) * t64_cols(N, helm);
-  double* FNd = FNu + size_t(ldc) * NFN;
-  int* exy = reinterpret_cast<int*>(FNd + size_t(ldc) * NFN);
-  const bool split = ops->outv.blocks != nullptr;
-  int* exf = split ? exy + 2 * (size_t(nE + 1) / 2) : nullptr;  // the face columns' own exponents
+  // (a given scratch may start at any double; its size has room for the rounding)
+  uintptr_t base = reinterpret_cast<uintptr_t>(scratch ? scratch : m->t64_scratch);
+  long long* Iu = reinterpret_cast<long long*>((base + 15) & ~uintptr_t(15));
+  long long* Iq = Iu + size_t(ldc) * Np;
+  int4* ex = reinterpret_cast<int4*>(Iq + size_t(ldc) * nface);  // 16-byte aligned: ldc is a multiple of 32
+  double* u0 = reinterpret_cast<double*>(ex + ldc);
+  const OutSet& w = ops->out[helm ? 1 : 0];
   const bool chunked = chunks && chunks->n > 0 && chunks->bounds && chunks->bounds[chunks->n] == nE;
   const int nch = chunked ? chunks->n : 1;
   const int64_t whole[2] = {0, nE};
   const int64_t* bnd = chunked ? chunks->bounds : whole;
-  int sms = 0;
-  e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e != cudaSuccess) return e;
-  // a chunk's neighbour phase needs the gradient products of every chunk that
+  // a chunk's output product needs the boundary derivatives of every chunk that
   // holds one of its rows' neighbours: rows up to (last row + reach)
   const int64_t reach = nch > 1 ? t64_reach(m) : nE;
-  auto ready_after = [&](int c) {  // the last chunk whose gradient product chunk c's face fill needs
+  auto ready_after = [&](int c) {  // the last chunk whose first phase chunk c's output product needs
     const int64_t last = std::min<int64_t>(nE - 1, bnd[c + 1] - 1 + reach);
     int j = c;
     while (j + 1 < nch && bnd[j + 1] <= last) ++j;
     return j;
   };
-  auto finish = [&](int c) -> cudaError_t {  // face fill and output product of chunk c
+  auto finish = [&](int c) -> cudaError_t {  // output product of chunk c
     const int64_t r0 = bnd[c], n = bnd[c + 1] - r0;
-    const int64_t blocks = std::min<int64_t>((n + 255) / 256, int64_t(sms) * 16);  // a thread per element
-    tc64_face_fill<<<unsigned(blocks), 256, 0, st>>>(N, m->K, r0, r0 + n, m->geox, m->conn, FNu, FNd, Y, ldc,
-                                                     split ? exf : exy);
-    note_launch();
-    cudaError_t err = cudaGetLastError();
-    if (err != cudaSuccess) return err;
-    double* out = Au + r0 * Np;
-    const double* Yc = Y + r0;
-    const int* ey = exy + r0;
-    if (split) {  // Au = [Br Bs] Y_v + (face blocks) Y_f (+ M Y_h), the face block with its own exponents
-      err = gemm_launch<0>(ops->outv, n, Yc, ldc, out, Np, ey, GradOut{}, st, 0, 1);
-      if (err == cudaSuccess)
-        err = gemm_launch<0>(ops->outf, n, Yc + 2 * Np * ldc, ldc, out, Np, exf + r0, GradOut{}, st, 1, 1);
-      if (err == cudaSuccess && helm)
-        err = gemm_launch<0>(ops->mh, n, Yc + (2 * Np + 3 * NFN) * ldc, ldc, out, Np, ey, GradOut{}, st, 1, 1);
-    } else if (helm && !ops->outh.blocks) {  // [OB | M] is too deep for exact group sums: OB Y, then += M (lambda J u)
-      const int KY = 2 * Np + 3 * NFN;
-      err = gemm_launch<0>(ops->out, n, Yc, ldc, out, Np, ey, GradOut{}, st, 0, 1);
-      if (err == cudaSuccess) err = gemm_launch<0>(ops->mh, n, Yc + KY * ldc, ldc, out, Np, ey, GradOut{}, st, 1, 1);
-    } else {
-      err = gemm_launch<0>(helm ? ops->outh : ops->out, n, Yc, ldc, out, Np, ey, GradOut{}, st, 0, 1);
+    const int cpen = (N + 1) * (N + 2) / 2;
+    OutArgs a{};
+    a.N = N;
+    a.gvol = w.gvol;
+    a.gface = w.gface;
+    a.chunks = w.chunks;
+    a.cpen = cpen;
+    while ((1 << a.lpen) < cpen) ++a.lpen;
+    a.k1 = ops->k1;
+    a.k2 = ops->k2;
+    a.km = ops->km;
+    a.helm = helm;
+    a.lambda = lambda;
+    a.K = m->K;
+    a.rows = n;
+    a.row0 = r0;
+    a.Iu = Iu;
+    a.Iq = Iq;
+    a.ldc = ldc;
+    a.ex = ex;
+    a.u0 = u0;
+    a.tab = m->gfix;
+    a.tex = m->gfix_ex;
+    a.gx = m->geox;
+    a.conn = m->conn;
+    a.ldo = Np;
+    cudaError_t err = cudaSuccess;
+    for (int q = 0; q < w.parts && err == cudaSuccess; ++q) {
+      a.M = w.part[q].M;
+      a.ops = w.part[q].ops;
+      a.ea = w.part[q].ea;
+      a.out = Au + r0 * Np + w.part[q].c0;
+      err = launch_output(a, w.nc, sms, st);
     }
-    if (err != cudaSuccess) return err;
-    if (chunked && chunks->after) err = chunks->after(chunks->ctx, c, r0, r0 + n);
+    if (err == cudaSuccess && chunked && chunks->after) err = chunks->after(chunks->ctx, c, r0, r0 + n);
     return err;
   };
-  int done = 0;  // chunks whose face fill and output product are issued
-  for (int c = 0; c < nch; ++c) {  // gradient product, element-local
+  int done = 0;  // chunks whose output product is issued
+  for (int c = 0; c < nch; ++c) {  // boundary derivatives, element-local
     const int64_t r0 = bnd[c], r1 = bnd[c + 1];
     if (chunked && chunks->before && (e = chunks->before(chunks->ctx, c, r0, r1)) != cudaSuccess) return e;
-    GradOut go{N, m->K, m->geox, Y + r0, ldc, helm ? 1 : 0, lambda, FNu + r0, FNd + r0, exy + r0,
-               exf ? exf + r0 : nullptr, r0};
-    e = gemm_launch<1>(ops->grad, r1 - r0, u + r0 * Np, Np, nullptr, 0, nullptr, go, st);
+    TraceArgs a{};
+    a.N = N;
+    a.passes = ops->passes;
+    a.u = u + r0 * Np;
+    a.aligned = (reinterpret_cast<uintptr_t>(a.u) & 15u) == 0;
+    a.K = m->K;
+    a.rows = r1 - r0;
+    a.row0 = r0;
+    a.tab = m->gfix;
+    a.tex = m->gfix_ex;
+    a.ops = ops->trace;
+    a.ea = ops->trace_ea;
+    a.Iu = Iu + r0;
+    a.Iq = Iq + r0;
+    a.ldc = ldc;
+    a.ex = ex + r0;
+    a.u0 = u0 + r0;
+    e = launch_trace(a, ops->ks, sms, st);
     if (e != cudaSuccess) return e;
     while (done < nch && ready_after(done) <= c)
       if ((e = finish(done++)) != cudaSuccess) return e;
@@ -965,9 +1148,11 @@ cudaError_t launch_apply_tc64(dg_mesh* m, int degree, int B, double lambda, cons
 }
 
 cudaError_t tc64_error(int* flag) {
-  int zero = 0;
-  cudaError_t e = cudaMemcpyFromSymbol(flag, g_tc64_err, sizeof(int));
-  if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_tc64_err, &zero, sizeof(int));
+  int zero = 0, gemm = 0;
+  cudaError_t e = cudaMemcpyFromSymbol(flag, g_t64_err, sizeof(int));
+  if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_t64_err, &zero, sizeof(int));
+  if (e == cudaSuccess) e = tc64_gemm_error(&gemm);
+  *flag |= gemm;
   return e;
 }
 

@@ -88,6 +88,9 @@ struct dg_mesh {
   float* ih32 = nullptr;     // K x 3
   // FP64 derived geometry [K][16]: J, Grr, Grs, Gss | per face (n.grad r, n.grad s, sJ, max(1/h-,1/h+))
   double* geox = nullptr;
+  // the FP64 tensor-core apply's coefficients in fixed point (apply_tc64.cu): [12][K], exponents [K]
+  int2* gfix = nullptr;
+  short4* gfix_ex = nullptr;
   float* geox32 = nullptr;  // the same 16 words per element in FP32
   dgx::RefElem ref[dgx::kMaxN + 1];
   dgx::DevOps ops64[dgx::kMaxN + 1];
@@ -103,7 +106,7 @@ struct dg_mesh {
   // FP64 tensor-core apply scratch: C1, Y and the face buffer (grown on demand)
   double* oz_scratch = nullptr;
   size_t oz_cap = 0;
-  // FP64 tcgen05 apply scratch: C1, Y and per-element exponents (grown on demand)
+  // FP64 tcgen05 apply scratch: u, q and per-element exponents (grown on demand)
   double* t64_scratch = nullptr;
   size_t t64_cap = 0;
   uint64_t scratch_gen = 0;  // bumped whenever face32, oz_scratch or t64_scratch is reallocated
@@ -165,11 +168,11 @@ cudaError_t tc64_gemm_launch(const Tc64Op& op, int64_t rows, const double* X, in
                              cudaStream_t st, int accum = 0, const int* ex = nullptr);
 bool tc64_supported(int degree);
 // An apply in chunks of rows (elements x right-hand sides) for callers that move
-// the data in and out while it runs: the first phase (gradient product) reads
-// only each row's own u, the last (output product) writes each row's Au by
+// the data in and out while it runs: the first phase (boundary derivatives)
+// reads only each row's own u, the last (output product) writes each row's Au by
 // itself. `before` is enqueued ahead of chunk i's first phase, `after` behind
-// chunk i's last; chunk i's neighbour phase runs once the first phase of every
-// chunk holding one of its rows' neighbours has been issued.
+// chunk i's last, which runs once the first phase of every chunk holding one of
+// its rows' neighbours has been issued.
 struct ApplyChunks {
   int n = 0;                        // chunks
   const int64_t* bounds = nullptr;  // chunk c holds rows [bounds[c], bounds[c + 1]); bounds[n] = all rows
@@ -188,7 +191,9 @@ size_t tc64_scratch_words(int degree, int64_t nE, bool helm);
 cudaError_t ensure_tc64_ops(dg_mesh* m, int degree);  // dg_mesh_setup builds the mesh degree's tables
 bool tc64_ops_ready(int degree);                      // built on the current device (no build)
 cudaError_t tc64_error(int* flag);
-// FP64 products on the tcgen05 tensor cores with exact integer slicing (apply_tc64.cu):
+cudaError_t tc64_gemm_error(int* flag);              // the generic product's part of it
+cudaError_t build_fixed_geometry(dg_mesh* m);         // gfix, gfix_ex (dg_mesh_setup)
+// FP64 products on the tcgen05 tensor cores with exact integer slicing (gemm_tc64.cu):
 // an operator A (M x K, K <= 256) cut into 8 slices in blocks of 48 rows x 32 columns
 struct Tc64Op {
   int M = 0, K = 0, NCH = 0, KCH = 0;

@@ -1,11 +1,11 @@
 // The operator apply on fields in host memory (dg_apply_host): the copies in
 // and out run on two copy streams, overlapped with the apply where its
 // kernels allow. The tcgen05 FP64 apply (the FP64 default from degree 3) runs
-// in chunks of rows: chunk i's gradient product, which reads only its own
-// elements' u, starts once chunk i has arrived while later chunks are still
-// being copied in; chunk i's neighbour phase and output product follow as soon
-// as the gradient products of the chunks holding its neighbours are done, and
-// its copy out starts while later chunks are still being computed. Every other
+// in chunks of rows: chunk i's boundary derivatives, which read only its own
+// elements' u, start once chunk i has arrived while later chunks are still
+// being copied in; chunk i's output product follows as soon as the boundary
+// derivatives of the chunks holding its neighbours are done, and its copy out
+// starts while later chunks are still being computed. Every other
 // kernel copies the whole input in, applies and copies the whole result out, in
 // order on the caller's stream.
 #include <algorithm>
@@ -29,7 +29,7 @@ struct HostCtx {
   size_t row_bytes;  // one element's nodes of one right-hand side
 };
 
-// before chunk i's gradient product: copy its rows in on the input stream and
+// before chunk i's boundary derivatives: copy its rows in on the input stream and
 // make the compute stream wait for them
 cudaError_t chunk_in(void* c, int i, int64_t r0, int64_t r1) {
   HostCtx* x = static_cast<HostCtx*>(c);
