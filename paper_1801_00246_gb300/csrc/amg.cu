@@ -18,6 +18,7 @@
 #include <cmath>
 #include <cstring>
 #include <random>
+#include <type_traits>
 #include <vector>
 
 #include "dg_internal.h"
@@ -42,7 +43,8 @@ struct AmgLevel {
   DevCsr A, P, R;      // P: n x n_next, R = P^T
   double* dinv = nullptr;
   double rho = 1.0;    // largest eigenvalue estimate of D^{-1} A
-  double *x = nullptr, *b = nullptr, *r = nullptr, *d = nullptr, *t = nullptr;  // [B][n]
+  double *x = nullptr, *b = nullptr;  // [B][n], from the second level (the caller's on the first)
+  double *r = nullptr, *d = nullptr;  // [B][n]
 };
 
 struct Amg {
@@ -214,61 +216,73 @@ __global__ void k_probe_vec(int64_t K, int Np, int ncol0, int nvec, const int32_
   }
 }
 
-// y[b] = alpha A x[b] + beta y[b]  (one row per thread group of 4 lanes)
-__global__ void k_spmv(int64_t n, int64_t xs, int64_t ys, int B, const int64_t* __restrict__ ptr,
+// What a row's product s = (A x)_i becomes; the Chebyshev steps use it where it
+// is formed, so that a smoothing reads and writes each vector once. The matrix
+// rows and the gathered vector are the traffic: at the degree-1 level of 524,288
+// triangles a product takes 88 us, and a step apart from it took 20 to 60 us more.
+enum SpmvOp {
+  SP_MUL,    // y = s
+  SP_ADD,    // y += s
+  SP_RES,    // y = b - s
+  SP_FIRST,  // y = b - s (residual); d = c1 dinv y
+  SP_PRE,    // y = x + (c1 x + c2 dinv (b - s)): x = the first step from zero
+  SP_POST    // y += x + (c1 x + c2 dinv (b - s)): x = the first step, b its residual
+};
+struct SpmvArgs {
+  const double *b = nullptr, *dinv = nullptr;
+  double* d = nullptr;
+  double c1 = 0.0, c2 = 0.0;
+};
+
+// One row per group of LPR lanes, LPR near a quarter of the rows' entries.
+template <int LPR, int OP>
+__global__ void k_spmv(int64_t n, int64_t xs, int64_t ys, const int64_t* __restrict__ ptr,
                        const int32_t* __restrict__ col, const double* __restrict__ val, const double* __restrict__ x,
-                       double* __restrict__ y, double alpha, double beta) {
-  const int64_t g = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 2;
-  const int lane = threadIdx.x & 3;
-  const int b = blockIdx.y;
+                       double* __restrict__ y, const SpmvArgs a) {
+  const int64_t g = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) / LPR;
+  const int lane = threadIdx.x & (LPR - 1);
   const bool valid = g < n;  // every lane stays for the shuffles below
-  const double* xb = x + size_t(b) * xs;
+  const double* xb = x + size_t(blockIdx.y) * xs;
   double s = 0.0;
   if (valid)
-    for (int64_t k = ptr[g] + lane; k < ptr[g + 1]; k += 4) s += val[k] * xb[col[k]];
-  s += __shfl_down_sync(0xffffffffu, s, 2, 4);
-  s += __shfl_down_sync(0xffffffffu, s, 1, 4);
-  if (valid && lane == 0) {
-    double* yb = y + size_t(b) * ys;
-    yb[g] = alpha * s + (beta != 0.0 ? beta * yb[g] : 0.0);
+    for (int64_t k = ptr[g] + lane; k < ptr[g + 1]; k += LPR) s += val[k] * xb[col[k]];
+#pragma unroll
+  for (int o = LPR / 2; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o, LPR);
+  if (!valid || lane != 0) return;
+  const size_t i = size_t(blockIdx.y) * ys + g;
+  if (OP == SP_MUL) y[i] = s;
+  if (OP == SP_ADD) y[i] += s;
+  if (OP == SP_RES) y[i] = a.b[i] - s;
+  if (OP == SP_FIRST) {
+    const double r = a.b[i] - s;
+    y[i] = r;
+    a.d[i] = a.c1 * a.dinv[g] * r;
+  }
+  if (OP == SP_PRE || OP == SP_POST) {
+    const double di = xb[g];
+    const double t = a.c1 * di + a.c2 * a.dinv[g] * (a.b[i] - s);
+    y[i] = OP == SP_PRE ? di + t : y[i] + di + t;
   }
 }
 
-// Chebyshev pieces on [B][n] vectors, dinv shared across the batch
-__global__ void k_cheb0(int64_t n, int B, const double* __restrict__ dinv, const double* __restrict__ res,
-                        double* __restrict__ d, double* __restrict__ x, double c0, int zero_x) {
-  const int64_t tot = n * B;
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < tot; i += int64_t(gridDim.x) * blockDim.x) {
-    const double di = c0 * dinv[i % n] * res[i];
-    d[i] = di;
-    x[i] = zero_x ? di : x[i] + di;
-  }
-}
-__global__ void k_cheb1(int64_t n, int B, const double* __restrict__ dinv, const double* __restrict__ Ad,
-                        double* __restrict__ res, double* __restrict__ d, double* __restrict__ x, double c1,
-                        double c2) {
-  const int64_t tot = n * B;
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < tot; i += int64_t(gridDim.x) * blockDim.x) {
-    const double r = res[i] - Ad[i];
-    res[i] = r;
-    const double di = c1 * d[i] + c2 * dinv[i % n] * r;
-    d[i] = di;
-    x[i] += di;
-  }
-}
-__global__ void k_copy(int64_t n, const double* __restrict__ a, double* __restrict__ b) {
+// d[b] = c0 dinv r[b]: the first Chebyshev step from zero
+__global__ void k_cheb0(int64_t n, const double* __restrict__ dinv, const double* __restrict__ r,
+                        double* __restrict__ d, double c0) {
+  const size_t off = size_t(blockIdx.y) * n;
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
-    b[i] = a[i];
+    d[off + i] = c0 * dinv[i] * r[off + i];
 }
-// y[b] = Minv x[b] (dense, n <= a few thousand)
+// y[b] = Minv x[b] (dense, n <= a few thousand), a warp per row
 __global__ void k_dense(int64_t n, const double* __restrict__ M, const double* __restrict__ x, double* __restrict__ y) {
-  const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  const int b = blockIdx.y;
+  const int64_t i = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
   if (i >= n) return;
-  const double* xb = x + size_t(b) * n;
+  const double* xb = x + size_t(blockIdx.y) * n;
   double s = 0.0;
-  for (int64_t j = 0; j < n; ++j) s += M[size_t(i) * n + j] * xb[j];
-  y[size_t(b) * n + i] = s;
+  for (int64_t j = lane; j < n; j += 32) s += M[size_t(i) * n + j] * xb[j];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  if (lane == 0) y[size_t(blockIdx.y) * n + i] = s;
 }
 
 inline int eg(int64_t n) {
@@ -301,11 +315,26 @@ cudaError_t upload(Amg* a, const Csr& h, DevCsr& d) {
   return cudaSuccess;
 }
 
-cudaError_t spmv(const DevCsr& A, int B, int64_t xs, int64_t ys, const double* x, double* y, double alpha,
-                 double beta, cudaStream_t st) {
-  const int64_t threads = A.n * 4;
-  dim3 grid(unsigned((threads + 255) / 256), unsigned(B));
-  k_spmv<<<grid, 256, 0, st>>>(A.n, xs, ys, B, A.ptr, A.col, A.val, x, y, alpha, beta);
+template <int OP>
+cudaError_t spmv(const DevCsr& A, int B, int64_t xs, int64_t ys, const double* x, double* y, cudaStream_t st,
+                 const SpmvArgs& a = {}) {
+  const int64_t avg = A.n ? A.nnz / A.n : 0;
+  auto go = [&](auto lanes) {
+    constexpr int LPR = decltype(lanes)::value;
+    const dim3 grid(unsigned((A.n * LPR + 255) / 256), unsigned(B));
+    k_spmv<LPR, OP><<<grid, 256, 0, st>>>(A.n, xs, ys, A.ptr, A.col, A.val, x, y, a);
+  };
+  if (avg <= 6) go(std::integral_constant<int, 2>{});
+  else if (avg <= 24) go(std::integral_constant<int, 4>{});
+  else if (avg <= 48) go(std::integral_constant<int, 8>{});
+  else if (avg <= 96) go(std::integral_constant<int, 16>{});
+  else go(std::integral_constant<int, 32>{});
+  note_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t dense(const Amg* a, int B, const double* b, double* x, cudaStream_t st) {
+  k_dense<<<dim3(unsigned((a->nc * 32 + 127) / 128), unsigned(B)), 128, 0, st>>>(a->nc, a->cinv, b, x);
   note_launch();
   return cudaGetLastError();
 }
@@ -486,9 +515,10 @@ cudaError_t amg_build(dg_mesh* m, int degree, double lambda, int B, Amg** out, c
     for (int64_t i = 0; i < A.n; ++i) di[i] = 1.0 / d[i];
     ACK(cudaMalloc(&L.dinv, sizeof(double) * A.n));
     a->allocs.push_back(L.dinv);
-    a->bytes += sizeof(double) * A.n * (1 + 5 * size_t(B));  // dinv and the five level vectors
+    a->bytes += sizeof(double) * A.n * (1 + (lev == 0 ? 2 : 4) * size_t(B));  // dinv and the level vectors
     ACK(cudaMemcpy(L.dinv, di.data(), sizeof(double) * A.n, cudaMemcpyHostToDevice));
-    for (double** p : {&L.x, &L.b, &L.r, &L.d, &L.t}) {
+    for (double** p : {&L.r, &L.d, &L.x, &L.b}) {
+      if (lev == 0 && (p == &L.x || p == &L.b)) continue;
       ACK(cudaMalloc(p, sizeof(double) * A.n * B));
       ACK(poison(*p, sizeof(double) * A.n * B, POISON_AMG));
       a->allocs.push_back(*p);
@@ -501,83 +531,43 @@ cudaError_t amg_build(dg_mesh* m, int degree, double lambda, int B, Amg** out, c
 
 namespace {
 
-// Chebyshev smoothing on level l (degree 2), x either zero or given
-cudaError_t smooth(Amg* a, int l, int B, bool zero_x, cudaStream_t st) {
+// One V-cycle from x = 0 on level l: Chebyshev smoothing of degree 2 before and
+// after the correction from the next level.
+cudaError_t vcyc(Amg* a, int l, int B, const double* b, double* x, cudaStream_t st) {
+  if (l == int(a->L.size())) return dense(a, B, b, x, st);
   AmgLevel& L = a->L[l];
   const int64_t n = L.A.n;
   const double lmin = L.rho / 10.0, lmax = 1.1 * L.rho;
   const double theta = 0.5 * (lmax + lmin), delta = 0.5 * (lmax - lmin), sigma = theta / delta;
-  double rk = 1.0 / sigma;
-  if (zero_x) {
-    k_copy<<<eg(n * B), 256, 0, st>>>(n * B, L.b, L.r);
-    note_launch();
-  } else {
-    k_copy<<<eg(n * B), 256, 0, st>>>(n * B, L.b, L.r);
-    note_launch();
-    ACK(spmv(L.A, B, n, n, L.x, L.r, -1.0, 1.0, st));
-  }
-  k_cheb0<<<eg(n * B), 256, 0, st>>>(n, B, L.dinv, L.r, L.d, L.x, 1.0 / theta, zero_x ? 1 : 0);
+  const double rk = 1.0 / sigma, rnew = 1.0 / (2.0 * sigma - rk);
+  const double c0 = 1.0 / theta, c1 = rnew * rk, c2 = 2.0 * rnew / delta;
+  k_cheb0<<<dim3(unsigned(eg(n)), unsigned(B)), 256, 0, st>>>(n, L.dinv, b, L.d, c0);
   note_launch();
-  const double rnew = 1.0 / (2.0 * sigma - rk);
-  ACK(spmv(L.A, B, n, n, L.d, L.t, 1.0, 0.0, st));
-  k_cheb1<<<eg(n * B), 256, 0, st>>>(n, B, L.dinv, L.t, L.r, L.d, L.x, rnew * rk, 2.0 * rnew / delta);
-  note_launch();
-  return cudaGetLastError();
-}
-
-cudaError_t vcyc(Amg* a, int l, int B, cudaStream_t st) {
-  if (l == int(a->L.size())) {
-    dim3 grid(unsigned((a->nc + 127) / 128), unsigned(B));
-    k_dense<<<grid, 128, 0, st>>>(a->nc, a->cinv, a->cb, a->cx);
-    note_launch();
-    return cudaGetLastError();
-  }
-  AmgLevel& L = a->L[l];
-  const int64_t n = L.A.n;
-  ACK(smooth(a, l, B, true, st));
-  // residual after pre-smoothing, restricted to the next level
-  k_copy<<<eg(n * B), 256, 0, st>>>(n * B, L.b, L.r);
-  note_launch();
-  ACK(spmv(L.A, B, n, n, L.x, L.r, -1.0, 1.0, st));
+  ACK(spmv<SP_PRE>(L.A, B, n, n, L.d, x, st, SpmvArgs{b, L.dinv, nullptr, c1, c2}));
+  ACK(spmv<SP_RES>(L.A, B, n, n, x, L.r, st, SpmvArgs{b}));
   const bool last = (l + 1 == int(a->L.size()));
   const int64_t nn = last ? a->nc : a->L[l + 1].A.n;
   double* nb = last ? a->cb : a->L[l + 1].b;
   double* nx = last ? a->cx : a->L[l + 1].x;
-  ACK(spmv(L.R, B, n, nn, L.r, nb, 1.0, 0.0, st));
-  ACK(vcyc(a, l + 1, B, st));
-  ACK(spmv(L.P, B, nn, n, nx, L.x, 1.0, 1.0, st));
-  ACK(smooth(a, l, B, false, st));
-  return cudaGetLastError();
+  ACK(spmv<SP_MUL>(L.R, B, n, nn, L.r, nb, st));
+  ACK(vcyc(a, l + 1, B, nb, nx, st));
+  ACK(spmv<SP_ADD>(L.P, B, nn, n, nx, x, st));
+  ACK(spmv<SP_FIRST>(L.A, B, n, n, x, L.r, st, SpmvArgs{b, L.dinv, L.d, c0}));
+  return spmv<SP_POST>(L.A, B, n, n, L.d, x, st, SpmvArgs{L.r, L.dinv, nullptr, c1, c2});
 }
 
 }  // namespace
 
-// x = V(b), one V-cycle for B right-hand sides ([B][n] each, n = rows of level 0)
-cudaError_t amg_vcycle(Amg* a, const double* b, double* x, cudaStream_t st) {
-  if (a->L.empty()) {  // tiny problem: dense solve only
-    k_copy<<<eg(a->nc * a->B), 256, 0, st>>>(a->nc * a->B, b, a->cb);
-    note_launch();
-    dim3 grid(unsigned((a->nc + 127) / 128), unsigned(a->B));
-    k_dense<<<grid, 128, 0, st>>>(a->nc, a->cinv, a->cb, x);
-    note_launch();
-    return cudaGetLastError();
-  }
-  AmgLevel& L0 = a->L[0];
-  const int64_t n = L0.A.n;
-  k_copy<<<eg(n * a->B), 256, 0, st>>>(n * a->B, b, L0.b);
-  note_launch();
-  ACK(vcyc(a, 0, a->B, st));
-  k_copy<<<eg(n * a->B), 256, 0, st>>>(n * a->B, L0.x, x);
-  note_launch();
-  return cudaGetLastError();
-}
+// x = V(b), one V-cycle for B right-hand sides ([B][n] each, n = rows of level 0; a
+// dense solve on a tiny problem)
+cudaError_t amg_vcycle(Amg* a, const double* b, double* x, cudaStream_t st) { return vcyc(a, 0, a->B, b, x, st); }
 
 int amg_levels(const Amg* a) { return a ? int(a->L.size()) + 1 : 0; }
 size_t amg_bytes(const Amg* a) { return a ? a->bytes : 0; }
 
 // y = A0 x for the Amg's batch of right-hand sides
 cudaError_t amg_apply_fine(Amg* a, const double* x, double* y, cudaStream_t st) {
-  return spmv(a->A0, a->B, a->A0.n, a->A0.n, x, y, 1.0, 0.0, st);
+  return spmv<SP_MUL>(a->A0, a->B, a->A0.n, a->A0.n, x, y, st);
 }
 
 }  // namespace dgx
