@@ -120,6 +120,20 @@ cudaError_t walloc(Workspace* w, T** p, size_t count) {
 
 inline int npd(int N) { return (N + 1) * (N + 2) / 2; }
 
+// V neighbouring values, one access
+template <typename T, int V>
+struct alignas(sizeof(T) * V) Pack {
+  T v[V];
+};
+template <typename T, int V>
+__device__ __forceinline__ Pack<T, V> load_pack(const T* p, int64_t i) {
+  return *reinterpret_cast<const Pack<T, V>*>(p + i * V);
+}
+template <typename T, int V>
+__device__ __forceinline__ void store_pack(T* p, int64_t i, const Pack<T, V>& a) {
+  *reinterpret_cast<Pack<T, V>*>(p + i * V) = a;
+}
+
 // ---------------------------------------------------------------- reductions
 __device__ __forceinline__ double block_sum(double v, double* sh) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
@@ -147,7 +161,11 @@ __global__ void k_dot(int64_t n, const TX* __restrict__ x, const TY* __restrict_
   if (threadIdx.x == 0) partial[(size_t(b) * kRedBlocks + blockIdx.x) * 2] = t;
 }
 
-// x += alpha p; r -= alpha Ap; partial: r.r and r.zold (zold may be null)
+// x += alpha p; r -= alpha Ap; partial: r.r and r.zold (zold may be null). Seven
+// passes over memory and four FP64 operations a value (157 us of the FP64 pipe and
+// 195 us of memory for 23.6M values): 16-byte accesses keep enough of them in flight
+// (268 -> 219 us).
+template <int V, int XV>
 __global__ void k_update_xr(int64_t n, const double* __restrict__ scal, double* __restrict__ x,
                             double* __restrict__ r, const double* __restrict__ p, const double* __restrict__ Ap,
                             const double* __restrict__ zold, double* __restrict__ partial) {
@@ -156,17 +174,37 @@ __global__ void k_update_xr(int64_t n, const double* __restrict__ scal, double* 
   const double alpha = scal[b * kNS + S_ALPHA];
   const size_t off = size_t(b) * n;
   double rr = 0.0, rz = 0.0;
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
-    x[off + i] += alpha * p[off + i];
-    const double ri = r[off + i] - alpha * Ap[off + i];
-    r[off + i] = ri;
-    rr += ri * ri;
-    if (zold) rz += ri * zold[off + i];
+  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n / V; i += int64_t(gridDim.x) * blockDim.x) {
+    Pack<double, V> xi, ri = load_pack<double, V>(r + off, i), zi{};
+#pragma unroll
+    for (int k = 0; k < V; k += XV) *reinterpret_cast<Pack<double, XV>*>(xi.v + k) = load_pack<double, XV>(x + off + i * V + k, 0);
+    const Pack<double, V> pi = load_pack<double, V>(p + off, i), ai = load_pack<double, V>(Ap + off, i);
+    if (zold) zi = load_pack<double, V>(zold + off, i);
+#pragma unroll
+    for (int k = 0; k < V; ++k) {
+      xi.v[k] += alpha * pi.v[k];
+      ri.v[k] -= alpha * ai.v[k];
+      rr += ri.v[k] * ri.v[k];
+      if (zold) rz += ri.v[k] * zi.v[k];
+    }
+#pragma unroll
+    for (int k = 0; k < V; k += XV) store_pack<double, XV>(x + off + i * V + k, 0, *reinterpret_cast<Pack<double, XV>*>(xi.v + k));
+    store_pack<double, V>(r + off, i, ri);
   }
   double t = block_sum(rr, sh);
   if (threadIdx.x == 0) partial[(size_t(b) * kRedBlocks + blockIdx.x) * 2] = t;
   t = block_sum(rz, sh);
   if (threadIdx.x == 0) partial[(size_t(b) * kRedBlocks + blockIdx.x) * 2 + 1] = t;
+}
+// Pairs where every right-hand side starts on one. x may be a caller's array off
+// 16-byte alignment: its accesses are split then, the order of the sums is the same.
+void update_xr(dim3 g, int64_t n, const double* scal, double* x, double* r, const double* p, const double* Ap,
+               const double* zold, double* partial, cudaStream_t st) {
+  if (n % 2 != 0) k_update_xr<1, 1><<<g, kRedThreads, 0, st>>>(n, scal, x, r, p, Ap, zold, partial);
+  else if ((reinterpret_cast<uintptr_t>(x) & 15u) == 0)
+    k_update_xr<2, 2><<<g, kRedThreads, 0, st>>>(n, scal, x, r, p, Ap, zold, partial);
+  else k_update_xr<2, 1><<<g, kRedThreads, 0, st>>>(n, scal, x, r, p, Ap, zold, partial);
+  note_launch();
 }
 
 enum FinMode { FIN_INIT_BB = 0, FIN_INIT_RZ, FIN_ALPHA, FIN_RR, FIN_BETA, FIN_BETA_FLEX };
@@ -364,62 +402,200 @@ __global__ void k_invmass(int Np, int64_t K, int B, const double* __restrict__ g
 }
 
 // ------------------------------------------------------------- multigrid pieces
-// Chebyshev first step: if zero_x: res = rhs, d = c0 dinv rhs, x = d;
-//                       else      d = c0 dinv res, x += d.
-template <typename T>
-__global__ void k_cheb_first(int64_t n, int64_t ntot, const T* __restrict__ dinv, const T* __restrict__ rhs,
+// Chebyshev steps on [B][n] vectors (the batch in the grid's second dimension),
+// V values at a time. They are bound by memory, so each writes only what a later
+// step reads: x is first formed by the second step (as the sum of the first two
+// corrections), the residual from x = 0 is the right-hand side itself, and the
+// last step after the coarse correction leaves only x. 37 instead of 44 vector
+// passes per V-cycle level at degree 3; with 16-byte accesses in place of 4-byte
+// ones and a 64-bit remainder per value.
+// r = rhs (- Ax), d = c0 dinv r; res = r if res is given; x = d (Ax null: from zero)
+// or x += d if x is given
+template <typename T, int V>
+__global__ void k_cheb_first(int64_t n, const T* __restrict__ dinv, const T* __restrict__ rhs,
                              const T* __restrict__ Ax, T* __restrict__ res, T* __restrict__ d, T* __restrict__ x,
                              T c0) {
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < ntot; i += int64_t(gridDim.x) * blockDim.x) {
-    const T ri = Ax ? rhs[i] - Ax[i] : rhs[i];  // Ax null: x = 0
-    res[i] = ri;
-    const T di = c0 * dinv[i % n] * ri;
-    d[i] = di;
-    x[i] = Ax ? x[i] + di : di;
+  const size_t off = size_t(blockIdx.y) * n;
+  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n / V; i += int64_t(gridDim.x) * blockDim.x) {
+    Pack<T, V> r = load_pack<T, V>(rhs + off, i), di, xi;
+    const Pack<T, V> w = load_pack<T, V>(dinv, i);
+    if (Ax) {
+      const Pack<T, V> a = load_pack<T, V>(Ax + off, i);
+#pragma unroll
+      for (int k = 0; k < V; ++k) r.v[k] -= a.v[k];
+    }
+#pragma unroll
+    for (int k = 0; k < V; ++k) di.v[k] = c0 * w.v[k] * r.v[k];
+    if (res) store_pack<T, V>(res + off, i, r);
+    if (d) store_pack<T, V>(d + off, i, di);
+    if (x) {
+      if (Ax) {
+        xi = load_pack<T, V>(x + off, i);
+#pragma unroll
+        for (int k = 0; k < V; ++k) di.v[k] += xi.v[k];
+      }
+      store_pack<T, V>(x + off, i, di);
+    }
   }
 }
 
-// res -= Ad; d = c1 d + c2 dinv res; x += d
-template <typename T>
-__global__ void k_cheb_step(int64_t n, int64_t ntot, const T* __restrict__ dinv, const T* __restrict__ Ad,
-                            T* __restrict__ res, T* __restrict__ d, T* __restrict__ x, T c1, T c2) {
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < ntot; i += int64_t(gridDim.x) * blockDim.x) {
-    const T ri = res[i] - Ad[i];
-    res[i] = ri;
-    const T di = c1 * d[i] + c2 * dinv[i % n] * ri;
-    d[i] = di;
-    x[i] += di;
+// r = res - Ad, e = c1 d + c2 dinv r; keep: res_out = r, d = e; then
+// x += e (SUM_X), x += d + e with the previous d (SUM_BOTH), x = d + e (SET_BOTH)
+enum { SUM_X, SUM_BOTH, SET_BOTH };
+template <typename T, int V>
+__global__ void k_cheb_step(int64_t n, const T* __restrict__ dinv, const T* __restrict__ Ad, const T* res,
+                            T* res_out, T* __restrict__ d, T* __restrict__ x, T c1, T c2, int keep, int mode) {
+  const size_t off = size_t(blockIdx.y) * n;
+  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n / V; i += int64_t(gridDim.x) * blockDim.x) {
+    Pack<T, V> r = load_pack<T, V>(res + off, i), dn, xi{};
+    const Pack<T, V> a = load_pack<T, V>(Ad + off, i), w = load_pack<T, V>(dinv, i), dp = load_pack<T, V>(d + off, i);
+    if (mode != SET_BOTH) xi = load_pack<T, V>(x + off, i);
+#pragma unroll
+    for (int k = 0; k < V; ++k) {
+      r.v[k] -= a.v[k];
+      dn.v[k] = c1 * dp.v[k] + c2 * w.v[k] * r.v[k];
+      xi.v[k] = mode == SUM_X ? xi.v[k] + dn.v[k] : (xi.v[k] + dp.v[k]) + dn.v[k];
+    }
+    if (keep) {
+      store_pack<T, V>(res_out + off, i, r);
+      store_pack<T, V>(d + off, i, dn);
+    }
+    store_pack<T, V>(x + off, i, xi);
   }
+}
+
+// Degree transfers, an element per thread: the block's elements pass through
+// shared memory (contiguous in memory both ways), the coarse values stay in
+// registers (NPC of them) and every thread reads the same entry of P at a time.
+// 8 -> 4 on 524,288 elements in FP32: 68 us each, against 163 us (restriction) and
+// 210 us (prolongation) with one thread per entry reading P and its element from L1;
+// with 4-byte accesses one at a time they took 119 and 134 us.
+template <typename T>
+__device__ __forceinline__ T* transfer_smem() {
+  extern __shared__ __align__(16) unsigned char transfer_raw[];
+  return reinterpret_cast<T*>(transfer_raw);
+}
+__host__ __device__ constexpr int pad4(int n) { return (n + 3) & ~3; }
+
+// A block's contiguous values, 16 bytes at a time with four accesses in flight
+// (a tile starts on a 16-byte boundary: its elements are a multiple of 32), and the
+// tail one by one; f(k, value) or f(k) per value.
+template <typename T, typename F>
+__device__ __forceinline__ void for_tile(int n, F&& f) {
+  constexpr int V = 16 / sizeof(T);
+#pragma unroll 4
+  for (int k = threadIdx.x * V; k < n / V * V; k += blockDim.x * V) f(k, std::integral_constant<int, V>{});
+  for (int k = n / V * V + threadIdx.x; k < n; k += blockDim.x) f(k, std::integral_constant<int, 1>{});
 }
 
 // rc[e][j] = sum_i P[i][j] (res[e][i] - Ad[e][i]) (restriction R = P^T of the
 // residual after the last smoothing step, which nothing else reads)
-template <typename T>
-__global__ void k_sub_restrict(int Npf, int Npc, int64_t nE, const T* __restrict__ P, const T* __restrict__ res,
-                               const T* __restrict__ Ad, T* __restrict__ rc) {
-  const int64_t idx = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (idx >= nE * Npc) return;
-  const int64_t e = nE * Npc < (int64_t(1) << 31) ? int64_t(uint32_t(idx) / uint32_t(Npc)) : idx / Npc;
-  const int j = int(idx - e * Npc);
-  const T* re = res + e * Npf;
-  const T* ae = Ad + e * Npf;
-  T acc = T(0);
-  for (int i = 0; i < Npf; ++i) acc += P[size_t(i) * Npc + j] * (re[i] - ae[i]);
-  rc[idx] = acc;
+template <typename T, int NPC>
+__global__ void __launch_bounds__(128) k_sub_restrict(int Npf, int64_t nE, const T* __restrict__ P,
+                                                      const T* __restrict__ res, const T* __restrict__ Ad,
+                                                      T* __restrict__ rc) {
+  T* sP = transfer_smem<T>();                // [Npf][pad4(NPC)]
+  T* sv = sP + Npf * pad4(NPC);              // [blockDim][Npf], then [blockDim][NPC]
+  const int64_t e0 = int64_t(blockIdx.x) * blockDim.x, base = e0 * Npf;
+  const int live = int(nE - e0 < int64_t(blockDim.x) ? nE - e0 : int64_t(blockDim.x));
+  for (int k = threadIdx.x; k < Npf * pad4(NPC); k += blockDim.x) {
+    const int i = k / pad4(NPC), q = k - i * pad4(NPC);
+    sP[k] = q < NPC ? P[i * NPC + q] : T(0);
+  }
+  for_tile<T>(live * Npf, [&](int k, auto v) {
+    constexpr int V = decltype(v)::value;
+    Pack<T, V> a = *reinterpret_cast<const Pack<T, V>*>(res + base + k);
+    const Pack<T, V> b = *reinterpret_cast<const Pack<T, V>*>(Ad + base + k);
+#pragma unroll
+    for (int t = 0; t < V; ++t) a.v[t] -= b.v[t];
+    *reinterpret_cast<Pack<T, V>*>(sv + k) = a;
+  });
+  __syncthreads();
+  T acc[NPC];
+#pragma unroll
+  for (int q = 0; q < NPC; ++q) acc[q] = T(0);
+#pragma unroll 4
+  for (int i = 0; i < Npf; ++i) {
+    const T v = sv[threadIdx.x * Npf + i];  // (past the last element: stale values, not stored)
+#pragma unroll
+    for (int q = 0; q < NPC; ++q) acc[q] += sP[i * pad4(NPC) + q] * v;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < NPC; ++q) sv[threadIdx.x * NPC + q] = acc[q];
+  __syncthreads();
+  for_tile<T>(live * NPC, [&](int k, auto v) {
+    constexpr int V = decltype(v)::value;
+    *reinterpret_cast<Pack<T, V>*>(rc + e0 * NPC + k) = *reinterpret_cast<const Pack<T, V>*>(sv + k);
+  });
 }
 
 // xf[e][i] += sum_j P[i][j] xc[e][j]
+template <typename T, int NPC>
+__global__ void __launch_bounds__(128) k_prolong(int Npf, int64_t nE, const T* __restrict__ P,
+                                                 const T* __restrict__ xc, T* __restrict__ xf) {
+  T* sP = transfer_smem<T>();
+  T* sv = sP + Npf * pad4(NPC);
+  const int64_t e0 = int64_t(blockIdx.x) * blockDim.x, base = e0 * Npf;
+  const int live = int(nE - e0 < int64_t(blockDim.x) ? nE - e0 : int64_t(blockDim.x));
+  for (int k = threadIdx.x; k < Npf * pad4(NPC); k += blockDim.x) {
+    const int i = k / pad4(NPC), q = k - i * pad4(NPC);
+    sP[k] = q < NPC ? P[i * NPC + q] : T(0);
+  }
+  for_tile<T>(live * NPC, [&](int k, auto v) {
+    constexpr int V = decltype(v)::value;
+    *reinterpret_cast<Pack<T, V>*>(sv + k) = *reinterpret_cast<const Pack<T, V>*>(xc + e0 * NPC + k);
+  });
+  __syncthreads();
+  T c[NPC];
+#pragma unroll
+  for (int q = 0; q < NPC; ++q) c[q] = sv[threadIdx.x * NPC + q];
+  __syncthreads();
+#pragma unroll 4
+  for (int i = 0; i < Npf; ++i) {
+    T acc = T(0);
+#pragma unroll
+    for (int q = 0; q < NPC; ++q) acc += sP[i * pad4(NPC) + q] * c[q];
+    sv[threadIdx.x * Npf + i] = acc;
+  }
+  __syncthreads();
+  for_tile<T>(live * Npf, [&](int k, auto v) {
+    constexpr int V = decltype(v)::value;
+    Pack<T, V> a = *reinterpret_cast<const Pack<T, V>*>(xf + base + k);
+    const Pack<T, V> b = *reinterpret_cast<const Pack<T, V>*>(sv + k);
+#pragma unroll
+    for (int t = 0; t < V; ++t) a.v[t] += b.v[t];
+    *reinterpret_cast<Pack<T, V>*>(xf + base + k) = a;
+  });
+}
+
+// Either transfer between degrees with Npf and Npc nodes: the largest block whose
+// tile fits the default 48 KB of shared memory (both operands are at most 66 wide).
+template <typename T, int NPC>
+void launch_transfer_n(int Npf, int64_t nE, const T* P, const T* a, const T* b, T* out, cudaStream_t st) {
+  auto bytes = [&](int E) { return (size_t(E) * Npf + size_t(Npf) * pad4(NPC)) * sizeof(T); };
+  int E = 128;
+  while (E > 32 && (bytes(E) > 48 * 1024 || nE / E < 304)) E /= 2;  // (two blocks per SM where the mesh allows)
+  const unsigned g = unsigned((nE + E - 1) / E);
+  if (b) k_sub_restrict<T, NPC><<<g, E, bytes(E), st>>>(Npf, nE, P, a, b, out);
+  else k_prolong<T, NPC><<<g, E, bytes(E), st>>>(Npf, nE, P, a, out);
+  note_launch();
+}
+// b given: out = P^T (a - b); b null: out += P a
 template <typename T>
-__global__ void k_prolong(int Npf, int Npc, int64_t nE, const T* __restrict__ P, const T* __restrict__ xc,
-                          T* __restrict__ xf) {
-  const int64_t idx = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (idx >= nE * Npf) return;
-  const int64_t e = nE * Npf < (int64_t(1) << 31) ? int64_t(uint32_t(idx) / uint32_t(Npf)) : idx / Npf;
-  const int i = int(idx - e * Npf);
-  const T* ce = xc + e * Npc;
-  T acc = T(0);
-  for (int j = 0; j < Npc; ++j) acc += P[size_t(i) * Npc + j] * ce[j];
-  xf[idx] += acc;
+cudaError_t launch_transfer(int Npf, int Npc, int64_t nE, const T* P, const T* a, const T* b, T* out, cudaStream_t st) {
+  switch (Npc) {
+    case 3: launch_transfer_n<T, 3>(Npf, nE, P, a, b, out, st); break;
+    case 6: launch_transfer_n<T, 6>(Npf, nE, P, a, b, out, st); break;
+    case 10: launch_transfer_n<T, 10>(Npf, nE, P, a, b, out, st); break;
+    case 15: launch_transfer_n<T, 15>(Npf, nE, P, a, b, out, st); break;
+    case 21: launch_transfer_n<T, 21>(Npf, nE, P, a, b, out, st); break;
+    case 28: launch_transfer_n<T, 28>(Npf, nE, P, a, b, out, st); break;
+    case 36: launch_transfer_n<T, 36>(Npf, nE, P, a, b, out, st); break;
+    case 45: launch_transfer_n<T, 45>(Npf, nE, P, a, b, out, st); break;
+    default: launch_transfer_n<T, 55>(Npf, nE, P, a, b, out, st); break;
+  }
+  return cudaGetLastError();
 }
 
 // Reductions always run kRedBlocks blocks per right-hand side (blocks past the
@@ -638,7 +814,7 @@ cudaError_t coarse_cg(Ctx& c, int degree, const double* rhs, double* x, int& ite
     CK(launch_apply(c.m, degree, DG_F64, B, c.lambda, w->cp, w->cAp, c.st));
     k_dot<<<g, kRedThreads, 0, c.st>>>(n, w->cp, w->cAp, w->cpartial); note_launch();
     k_finalize<<<B, kRedThreads, 0, c.st>>>(FIN_ALPHA, w->cscal, w->cpartial); note_launch();
-    k_update_xr<<<g, kRedThreads, 0, c.st>>>(n, w->cscal, x, w->cr, w->cp, w->cAp, nullptr, w->cpartial); note_launch();
+    update_xr(g, n, w->cscal, x, w->cr, w->cp, w->cAp, nullptr, w->cpartial, c.st);
     k_finalize<<<B, kRedThreads, 0, c.st>>>(FIN_RR, w->cscal, w->cpartial); note_launch();
     k_dot<<<g, kRedThreads, 0, c.st>>>(n, w->cr, w->cr, w->cpartial); note_launch();
     k_finalize<<<B, kRedThreads, 0, c.st>>>(FIN_BETA, w->cscal, w->cpartial); note_launch();
@@ -714,8 +890,7 @@ cudaError_t coarse_pcg_amg(Ctx& c, int degree, const double* rhs, double* x, int
     CK(amg_apply_fine(w->amg, w->cp, w->cAp, c.st));  // the probed matrix is this degree's operator
     k_dot<<<g, kRedThreads, 0, c.st>>>(n, w->cp, w->cAp, w->cpartial); note_launch();
     k_finalize<<<B, kRedThreads, 0, c.st>>>(FIN_ALPHA, w->cscal, w->cpartial); note_launch();
-    k_update_xr<<<g, kRedThreads, 0, c.st>>>(n, w->cscal, x, w->cr, w->cp, w->cAp, nullptr, w->cpartial);
-    note_launch();
+    update_xr(g, n, w->cscal, x, w->cr, w->cp, w->cAp, nullptr, w->cpartial, c.st);
     k_finalize<<<B, kRedThreads, 0, c.st>>>(FIN_RR, w->cscal, w->cpartial); note_launch();
     return cudaSuccess;
   };
@@ -775,28 +950,43 @@ const double* transfer_ptr<double>(dg_mesh* m, int Nf, int Nc) { return m->trans
 template <typename T>
 constexpr dg_prec prec_of() { return std::is_same<T, double>::value ? DG_F64 : DG_F32; }
 
-// Chebyshev smoothing of the given degree on level l.
-template <typename T>
-cudaError_t chebyshev(Ctx& c, int l, bool zero_x) {
+// Chebyshev smoothing of the given degree on level l: from x = 0 before the coarse
+// correction (d, and through *res the residual it belongs to, are kept for the
+// restriction), or from the corrected x after it (only x is kept).
+template <typename T, int V>
+cudaError_t chebyshev_v(Ctx& c, int l, bool zero_x, const T** res) {
   LevelVecs<T>& v = levels<T>(c.w)[l];
-  const int deg = c.o->degrees[l];
+  const int deg = c.o->degrees[l], steps = c.o->cheb_degree;
   const int64_t n = int64_t(c.m->K) * npd(deg);
-  const int64_t nt = n * c.B;
+  const dim3 g(unsigned(egrid(n / V)), unsigned(c.B));
   const double rho = c.w->rho[l];
   const double lmin = rho / 10.0, lmax = 1.1 * rho;
   const double theta = 0.5 * (lmax + lmin), delta = 0.5 * (lmax - lmin), sigma = theta / delta;
   double rk = 1.0 / sigma;
+  const bool only = steps == 1;  // no second step forms x
   if (!zero_x) CK(launch_apply(c.m, deg, prec_of<T>(), c.B, c.lambda, v.x, v.Ad, c.st));
-  // res = rhs (- A x), d = D^{-1} res / theta, x (+)= d
-  k_cheb_first<T><<<egrid(nt), 256, 0, c.st>>>(n, nt, v.dinv, v.rhs, zero_x ? nullptr : v.Ad, v.res, v.d, v.x,
-                                                T(1.0 / theta)); note_launch();
-  for (int k = 1; k < c.o->cheb_degree; ++k) {
+  // r = rhs (- A x), d = D^{-1} r / theta
+  k_cheb_first<T, V><<<g, 256, 0, c.st>>>(n, v.dinv, v.rhs, zero_x ? nullptr : v.Ad, zero_x || only ? nullptr : v.res,
+                                          zero_x || !only ? v.d : nullptr, only ? v.x : nullptr, T(1.0 / theta));
+  note_launch();
+  for (int k = 1; k < steps; ++k) {
     CK(launch_apply(c.m, deg, prec_of<T>(), c.B, c.lambda, v.d, v.Ad, c.st));
     const double rnew = 1.0 / (2.0 * sigma - rk);
-    k_cheb_step<T><<<egrid(nt), 256, 0, c.st>>>(n, nt, v.dinv, v.Ad, v.res, v.d, v.x, T(rnew * rk), T(2.0 * rnew / delta)); note_launch();
+    k_cheb_step<T, V><<<g, 256, 0, c.st>>>(n, v.dinv, v.Ad, zero_x && k == 1 ? v.rhs : v.res, v.res, v.d, v.x,
+                                           T(rnew * rk), T(2.0 * rnew / delta), zero_x || k + 1 < steps,
+                                           k > 1 ? SUM_X : (zero_x ? SET_BOTH : SUM_BOTH));
+    note_launch();
     rk = rnew;
   }
+  if (res) *res = only ? v.rhs : v.res;
   return cudaGetLastError();
+}
+template <typename T>
+cudaError_t chebyshev(Ctx& c, int l, bool zero_x, const T** res) {
+  // 16-byte accesses where every right-hand side starts on a 16-byte boundary
+  const int64_t n = int64_t(c.m->K) * npd(c.o->degrees[l]);
+  constexpr int V = 16 / sizeof(T);
+  return n % V == 0 ? chebyshev_v<T, V>(c, l, zero_x, res) : chebyshev_v<T, 1>(c, l, zero_x, res);
 }
 
 template <typename T>
@@ -824,19 +1014,19 @@ cudaError_t vcycle(Ctx& c, int l, int& coarse_iters) {
   }
   LevelVecs<T>& v = lv[l];
   // pre-smoothing from x = 0, then res = rhs - A x
-  CK(chebyshev<T>(c, l, true));
+  const T* res = nullptr;
+  CK(chebyshev<T>(c, l, true, &res));
   CK(launch_apply(c.m, deg, prec_of<T>(), c.B, c.lambda, v.d, v.Ad, c.st));
   // restrict res - A d, recurse, prolong
   const int degc = c.o->degrees[l + 1];
   const int Npf = npd(deg), Npc = npd(degc);
   const int64_t nE = int64_t(c.m->K) * c.B;
   const T* P = transfer_ptr<T>(c.m, deg, degc);
-  k_sub_restrict<T><<<int((nE * Npc + 255) / 256), 256, 0, c.st>>>(Npf, Npc, nE, P, v.res, v.Ad, lv[l + 1].rhs);
-  note_launch();
+  CK(launch_transfer<T>(Npf, Npc, nE, P, res, v.Ad, lv[l + 1].rhs, c.st));
   CK(vcycle<T>(c, l + 1, coarse_iters));
-  k_prolong<T><<<int((nE * Npf + 255) / 256), 256, 0, c.st>>>(Npf, Npc, nE, P, lv[l + 1].x, v.x); note_launch();
+  CK(launch_transfer<T>(Npf, Npc, nE, P, lv[l + 1].x, nullptr, v.x, c.st));
   // post-smoothing
-  CK(chebyshev<T>(c, l, false));
+  CK(chebyshev<T>(c, l, false, nullptr));
   return cudaGetLastError();
 }
 
@@ -970,7 +1160,7 @@ cudaError_t pcg_half1(Ctx& c, double* x, bool flexible) {
   CK(launch_apply(c.m, c.m->N, DG_F64, B, c.lambda, w->p, w->Ap, c.st));
   k_dot<<<g, kRedThreads, 0, c.st>>>(n, w->p, w->Ap, w->partial); note_launch();
   k_finalize<<<B, kRedThreads, 0, c.st>>>(FIN_ALPHA, w->scal, w->partial); note_launch();
-  k_update_xr<<<g, kRedThreads, 0, c.st>>>(n, w->scal, x, w->r, w->p, w->Ap, flexible ? w->z : nullptr, w->partial); note_launch();
+  update_xr(g, n, w->scal, x, w->r, w->p, w->Ap, flexible ? w->z : nullptr, w->partial, c.st);
   k_finalize<<<B, kRedThreads, 0, c.st>>>(FIN_RR, w->scal, w->partial); note_launch();
   return cudaGetLastError();
 }
@@ -1398,7 +1588,7 @@ extern "C" dg_status dg_pcg_jacobi_solve_static(const dg_mesh* mc, int B, double
     SCK(launch_apply(m, m->N, DG_F64, B, lambda, p, Ap, st, c1));
     k_dot<<<g, kRedThreads, 0, st>>>(n, p, Ap, partial); note_launch();
     k_finalize<<<B, kRedThreads, 0, st>>>(FIN_ALPHA, scal, partial); note_launch();
-    k_update_xr<<<g, kRedThreads, 0, st>>>(n, scal, x, r, p, Ap, nullptr, partial); note_launch();
+    update_xr(g, n, scal, x, r, p, Ap, nullptr, partial, st);
     k_finalize<<<B, kRedThreads, 0, st>>>(FIN_RR, scal, partial); note_launch();
     ++it;
     if (it % 4 == 0 || it == max_iter) {
