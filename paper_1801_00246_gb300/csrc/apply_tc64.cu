@@ -78,30 +78,6 @@ __device__ __forceinline__ void bar_sync(int id, int threads) {
 
 __device__ __forceinline__ int64_t elem_of(int64_t row, int64_t K) { return row < K ? row : row % K; }
 
-// accumulator columns d .. d + rows += data digit x the operator's stacked rows
-__device__ __forceinline__ void issue_rows(uint32_t d, uint64_t a, uint64_t b, int rows, uint32_t acc) {
-  const int n0 = rows <= 256 ? rows : ((rows / 2 + 15) & ~15);
-  tc::mma_ss(d, a, b, tc::idesc_f16(128, n0, false), acc);
-  if (n0 < rows) tc::mma_ss(d + n0, a, b + ((n0 * 32) >> 4), tc::idesc_f16(128, rows - n0, false), acc);
-}
-// The digit products i + j <= 7 of 16 columns: data digits (slices of `aslice`
-// bytes at a) with the operator's (nc stacked rows each at b); `first` starts the sums.
-__device__ __forceinline__ void issue_step(uint32_t d, uint64_t a, int aslice, uint64_t b, int nc, bool first) {
-  issue_rows(d, a, b, kDigits * nc, first ? 0u : 1u);  // sums 0 .. 6
-  a += aslice >> 4;
-  if (first) {  // sums 1 .. 6 are there, sum 7 starts here
-    issue_rows(d + nc, a, b, (kDigits - 1) * nc, 1u);
-    issue_rows(d + kDigits * nc, a, b + (((kDigits - 1) * nc * 32) >> 4), nc, 0u);
-  } else {
-    issue_rows(d + nc, a, b, kDigits * nc, 1u);
-  }
-#pragma unroll 1
-  for (int j = 2; j < kDigits; ++j) {
-    a += aslice >> 4;
-    issue_rows(d + j * nc, a, b, (kSums - j) * nc, 1u);
-  }
-}
-
 __device__ __forceinline__ int node_of(int N, int f, int j) {  // local node of face f's j-th node
   auto rs = [N](int row) { return row * (N + 1) - row * (row - 1) / 2; };
   return f == 0 ? j : (f == 1 ? rs(j) + (N - j) : rs(N - j));
@@ -227,7 +203,7 @@ __global__ void __launch_bounds__(288, KS <= 3 ? 2 : 1) t64_trace(const TraceArg
           const uint64_t b0 = bd + ((kResident ? p * kPass : 0) >> 4);
 #pragma unroll 1
           for (int ks = 0; ks < KS; ++ks)
-            issue_step(tb, ad + ((ks * 256) >> 4), kSlice, b0 + ((ks * kTraceStep) >> 4), kTraceN, ks == 0);
+            fx::issue_step<32>(tb, ad + ((ks * 256) >> 4), kSlice, b0 + ((ks * kTraceStep) >> 4), kTraceN, ks == 0);
           tc::mma_commit(accf);
         }
         __syncwarp();
@@ -483,7 +459,7 @@ __global__ void __launch_bounds__(kOutThreads, 1) t64_output(const OutArgs a) {
           wait(bfull + b, (n / kStages) & 1u, abort_flag);
           tc::fence_after();
           if (lane == 0) {
-            issue_step(tb + ab * kSums * NC, ad + (((g & 1u) * kChunkBytes + c * 256) >> 4), kChunkSlice,
+            fx::issue_step<32>(tb + ab * kSums * NC, ad + (((g & 1u) * kChunkBytes + c * 256) >> 4), kChunkSlice,
                        bd + ((b * kStage) >> 4), NC, kc == 0 && c == 0);
             tc::mma_commit(bempty + b);
             if (c == 2) tc::mma_commit(empty + (g & 1u));
@@ -721,23 +697,6 @@ __global__ void __launch_bounds__(kOutThreads, 1) t64_output(const OutArgs a) {
 // An operator block image: rows scaled to integers below 2^56 (one exponent
 // per row, or one for all), cut into digits (fix64.cuh), digit i of row r at
 // stacked row i nc + r, in 16-column steps of the canonical layout.
-int ceil_log2(double x) {  // e with x < 2^e (0 for zero)
-  int e = 0;
-  std::frexp(x, &e);
-  return e;
-}
-// A row's exponent: its entries below 2^e, and its absolute sum below 2^{e+6}, so
-// that a product's digit sums stay below 2^62 where fx::from_sums joins them.
-int row_exp(double mx, double l1) { return std::max(ceil_log2(mx), ceil_log2(l1) - 6); }
-
-uint16_t fp16_int(int d) {  // exact for |d| <= 2048
-  if (d == 0) return 0;
-  const int m = std::abs(d);
-  int e = 0;
-  while ((m >> e) > 1) ++e;
-  return uint16_t((d < 0 ? 0x8000 : 0) | ((e + 15) << 10) | (((m << 10) >> e) & 0x3ff));
-}
-
 // A(r, k) for r < M <= nc, k < K (columns past K are zero; K a multiple of 16 on
 // the way out), ea[r] the row exponents to use.
 template <typename F>
@@ -750,13 +709,12 @@ void slice_block(const F& A, int M, int nc, int K, const int* ea, std::vector<ui
     for (int k = 0; k < K; ++k) {
       const double v = A(r, k);
       if (v == 0.0) continue;
-      long long x = std::llround(std::ldexp(v, 56 - ea[r]));
+      int d[kDigits];
+      fx::digits_of(v, ea[r], d);
       uint8_t* blk = img.data() + base + size_t(k / 16) * step_bytes;
-      for (int i = kDigits - 1; i >= 0; --i) {  // last digit first
-        const int d = i == 0 ? int(x) : int((x + 128) & 255) - 128;
-        x = (x - d) >> 8;
+      for (int i = 0; i < kDigits; ++i) {
         const int R = i * nc + r, c = k % 16;
-        const uint16_t h = fp16_int(d);
+        const uint16_t h = fx::fp16_int(d[i]);
         std::memcpy(blk + size_t(R / 8) * 256 + (c / 8) * 128 + (R % 8) * 16 + (c % 8) * 2, &h, 2);
       }
     }
@@ -806,7 +764,7 @@ cudaError_t build_t64(const RefElem& R, Tc64Apply& o) {
     }
     l1 = std::max(l1, s);
   }
-  o.trace_ea = row_exp(mx, l1);
+  o.trace_ea = fx::row_exp(mx, l1);
   o.passes = (6 * N + kTraceN - 1) / kTraceN;
   o.ks = (Np + 15) / 16;
   std::vector<uint8_t> img;
@@ -888,7 +846,7 @@ cudaError_t build_t64(const RefElem& R, Tc64Apply& o) {
           m = std::max(m, std::fabs(entry(p.c0 + r, k)));
           s += std::fabs(entry(p.c0 + r, k));
         }
-        ea[r] = row_exp(m, s);
+        ea[r] = fx::row_exp(m, s);
       }
       std::vector<uint8_t> im;
       slice_block([&](int r, int k) { return entry(p.c0 + r, k); }, p.M, w.nc, 48 * w.chunks, ea.data(), im);

@@ -194,7 +194,7 @@ cudaError_t tc64_error(int* flag);
 cudaError_t tc64_gemm_error(int* flag);              // the generic product's part of it
 cudaError_t build_fixed_geometry(dg_mesh* m);         // gfix, gfix_ex (dg_mesh_setup)
 // FP64 products on the tcgen05 tensor cores with exact integer slicing (gemm_tc64.cu):
-// an operator A (M x K, K <= 256) cut into 8 slices in blocks of 48 rows x 32 columns
+// an operator A (M x K, K <= 256) cut into 7 digits in blocks of 48 rows x 32 columns
 struct Tc64Op {
   int M = 0, K = 0, NCH = 0, KCH = 0;
   uint8_t* blocks = nullptr;

@@ -19,11 +19,14 @@
 // leading digits), so FP32 accumulators hold sums of several hundred exactly.
 #pragma once
 
+#include <cmath>
 #include <cstdint>
 #include <cstring>
 
 #ifdef __CUDACC__
 #include <cuda_fp16.h>
+
+#include "tc05.cuh"
 #define DGX_HD __host__ __device__ __forceinline__
 #else
 #define DGX_HD inline
@@ -65,7 +68,7 @@ DGX_HD int exp_bound(double v) {
   return E == 0 ? kZeroExp : E - 1022;
 }
 
-// v 2^{B-E} for |v| < 2^E, truncated towards zero (B = 59 or 62)
+// v 2^{B-E} for |v| < 2^E, truncated towards zero (53 < B <= 62)
 template <int B>
 DGX_HD long long fix(double v, int E) {
   const long long b = bits_of(v);
@@ -183,7 +186,61 @@ __device__ __forceinline__ void digits4(const long long (&x)[4], uint8_t* dst, i
   for (int j = 0; j < kDigits; ++j)
     *reinterpret_cast<uint2*>(dst + j * slice_stride) = make_uint2(w[0][j], w[1][j]);
 }
+
+// accumulator columns d .. d + rows += data digit x the operator's stacked rows
+// (ROW bytes of shared memory apart: 32 for blocks 16 columns wide, 64 for 32)
+template <int ROW>
+__device__ __forceinline__ void issue_rows(uint32_t d, uint64_t a, uint64_t b, int rows, uint32_t acc) {
+  const int n0 = rows <= 256 ? rows : ((rows / 2 + 15) & ~15);
+  tc::mma_ss(d, a, b, tc::idesc_f16(128, n0, false), acc);
+  if (n0 < rows) tc::mma_ss(d + n0, a, b + ((n0 * ROW) >> 4), tc::idesc_f16(128, rows - n0, false), acc);
+}
+// The digit products i + j <= 7 of 16 columns: data digits (slices of `aslice`
+// bytes at a) with the operator's (nc stacked rows each at b); `first` starts the sums.
+template <int ROW>
+__device__ __forceinline__ void issue_step(uint32_t d, uint64_t a, int aslice, uint64_t b, int nc, bool first) {
+  issue_rows<ROW>(d, a, b, kDigits * nc, first ? 0u : 1u);  // sums 0 .. 6
+  a += aslice >> 4;
+  if (first) {  // sums 1 .. 6 are there, sum 7 starts here
+    issue_rows<ROW>(d + nc, a, b, (kDigits - 1) * nc, 1u);
+    issue_rows<ROW>(d + kDigits * nc, a, b + (((kDigits - 1) * nc * ROW) >> 4), nc, 0u);
+  } else {
+    issue_rows<ROW>(d + nc, a, b, kDigits * nc, 1u);
+  }
+#pragma unroll 1
+  for (int j = 2; j < kDigits; ++j) {
+    a += aslice >> 4;
+    issue_rows<ROW>(d + j * nc, a, b, (kSums - j) * nc, 1u);
+  }
+}
 #endif
+
+// ------------------------------------------------------------------ operators (host)
+inline int ceil_log2(double x) {  // e with x < 2^e (0 for zero)
+  int e = 0;
+  std::frexp(x, &e);
+  return e;
+}
+// A row's exponent: its entries below 2^e, and its absolute sum below 2^{e+6}, so
+// that a product's digit sums stay below 2^62 where from_sums joins them.
+inline int row_exp(double mx, double l1) { return imax(ceil_log2(mx), ceil_log2(l1) - 6); }
+
+inline uint16_t fp16_int(int d) {  // exact for |d| <= 2048
+  if (d == 0) return 0;
+  const int m = d < 0 ? -d : d;
+  int e = 0;
+  while ((m >> e) > 1) ++e;
+  return uint16_t((d < 0 ? 0x8000 : 0) | ((e + 15) << 10) | (((m << 10) >> e) & 0x3ff));
+}
+// The digits of v 2^{56-e} (|v| < 2^e), leading one first.
+inline void digits_of(double v, int e, int (&out)[kDigits]) {
+  long long x = std::llround(std::ldexp(v, 56 - e));
+  for (int i = kDigits - 1; i >= 0; --i) {  // last digit first
+    const int d = i == 0 ? int(x) : int((x + 128) & 255) - 128;
+    x = (x - d) >> 8;
+    out[i] = d;
+  }
+}
 
 }  // namespace fx
 }  // namespace dgx
