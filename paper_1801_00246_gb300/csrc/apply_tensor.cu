@@ -907,45 +907,6 @@ cudaError_t ensure_tensor_ops(dg_mesh* m, int degree, bool f64) {
   return f64 ? tensor_ops<double>(m, degree, &op) : tensor_ops<float>(m, degree, &op);
 }
 
-// A general FP64 operator for batched row products out[r] = A X[r] (the
-// advection's cubature interpolation and projection): sliced once on the host.
-cudaError_t sliced_op_create(const std::vector<double>& A, int M, int K, SlicedOp* op) {
-  std::vector<uint32_t> frag;
-  std::vector<int> ea;
-  op->M = M;
-  op->K = K;
-  // too long a sum for the FP32 group sums to stay exact (both kernels: 4 products
-  // of |slice| <= 127 over 256 terms stay below 2^24)
-  if (K > 256) return cudaErrorInvalidValue;
-  // the tcgen05 GEMM takes any row count; the mma.sync copy only within its
-  // instantiated shapes (it serves when the tcgen05 one is not built)
-  cudaError_t e = tc64_op_create(A, M, K, &op->t64);
-  if (e != cudaSuccess) return e;
-  slice_operator(A, M, K, Slices<double>::KS, false, op->Mt, op->Kt, frag, ea);
-  if (op->Mt * ONT > 48) return cudaSuccess;
-  e = cudaMalloc(&op->A, frag.size() * sizeof(uint32_t));
-  if (e == cudaSuccess) e = cudaMemcpy(op->A, frag.data(), frag.size() * sizeof(uint32_t), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMalloc(&op->ea, ea.size() * sizeof(int));
-  if (e == cudaSuccess) e = cudaMemcpy(op->ea, ea.data(), ea.size() * sizeof(int), cudaMemcpyHostToDevice);
-  return e;
-}
-
-void sliced_op_free(SlicedOp* op) {
-  cudaFree(op->A);
-  cudaFree(op->ea);
-  op->A = nullptr;
-  op->ea = nullptr;
-  tc64_op_free(&op->t64);
-}
-
-cudaError_t sliced_gemm(const SlicedOp& op, int64_t rows, const double* X, int64_t ldx, double* out, int64_t ldo,
-                        cudaStream_t st) {
-  if (op.t64.blocks) return tc64_gemm_launch(op.t64, rows, X, ldx, out, ldo, st);
-  if (!op.A) return cudaErrorInvalidValue;
-  return gemm<double>(op.Mt, rows, op.M, op.K, op.Kt, reinterpret_cast<const uint4*>(op.A), op.ea, X, ldx, out, ldo,
-                      nullptr, st);
-}
-
 // Reads and clears the pipelined kernels' timeout flag (synchronises the device).
 cudaError_t tensor_pipe_error(int* flag) {
   int zero = 0;

@@ -194,24 +194,13 @@ cudaError_t tc64_error(int* flag);
 cudaError_t tc64_gemm_error(int* flag);              // the generic product's part of it
 cudaError_t build_fixed_geometry(dg_mesh* m);         // gfix, gfix_ex (dg_mesh_setup)
 // FP64 products on the tcgen05 tensor cores with exact integer slicing (gemm_tc64.cu):
-// an operator A (M x K, K <= 256) cut into 7 digits in blocks of 48 rows x 32 columns
+// an operator A (M x K, sums short enough to stay exact) cut into 7 digits in blocks of
+// 48 rows x 32 columns
 struct Tc64Op {
   int M = 0, K = 0, NCH = 0, KCH = 0;
   uint8_t* blocks = nullptr;
   int* ea = nullptr;
 };
-// FP64 operator A (M x K, row-major) sliced for the tensor-core products out[r] = A X[r]:
-// the mma.sync fragment layout and the tcgen05 block layout (used when built)
-struct SlicedOp {
-  int M = 0, K = 0, Mt = 0, Kt = 0;
-  uint32_t* A = nullptr;
-  int* ea = nullptr;
-  Tc64Op t64;
-};
-cudaError_t sliced_op_create(const std::vector<double>& A, int M, int K, SlicedOp* op);
-void sliced_op_free(SlicedOp* op);
-cudaError_t sliced_gemm(const SlicedOp& op, int64_t rows, const double* X, int64_t ldx, double* out, int64_t ldo,
-                        cudaStream_t st);
 cudaError_t launch_nodes(const dg_mesh* m, int degree, double* x, double* y, cudaStream_t st);
 
 void set_error(const std::string& msg);

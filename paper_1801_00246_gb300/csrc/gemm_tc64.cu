@@ -27,10 +27,6 @@ using fx::kSums;
 constexpr int kT = 128;                      // rows per tile (MMA M)
 constexpr int kKC = 32;                      // data columns per chunk
 constexpr int kNC = 48;                      // output columns per pass (MMA N)
-// Longest sum: digit products are at most 2^14 (2^15 and 2^16 with a leading digit),
-// so the sums that carry the result (s <= 3: at most 2^16 + 3 2^14 a term, half of
-// it for an operator's lower digits) stay integers below 2^24 to this depth.
-constexpr int kMaxDepth = 256;
 constexpr int kASlice = kT * kKC * 2, kABytes = kDigits * kASlice;   // one data chunk, 7 digits: 56 KB
 constexpr int kBSlice = kNC * kKC * 2, kBBytes = kDigits * kBSlice;  // one operator block, 7 digits: 21 KB
 constexpr int kSmem = 2 * kABytes + 2 * kBBytes + 4 * kT * 4 + 12 * 8;  // the tail: 10 mbarriers, slot, 2 flags
@@ -270,13 +266,13 @@ __global__ void __launch_bounds__(kSlicers + 32, 1) tc64_gemm(int64_t rows, int 
 // ------------------------------------------------------------------ host side
 }  // namespace
 
-// A (M x K, row-major FP64) into the block layout of tc64_gemm.
+// A (M x K, row-major FP64) into the block layout of tc64_gemm; cudaErrorInvalidValue if
+// its sums are too long to stay exact (beyond some 400 terms).
 cudaError_t tc64_op_create(const std::vector<double>& A, int M, int K, Tc64Op* op) {
   op->M = M;
   op->K = K;
   op->NCH = (M + kNC - 1) / kNC;
   op->KCH = (K + kKC - 1) / kKC;
-  if (K > kMaxDepth) return cudaErrorInvalidValue;  // longer sums would leave the FP32 group sums inexact
   std::vector<uint8_t> img(size_t(op->NCH) * op->KCH * kBBytes, 0);
   std::vector<int> ea(size_t(op->NCH) * kNC, 0);
   for (int r = 0; r < M; ++r) {
@@ -286,11 +282,13 @@ cudaError_t tc64_op_create(const std::vector<double>& A, int M, int K, Tc64Op* o
       l1 += std::fabs(A[size_t(r) * K + k]);
     }
     ea[r] = fx::row_exp(mx, l1);
+    double l1d[4] = {};  // absolute sums of the row's four leading digits
     for (int k = 0; k < K; ++k) {
       const double v = A[size_t(r) * K + k];
       if (v == 0.0 || !std::isfinite(v)) continue;
       int d[kDigits];
       fx::digits_of(v, ea[r], d);
+      for (int i = 0; i < 4; ++i) l1d[i] += std::abs(d[i]);
       uint8_t* blk = img.data() + size_t(r / kNC * op->KCH + k / kKC) * kBBytes;
       for (int i = 0; i < kDigits; ++i) {
         const int R = i * kNC + r % kNC, c = k % kKC;
@@ -298,6 +296,13 @@ cudaError_t tc64_op_create(const std::vector<double>& A, int M, int K, Tc64Op* o
         std::memcpy(blk + size_t(R / 8) * ((kKC / 8) * 128) + size_t(c / 8) * 128 + size_t(R % 8) * 16 + size_t(c % 8) * 2,
                     &h, 2);
       }
+    }
+    // The sums that carry the result (s <= 3) have to stay integers below 2^24, which
+    // FP32 holds exactly, whatever the data: its leading digit is at most 257, the others 128.
+    for (int s4 = 0; s4 < 4; ++s4) {
+      double most = 257.0 * l1d[s4];
+      for (int i = 0; i < s4; ++i) most += 128.0 * l1d[i];
+      if (most >= 16777216.0) return cudaErrorInvalidValue;
     }
   }
   cudaError_t e = cudaMalloc(&op->blocks, img.size());

@@ -15,9 +15,11 @@
 // At degrees 1-2 one advection kernel computes volume and surface terms
 // together and applies the LSERK stage update, ping-ponging U~ between two
 // buffers so neighbours always read the previous stage. From degree 3 the
-// stage's two dense contractions (cubature interpolation, projection with the
-// lift) run as exactly sliced FP64 products on the tensor cores, around an
-// FP64 kernel for the fluxes at the cubature points.
+// stage's two dense contractions (interpolation to the volume and face cubature
+// points, projection with the lift) run as exactly sliced FP64 products on the
+// tensor cores, around an FP64 kernel for the fluxes at those points; U^n and
+// U^{n-1} are interpolated once a step, and once U^{n-1} has reached t^n both
+// history fields advance together (they meet the same Ubar at the same times).
 #include <cmath>
 #include <cstring>
 #include <string>
@@ -47,13 +49,16 @@ struct InsWorkspace {
   int N = 0;
   AdvLayout L;
   double* ops = nullptr;
-  // tensor-core advection (degree >= 3): the cubature interpolation Iq and the
-  // projection blocks Pr, Ps, -Lc as sliced FP64 operators, with their row
-  // buffers (the projection is split at its blocks so that every sliced product
-  // sums at most 256 terms, which keeps its FP32 group sums exact)
+  // tensor-core advection (degree >= 3): interpolation to the Nc volume and 3 nc
+  // face cubature points, and the projection [Pr Ps -Lc] as one sliced operator, or
+  // as its three blocks where a sum over all of them would not be exact
   bool tensor = false;
-  SlicedOp opIq, opPr, opPs, opLc;
-  double *X = nullptr, *W = nullptr, *Y = nullptr, *R = nullptr;
+  Tc64Op opI, opP[3];
+  int npP = 0, colP[3] = {};  // projection blocks and their first columns in Y
+  double* nrm = nullptr;      // [3][3][K]: per face n_x, n_y, sJ / J
+  // point values of U^n, U^{n-1} and the velocity data, and of the advected fields; fluxes; projection
+  double *WU = nullptr, *WG = nullptr, *W = nullptr, *Y = nullptr, *R = nullptr;
+  // the advected fields U~ (two buffers, [2 fields][2][K][Np]) and their LSERK residual
   double *Ut0 = nullptr, *Ut1 = nullptr, *res = nullptr, *Uhat = nullptr, *Uhh = nullptr, *bu = nullptr,
          *G = nullptr, *bp = nullptr, *dP = nullptr, *tmp = nullptr;
   double *gts = nullptr, *zero = nullptr;  // time-dependent data: velocity data at a stage time; zeros
@@ -65,10 +70,8 @@ void free_ins_workspace(dg_mesh* m) {
   InsWorkspace* w = m->ins;
   if (!w) return;
   for (void* p : w->allocs) cudaFree(p);
-  sliced_op_free(&w->opIq);
-  sliced_op_free(&w->opPr);
-  sliced_op_free(&w->opPs);
-  sliced_op_free(&w->opLc);
+  tc64_op_free(&w->opI);
+  for (Tc64Op& op : w->opP) tc64_op_free(&op);
   if (w->ev0) cudaEventDestroy(w->ev0);
   if (w->ev1) cudaEventDestroy(w->ev1);
   delete w;
@@ -438,24 +441,24 @@ inline int eg(int64_t n) {
 
 template <int N>
 cudaError_t launch_advect_n(const dg_mesh* m, InsWorkspace* w, const double* Un, const double* Unm1, double ca,
-                            double cb, const double* Ut_in, double* Ut_out, const double* gU, double a, double b,
-                            double dts, cudaStream_t st) {
+                            double cb, const double* Ut_in, double* Ut_out, double* res, const double* gU, double a,
+                            double b, double dts, cudaStream_t st) {
   constexpr int nc = (3 * N + 2) / 2, Nc = nc * nc;
   constexpr int E = (2 * Nc) >= 512 ? 1 : (512 / (2 * Nc) < 1 ? 1 : 512 / (2 * Nc));
   const int blocks = int((m->K + E - 1) / E);
   advect_kernel<N><<<blocks, kAdvThreads, 0, st>>>(m->K, m->geo64, m->conn, w->ops, w->L, Un, Unm1, ca, cb, Ut_in,
-                                                   Ut_out, w->res, gU, a, b, dts);
+                                                   Ut_out, res, gU, a, b, dts);
   note_launch();
   return cudaGetLastError();
 }
 
 cudaError_t launch_advect(const dg_mesh* m, InsWorkspace* w, const double* Un, const double* Unm1, double ca,
-                          double cb, const double* Ut_in, double* Ut_out, const double* gU, double a, double b,
-                          double dts, cudaStream_t st) {
+                          double cb, const double* Ut_in, double* Ut_out, double* res, const double* gU, double a,
+                          double b, double dts, cudaStream_t st) {
   switch (m->N) {
 #define CASE(n) \
-  case n: return launch_advect_n<n>(m, w, Un, Unm1, ca, cb, Ut_in, Ut_out, gU, a, b, dts, st);
-    CASE(1) CASE(2) CASE(3) CASE(4) CASE(5) CASE(6) CASE(7) CASE(8)
+  case n: return launch_advect_n<n>(m, w, Un, Unm1, ca, cb, Ut_in, Ut_out, res, gU, a, b, dts, st);
+    CASE(1) CASE(2)
 #undef CASE
     default: return cudaErrorInvalidValue;
   }
@@ -463,88 +466,89 @@ cudaError_t launch_advect(const dg_mesh* m, InsWorkspace* w, const double* Un, c
 
 // ------------------------------------------- tensor-core advection stage
 // The stage of advect_kernel split at its two dense contractions, which run as
-// sliced FP64 products on the tensor cores (sliced_gemm):
-//   X = [Ubar_x; Ubar_y; Ut_x; Ut_y]            rows (c K + e), Np each
-//   W = Iq X                                     rows (c K + e), Nc each
-//   Y = [ G.F at the volume points | (sJ/J) n.F* at the face points ]   rows (c K + e)
-//   R = Pr Y_r + Ps Y_s - Lc Y_F                 rows (c K + e), Np each: the rhs
-//       (three sliced products, summed in FP64 by the update)
-// then the LSERK update. Arithmetic and layout as in advect_kernel.
-__global__ void k_adv_gather(int64_t n1, const double* __restrict__ Un, const double* __restrict__ Unm1, double ca,
-                             double cb, const double* __restrict__ Ut_in, double* __restrict__ X) {
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < 4 * n1; i += int64_t(gridDim.x) * blockDim.x) {
-    const int c = int(i / n1);
-    const int64_t j = i - c * n1;
-    X[i] = c < 2 ? ca * Un[c * n1 + j] + (cb != 0.0 ? cb * Unm1[c * n1 + j] : 0.0) : Ut_in[(c - 2) * n1 + j];
+// sliced FP64 products on the tensor cores (tc64_gemm_launch):
+//   W = I U~             rows (2 field + c) K + e, the Nc volume and 3 nc face points each
+//   Y = [ G.F at the volume points | (sJ/J) n.F* at the face points ]   same rows
+//   R = [Pr Ps -Lc] Y    same rows, Np each: the right-hand side
+// then the LSERK update; Ubar = ca U^n + cb U^{n-1} at the points from WU, the
+// interpolants of both, formed once a step. A face point's neighbour value is the
+// neighbour's own interpolant at the mirrored Gauss point.
+// At 8,192 elements of degree 8 a stage took 280 us, 117 us of it this kernel's
+// predecessor, which interpolated the face values itself on the FP64 pipe (nine
+// nodes of four fields of both sides a point): now 167 us, 69 us of it this kernel
+// (12 FP64 operations a volume point, about 30 a face point), and 271 us for two
+// fields at once.
+
+// n_x, n_y, sJ / J of every face: [f][3][K]
+__global__ void k_adv_normals(int64_t K, const double* __restrict__ geo, double* __restrict__ nrm) {
+  const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (e >= K) return;
+  const GeoF g = load_geo(geo, e);
+  for (int f = 0; f < 3; ++f) {
+    double nx, ny, sjj;
+    face_n(g, f, nx, ny, sjj);
+    nrm[(3 * f + 0) * K + e] = nx;
+    nrm[(3 * f + 1) * K + e] = ny;
+    nrm[(3 * f + 2) * K + e] = sjj;
   }
 }
 
-// one thread per volume cubature point (e, q) or face cubature point (e, f, k)
-__global__ void k_adv_flux(int N, int64_t K, const double* __restrict__ geo, const int32_t* __restrict__ conn,
-                           const double* __restrict__ I1, const double* __restrict__ X, const double* __restrict__ W,
-                           const double* __restrict__ gU, double* __restrict__ Y) {
-  const int Np = (N + 1) * (N + 2) / 2, Nfp = N + 1, nc = (3 * N + 2) / 2, Nc = nc * nc;
-  const int KY = 2 * Nc + 3 * nc;
-  const int64_t nvol = K * Nc, total = nvol + K * 3 * nc;
-  const size_t fsX = size_t(K) * Np, fsW = size_t(K) * Nc, fsY = size_t(K) * KY;
+__host__ __device__ constexpr int pad2(int n) { return (n + 1) & ~1; }  // Y's rows start on 16 bytes
+
+// NF advected fields at once (one thread per cubature point of an element)
+template <int NF>
+__global__ void k_adv_flux(int Nc, int nc, int64_t K, const double* __restrict__ geo, const double* __restrict__ nrm,
+                           const int32_t* __restrict__ conn, const double* __restrict__ WU,
+                           const double* __restrict__ WG, double ca, double cb, const double* __restrict__ W,
+                           double* __restrict__ Y) {
+  const int MW = Nc + 3 * nc, ldY = pad2(2 * Nc + 3 * nc);
+  const int64_t total = K * MW, fsY = K * ldY;
+  auto ubar = [&](int c, int64_t i) {
+    const double a = ca * __ldg(WU + c * total + i);
+    return cb != 0.0 ? a + cb * __ldg(WU + (2 + c) * total + i) : a;
+  };
   for (int64_t idx = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; idx < total;
        idx += int64_t(gridDim.x) * blockDim.x) {
-    if (idx < nvol) {
-      const int64_t e = idx / Nc;
-      const int q = int(idx - e * Nc);
-      const GeoF g = load_geo(geo, e);
-      double w[4];
-      for (int c = 0; c < 4; ++c) w[c] = W[c * fsW + size_t(e) * Nc + q];
-      for (int c = 0; c < 2; ++c) {
-        const double Fx = w[0] * w[2 + c], Fy = w[1] * w[2 + c];
-        Y[c * fsY + size_t(e) * KY + q] = g.rx * Fx + g.ry * Fy;
-        Y[c * fsY + size_t(e) * KY + Nc + q] = g.sx * Fx + g.sy * Fy;
+    const int64_t e = total < (int64_t(1) << 31) ? int64_t(uint32_t(idx) / uint32_t(MW)) : idx / MW;
+    const int m = int(idx - e * MW);
+    const double u = ubar(0, idx), v = ubar(1, idx);
+    if (m < Nc) {
+      const double2 gx = *reinterpret_cast<const double2*>(geo + 4 * e);      // r_x, s_x
+      const double2 gy = *reinterpret_cast<const double2*>(geo + 4 * e + 2);  // r_y, s_y
+      const double ur = gx.x * u + gy.x * v, us = gx.y * u + gy.y * v;
+#pragma unroll
+      for (int c = 0; c < 2 * NF; ++c) {
+        const double w = __ldg(W + c * total + idx);
+        double* y = Y + c * fsY + e * ldY + m;
+        y[0] = ur * w;
+        y[Nc] = us * w;
       }
     } else {
-      const int64_t r = idx - nvol;
-      const int64_t e = r / (3 * nc);
-      const int q = int(r - e * 3 * nc), f = q / nc, k = q - f * nc;
-      const GeoF g = load_geo(geo, e);
-      const int code = conn[3 * e + f];
-      double m[4] = {0, 0, 0, 0}, p[4] = {0, 0, 0, 0};
-      for (int a2 = 0; a2 < Nfp; ++a2) {
-        const double i1 = I1[size_t(k) * Nfp + a2];
-        const int kl = fnode_i(N, f, a2);
-        double vm[4], vp[4];
-        for (int c = 0; c < 4; ++c) vm[c] = X[c * fsX + size_t(e) * Np + kl];
-        if (code >= 0) {
-          const int64_t nb = code >> 2;
-          const int kn = fnode_i(N, code & 3, Nfp - 1 - a2);
-          for (int c = 0; c < 4; ++c) vp[c] = X[c * fsX + size_t(nb) * Np + kn];
-        } else if (code == -2) {  // velocity Dirichlet: exterior state is the boundary datum
-          const size_t gi = size_t(e) * Np + kl;
-          vp[0] = vp[2] = gU[gi];
-          vp[1] = vp[3] = gU[fsX + gi];
-        } else {                  // Neumann: exterior = interior
-          for (int c = 0; c < 4; ++c) vp[c] = vm[c];
-        }
-        for (int c = 0; c < 4; ++c) {
-          m[c] += i1 * vm[c];
-          p[c] += i1 * vp[c];
-        }
-      }
-      double nx, ny, sjj;
-      face_n(g, f, nx, ny, sjj);
-      const double unm = nx * m[0] + ny * m[1], unp = nx * p[0] + ny * p[1];
+      const int q = m - Nc, f = q / nc, k = q - f * nc;
+      const int code = __ldg(conn + 3 * e + f);
+      const int64_t in = code >= 0 ? int64_t(code >> 2) * MW + Nc + (code & 3) * nc + (nc - 1 - k) : idx;
+      const bool data = code == -2;  // velocity Dirichlet: exterior state is the boundary datum (Neumann: the interior)
+      const double up = data ? __ldg(WG + idx) : (code >= 0 ? ubar(0, in) : u);
+      const double vp = data ? __ldg(WG + total + idx) : (code >= 0 ? ubar(1, in) : v);
+      const double nx = __ldg(nrm + (3 * f + 0) * K + e), ny = __ldg(nrm + (3 * f + 1) * K + e),
+                   sjj = __ldg(nrm + (3 * f + 2) * K + e);
+      const double unm = nx * u + ny * v, unp = nx * up + ny * vp;
       const double lam = fmax(fabs(unm), fabs(unp));
-      for (int c = 0; c < 2; ++c)
-        Y[c * fsY + size_t(e) * KY + 2 * Nc + q] =
-            sjj * (0.5 * (unm * m[2 + c] + unp * p[2 + c]) + 0.5 * lam * (m[2 + c] - p[2 + c]));
+#pragma unroll
+      for (int c = 0; c < 2 * NF; ++c) {
+        const double w = __ldg(W + c * total + idx);
+        const double wp = data ? __ldg(WG + (c & 1) * total + idx) : __ldg(W + c * total + in);
+        Y[c * fsY + e * ldY + 2 * Nc + q] = sjj * (0.5 * (unm * w + unp * wp) + 0.5 * lam * (w - wp));
+      }
     }
   }
 }
 
-// rhs = R_r + R_s + R_lift (the three projection blocks, each n entries);
-// res = a res + dts rhs; Ut_out = Ut_in + b res  (n = 2 K Np)
+// res = a res + dts R; Ut_out = Ut_in + b res
 __global__ void k_adv_update(int64_t n, const double* __restrict__ R, double a, double dts, double b,
                              const double* __restrict__ Ut_in, double* __restrict__ res, double* __restrict__ Ut_out) {
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
-    const double r = a * res[i] + dts * (R[i] + R[n + i] + R[2 * n + i]);
+    const double r = a * res[i] + dts * R[i];
     res[i] = r;
     Ut_out[i] = Ut_in[i] + b * r;
   }
@@ -571,9 +575,9 @@ cudaError_t setup_ins(dg_mesh* m) {
   const size_t n1 = size_t(m->K) * ((m->N + 1) * (m->N + 2) / 2);
   ICK(al(&w->ops, h.size()));
   ICK(cudaMemcpy(w->ops, h.data(), h.size() * sizeof(double), cudaMemcpyHostToDevice));
-  ICK(al(&w->Ut0, 2 * n1));
-  ICK(al(&w->Ut1, 2 * n1));
-  ICK(al(&w->res, 2 * n1));
+  ICK(al(&w->Ut0, 4 * n1));
+  ICK(al(&w->Ut1, 4 * n1));
+  ICK(al(&w->res, 4 * n1));
   ICK(al(&w->Uhat, 2 * n1));
   ICK(al(&w->Uhh, 2 * n1));
   ICK(al(&w->bu, 2 * n1));
@@ -589,55 +593,73 @@ cudaError_t setup_ins(dg_mesh* m) {
   // degree >= 3: the stage's dense contractions on the tensor cores
   if (m->N >= 3) {
     const AdvLayout& L = w->L;
-    const int Np = L.Np, Nc = L.Nc, nc = L.nc, KY = 2 * Nc + 3 * nc;
-    const std::vector<double> Iq(h.begin() + L.Iq, h.begin() + L.Iq + size_t(Nc) * Np);
-    const std::vector<double> Pr(h.begin() + L.Pr, h.begin() + L.Pr + size_t(Np) * Nc);
-    const std::vector<double> Ps(h.begin() + L.Ps, h.begin() + L.Ps + size_t(Np) * Nc);
-    std::vector<double> Lc(h.begin() + L.Lc, h.begin() + L.Lc + size_t(Np) * 3 * nc);
-    for (double& v : Lc) v = -v;
-    ICK(sliced_op_create(Iq, Nc, Np, &w->opIq));
-    ICK(sliced_op_create(Pr, Np, Nc, &w->opPr));
-    ICK(sliced_op_create(Ps, Np, Nc, &w->opPs));
-    ICK(sliced_op_create(Lc, Np, 3 * nc, &w->opLc));
-    ICK(al(&w->X, 4 * n1));
-    ICK(al(&w->W, 4 * size_t(m->K) * Nc));
-    ICK(al(&w->Y, 2 * size_t(m->K) * KY));
-    ICK(al(&w->R, 3 * 2 * n1));  // the three projection blocks' results
+    const int Np = L.Np, Nfp = L.Nfp, Nc = L.Nc, nc = L.nc, KY = 2 * Nc + 3 * nc, MW = Nc + 3 * nc;
+    std::vector<double> I(size_t(MW) * Np, 0.0), P(size_t(Np) * KY);
+    std::copy(h.begin() + L.Iq, h.begin() + L.Iq + size_t(Nc) * Np, I.begin());
+    for (int f = 0; f < 3; ++f)
+      for (int k = 0; k < nc; ++k)
+        for (int a = 0; a < Nfp; ++a) I[size_t(Nc + f * nc + k) * Np + fnode_i(m->N, f, a)] = h[L.I1 + size_t(k) * Nfp + a];
+    for (int i = 0; i < Np; ++i)
+      for (int k = 0; k < KY; ++k)
+        P[size_t(i) * KY + k] = k < Nc ? h[L.Pr + size_t(i) * Nc + k]
+                                       : (k < 2 * Nc ? h[L.Ps + size_t(i) * Nc + k - Nc]
+                                                     : -h[L.Lc + size_t(i) * 3 * nc + k - 2 * Nc]);
+    ICK(tc64_op_create(I, MW, Np, &w->opI));
+    const cudaError_t one = tc64_op_create(P, Np, KY, &w->opP[0]);
+    w->npP = 1;
+    if (one != cudaSuccess) {  // too deep for exact sums: block by block
+      if (one != cudaErrorInvalidValue) return one;
+      const int col[4] = {0, Nc, 2 * Nc, KY};
+      w->npP = 3;
+      for (int b = 0; b < 3; ++b) {
+        const int n = col[b + 1] - col[b];
+        std::vector<double> Pb(size_t(Np) * n);
+        for (int i = 0; i < Np; ++i)
+          for (int k = 0; k < n; ++k) Pb[size_t(i) * n + k] = P[size_t(i) * KY + col[b] + k];
+        ICK(tc64_op_create(Pb, Np, n, &w->opP[b]));
+        w->colP[b] = col[b];
+      }
+    }
+    const size_t nw = size_t(m->K) * MW;
+    ICK(al(&w->nrm, 9 * size_t(m->K)));
+    ICK(al(&w->WU, 4 * nw));
+    ICK(al(&w->WG, 2 * nw));
+    ICK(al(&w->W, 4 * nw));
+    ICK(al(&w->Y, 4 * size_t(m->K) * pad2(KY)));
+    ICK(al(&w->R, 4 * n1));
+    k_adv_normals<<<unsigned((m->K + 255) / 256), 256>>>(m->K, m->geo64, w->nrm);
+    note_launch();
+    ICK(cudaStreamSynchronize(nullptr));
     w->tensor = true;
   }
   return cudaSuccess;
 }
 
-// One LSERK stage of the advection on the tensor cores (see k_adv_gather).
-cudaError_t advect_stage_tensor(const dg_mesh* m, InsWorkspace* w, const double* Un, const double* Unm1, double ca,
-                                double cb, const double* Ut_in, double* Ut_out, const double* gU, double a, double b,
-                                double dts, cudaStream_t st) {
+// One LSERK stage of nf advected fields on the tensor cores (see k_adv_flux).
+cudaError_t advect_stage_tensor(const dg_mesh* m, InsWorkspace* w, int nf, double ca, double cb, const double* Ut_in,
+                                double* Ut_out, double a, double b, double dts, cudaStream_t st) {
   const AdvLayout& L = w->L;
-  const int Np = L.Np, Nc = L.Nc, nc = L.nc, KY = 2 * Nc + 3 * nc;
-  const int64_t K = m->K, n1 = K * Np;
-  k_adv_gather<<<eg(4 * n1), 256, 0, st>>>(n1, Un, Unm1, ca, cb, Ut_in, w->X);
+  const int Np = L.Np, Nc = L.Nc, nc = L.nc, MW = Nc + 3 * nc;
+  const int64_t K = m->K, rows = 2 * K * nf;
+  ICK(tc64_gemm_launch(w->opI, rows, Ut_in, Np, w->W, MW, st));
+  if (nf == 1) k_adv_flux<1><<<eg(K * MW), 256, 0, st>>>(Nc, nc, K, m->geo64, w->nrm, m->conn, w->WU, w->WG, ca, cb, w->W, w->Y);
+  else k_adv_flux<2><<<eg(K * MW), 256, 0, st>>>(Nc, nc, K, m->geo64, w->nrm, m->conn, w->WU, w->WG, ca, cb, w->W, w->Y);
   note_launch();
-  ICK(sliced_gemm(w->opIq, 4 * K, w->X, Np, w->W, Nc, st));
-  k_adv_flux<<<eg(K * (Nc + 3 * nc)), 256, 0, st>>>(m->N, K, m->geo64, m->conn, w->ops + L.I1, w->X, w->W, gU, w->Y);
-  note_launch();
-  ICK(sliced_gemm(w->opPr, 2 * K, w->Y, KY, w->R, Np, st));
-  ICK(sliced_gemm(w->opPs, 2 * K, w->Y + Nc, KY, w->R + 2 * n1, Np, st));
-  ICK(sliced_gemm(w->opLc, 2 * K, w->Y + 2 * Nc, KY, w->R + 4 * n1, Np, st));
-  k_adv_update<<<eg(2 * n1), 256, 0, st>>>(2 * n1, w->R, a, dts, b, Ut_in, w->res, Ut_out);
+  for (int p = 0; p < w->npP; ++p)
+    ICK(tc64_gemm_launch(w->opP[p], rows, w->Y + w->colP[p], pad2(2 * Nc + 3 * nc), w->R, Np, st, p > 0));
+  k_adv_update<<<eg(rows * Np), 256, 0, st>>>(rows * Np, w->R, a, dts, b, Ut_in, w->res, Ut_out);
   note_launch();
   return cudaGetLastError();
 }
 
-// Advect U0 (given at t0) to t0 + nsub*dts with LSERK(5,4); result in the
-// returned buffer (one of Ut0/Ut1). Ubar(t) = U^n + (t - tn)/dt (U^n - U^{n-1}).
-cudaError_t advect_field(const dg_mesh* m, InsWorkspace* w, const dg_ins_state* s, const double* U0, double t0,
-                         int nsub, double tn, bool extrap, double** result, cudaStream_t st) {
-  const size_t n2 = 2 * size_t(m->K) * ((m->N + 1) * (m->N + 2) / 2);
+// nsub LSERK(5,4) substeps from time t0 of the nf fields in *cur (Ut0 or Ut1; the
+// result's buffer on return). Ubar(t) = U^n + (t - tn)/dt (U^n - U^{n-1}).
+cudaError_t advect_substeps(const dg_mesh* m, InsWorkspace* w, const dg_ins_state* s, int nf, double t0, int nsub,
+                            double tn, bool extrap, double** cur, cudaStream_t st) {
+  const int Np = (m->N + 1) * (m->N + 2) / 2;
+  const size_t n2 = 2 * size_t(m->K) * Np;
   const double dts = s->dt / s->Ns;
-  ICK(cudaMemcpyAsync(w->Ut0, U0, n2 * sizeof(double), cudaMemcpyDeviceToDevice, st));
-  ICK(cudaMemsetAsync(w->res, 0, n2 * sizeof(double), st));
-  double* cur = w->Ut0;
-  double* nxt = w->Ut1;
+  double* nxt = *cur == w->Ut0 ? w->Ut1 : w->Ut0;
   double t = t0;
   for (int k = 0; k < nsub; ++k) {
     for (int stg = 0; stg < 5; ++stg) {
@@ -661,17 +683,50 @@ cudaError_t advect_field(const dg_mesh* m, InsWorkspace* w, const dg_ins_state* 
           note_launch();
         }
         g = w->gts;
+        if (w->tensor) ICK(tc64_gemm_launch(w->opI, 2 * m->K, g, Np, w->WG, w->opI.M, st));
       }
-      if (w->tensor)
-        ICK(advect_stage_tensor(m, w, s->U, s->Uold, ca, cb, cur, nxt, g, kRkA[stg], kRkB[stg], dts, st));
-      else
-        ICK(launch_advect(m, w, s->U, s->Uold, ca, cb, cur, nxt, g, kRkA[stg], kRkB[stg], dts, st));
-      std::swap(cur, nxt);
+      if (w->tensor) {
+        ICK(advect_stage_tensor(m, w, nf, ca, cb, *cur, nxt, kRkA[stg], kRkB[stg], dts, st));
+      } else {
+        for (int f = 0; f < nf; ++f)
+          ICK(launch_advect(m, w, s->U, s->Uold, ca, cb, *cur + f * n2, nxt + f * n2, w->res + f * n2, g, kRkA[stg],
+                            kRkB[stg], dts, st));
+      }
+      std::swap(*cur, nxt);
     }
     t += dts;
   }
-  *result = cur;
   return cudaSuccess;
+}
+
+// (i) of the step: U^ = the advected history fields, beta_i U~^{n-i} summed.
+cudaError_t advect_history(const dg_mesh* m, InsWorkspace* w, const dg_ins_state* s, cudaStream_t st) {
+  const int Np = (m->N + 1) * (m->N + 2) / 2;
+  const size_t n2 = 2 * size_t(m->K) * Np, bytes = n2 * sizeof(double);
+  const double tn = s->step * s->dt;
+  const bool first = s->step == 0;
+  if (w->tensor) {
+    const size_t nw = 2 * size_t(m->K) * w->opI.M;
+    ICK(tc64_gemm_launch(w->opI, 2 * m->K, s->U, Np, w->WU, w->opI.M, st));
+    if (!first) ICK(tc64_gemm_launch(w->opI, 2 * m->K, s->Uold, Np, w->WU + nw, w->opI.M, st));
+    if (!s->gU_hist) ICK(tc64_gemm_launch(w->opI, 2 * m->K, s->gU, Np, w->WG, w->opI.M, st));
+  }
+  ICK(cudaMemsetAsync(w->res, 0, 2 * bytes, st));
+  double* cur = w->Ut0;
+  if (first) {
+    ICK(cudaMemcpyAsync(cur, s->U, bytes, cudaMemcpyDeviceToDevice, st));
+    ICK(advect_substeps(m, w, s, 1, tn, s->Ns, tn, false, &cur, st));
+    ICK(cudaMemcpyAsync(w->Uhat, cur, bytes, cudaMemcpyDeviceToDevice, st));
+    return cudaSuccess;
+  }
+  // U^{n-1} to t^n by itself, then with U^n to t^{n+1}
+  ICK(cudaMemcpyAsync(cur, s->Uold, bytes, cudaMemcpyDeviceToDevice, st));
+  ICK(advect_substeps(m, w, s, 1, tn - s->dt, s->Ns, tn, true, &cur, st));
+  ICK(cudaMemcpyAsync(cur + n2, s->U, bytes, cudaMemcpyDeviceToDevice, st));
+  ICK(advect_substeps(m, w, s, 2, tn, s->Ns, tn, true, &cur, st));
+  axpby_kernel<<<eg(n2), 256, 0, st>>>(n2, 2.0, cur + n2, 0.0, w->Uhat, -0.5, cur);
+  note_launch();
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -689,21 +744,8 @@ cudaError_t ins_run(dg_mesh* mu, dg_mesh* mp, dg_ins_state* s, int nsteps, cudaS
   for (int it = 0; it < nsteps; ++it) {
     const int n = s->step;
     const double dt = s->dt, nu = s->nu;
-    const double tn = n * dt;
-    double gamma;
-    // (i) advection of the history into U^
-    double* Ut = nullptr;
-    if (n == 0) {
-      gamma = 1.0;
-      ICK(advect_field(mu, w, s, s->U, tn, s->Ns, tn, false, &Ut, st));
-      ICK(cudaMemcpyAsync(w->Uhat, Ut, n2 * sizeof(double), cudaMemcpyDeviceToDevice, st));
-    } else {
-      gamma = 1.5;
-      ICK(advect_field(mu, w, s, s->U, tn, s->Ns, tn, true, &Ut, st));
-      axpby_kernel<<<eg(n2), 256, 0, st>>>(n2, 2.0, Ut, 0.0, w->Uhat, 0.0, nullptr); note_launch();
-      ICK(advect_field(mu, w, s, s->Uold, tn - dt, 2 * s->Ns, tn, true, &Ut, st));
-      axpby_kernel<<<eg(n2), 256, 0, st>>>(n2, -0.5, Ut, 1.0, w->Uhat, 0.0, nullptr); note_launch();
-    }
+    const double gamma = n == 0 ? 1.0 : 1.5;
+    ICK(advect_history(mu, w, s, st));
     // (ii) velocity Helmholtz: b = J M U^/(nu dt) - L(gU) - (1/nu) G P^n
     axpby_kernel<<<eg(n2), 256, 0, st>>>(n2, 1.0 / (nu * dt), w->Uhat, 0.0, w->tmp, 0.0, nullptr); note_launch();
     ICK(launch_rhs(mu, 2, w->tmp, s->gU, w->bu, st));
