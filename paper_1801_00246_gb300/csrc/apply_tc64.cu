@@ -62,20 +62,12 @@ constexpr int kCoefs = 12;    // Grr, Grs, Gss | per face nr sJ, ns sJ | per fac
 
 __device__ int g_t64_err;
 
-__device__ __forceinline__ void mbar_arrive(uint64_t* b) {
-  asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.shared::cta.b64 st, [%0];\n}\n" ::"r"(tc::smem_addr(b)) : "memory");
-}
-// A wait that gave up sets the block's abort flag, and every later wait then
-// returns at once: all warps run to the end of their loops (their named
-// barriers stay matched) and the block ends.
-__device__ __forceinline__ bool aborted(volatile int* flag) { return __any_sync(0xffffffffu, *flag != 0); }
+using tc::aborted;
+using tc::bar_sync;
+using tc::mbar_arrive;
 __device__ __forceinline__ void wait(uint64_t* b, uint32_t parity, volatile int* abort_flag) {
-  if (!aborted(abort_flag) && !tc::mbar_wait(b, parity)) *abort_flag = 1;
+  tc::wait_or_abort(b, parity, abort_flag);
 }
-__device__ __forceinline__ void bar_sync(int id, int threads) {
-  asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(threads) : "memory");
-}
-
 __device__ __forceinline__ int64_t elem_of(int64_t row, int64_t K) { return row < K ? row : row % K; }
 
 __device__ __forceinline__ int node_of(int N, int f, int j) {  // local node of face f's j-th node

@@ -195,9 +195,9 @@ cudaError_t tc64_gemm_error(int* flag);              // the generic product's pa
 cudaError_t build_fixed_geometry(dg_mesh* m);         // gfix, gfix_ex (dg_mesh_setup)
 // FP64 products on the tcgen05 tensor cores with exact integer slicing (gemm_tc64.cu):
 // an operator A (M x K, sums short enough to stay exact) cut into 7 digits in blocks of
-// 48 rows x 32 columns
+// 32 or 48 rows x 32 columns
 struct Tc64Op {
-  int M = 0, K = 0, NCH = 0, KCH = 0;
+  int M = 0, K = 0, nc = 0, NCH = 0, KCH = 0;  // nc: output columns per pass
   uint8_t* blocks = nullptr;
   int* ea = nullptr;
 };

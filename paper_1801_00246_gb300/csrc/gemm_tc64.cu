@@ -26,46 +26,57 @@ using fx::kSums;
 
 constexpr int kT = 128;                      // rows per tile (MMA M)
 constexpr int kKC = 32;                      // data columns per chunk
-constexpr int kNC = 48;                      // output columns per pass (MMA N)
-constexpr int kASlice = kT * kKC * 2, kABytes = kDigits * kASlice;   // one data chunk, 7 digits: 56 KB
-constexpr int kBSlice = kNC * kKC * 2, kBBytes = kDigits * kBSlice;  // one operator block, 7 digits: 21 KB
-constexpr int kSmem = 2 * kABytes + 2 * kBBytes + 4 * kT * 4 + 12 * 8;  // the tail: 10 mbarriers, slot, 2 flags
+constexpr int kASlice = kT * kKC * 2, kABytes = kDigits * kASlice;  // one data chunk, 7 digits: 56 KB
+constexpr int kStages = 4;                   // operator blocks in flight
+__host__ __device__ constexpr int block_bytes(int nc) { return kDigits * nc * kKC * 2; }
+// the tail: row exponents, 20 mbarriers, slot, flag
+__host__ __device__ constexpr int gemm_smem(int nc) {
+  return 2 * kABytes + kStages * block_bytes(nc) + 4 * kT * 4 + 20 * 8 + 16;
+}
+// Output columns per pass (MMA N): 32, with two accumulator sets in tensor memory so
+// that a pass's products run under the drain of the one before, where all of a row's
+// data stays in shared memory for its passes (two chunks) or one pass is enough;
+// else 48 in one set, so that a deep row is sliced once (more than 48 columns of
+// output: once per pass).
+int pass_columns(int M, int K) { return K <= 2 * kKC || M <= 32 ? 32 : 48; }
 
 __device__ int g_tc64_err;
 
 // out[r][c] = sum_k A[c][k] X[r][k] for r < rows, c < M, k < Kd (A sliced in
-// blocks of kNC rows x kKC columns: block (nc, kc) at (nc KCH + kc) kBBytes).
+// blocks of NC rows x kKC columns: block (nc, kc) at (nc KCH + kc) block_bytes).
 //
 // Warp-specialised pipeline over a stream of data chunks (tile, output pass
 // nc, column chunk kc), chunk g using shared-memory buffer g & 1:
 //  * warps 0-15 (four threads per row of the 128-row tile) find each row's
 //    scale exponent, slice chunk g into buffer g & 1 once the products of
 //    chunk g - 2 have released it (mbarrier `empty`), signal `full`, and after
-//    a pass's last chunk wait for its accumulators (`acc_full`), drain them
-//    (Horner's rule, epilogue) and release them (`acc_empty`);
-//  * warp 16 loads operator block g by bulk copy, waits for `full`, issues the
-//    36 slice products per 16 columns from one lane and commits to `empty`
-//    (and to `acc_full` after a pass's last chunk); before a pass's first
-//    chunk it waits until the previous pass has been drained.
+//    a pass's last chunk wait for its accumulators (`accf`), drain them and
+//    release them (`acce`);
+//  * warp 16 waits for `full`, issues the 34 digit products per 16 columns from
+//    one lane and commits to `empty` (and to `accf` after a pass's last chunk);
+//  * warp 17 keeps a ring of operator blocks filled by bulk copies (loaded by
+//    warp 16 only when a chunk needed them, their latency was in every chunk:
+//    16,384 rows of 208 outputs, 45 deep, took 44 us).
 // No CTA-wide barrier in the steady state; every wait is bounded in time.
 constexpr int kSlicers = 512;  // threads of warps 0-15
-__global__ void __launch_bounds__(kSlicers + 32, 1) tc64_gemm(int64_t rows, int M, int Kd, int NCH, int KCH,
+template <int NC>
+__global__ void __launch_bounds__(kSlicers + 64, 1) tc64_gemm(int64_t rows, int M, int Kd, int NCH, int KCH,
                                                               const double* __restrict__ X, int64_t ldx, int vec2,
                                                               const int* __restrict__ ex_given,
                                                               const uint8_t* __restrict__ Bops,
                                                               const int* __restrict__ ea, double* __restrict__ out,
                                                               int64_t ldo, int accum) {
   extern __shared__ __align__(1024) uint8_t sm[];
+  constexpr int kBBytes = block_bytes(NC);
+  constexpr int kAcc = 2 * kSums * NC <= 512 ? 2 : 1;  // accumulator sets
   uint8_t* sA = sm;                        // [2][7 digits][128 rows][32] canonical
-  uint8_t* sB = sm + 2 * kABytes;          // [2][7 digits x 48 rows][32] canonical
-  int* pmax = reinterpret_cast<int*>(sB + 2 * kBBytes);  // [4][kT]
-  // full[2], empty[2], bfull[2], acc_full, acc_empty, bempty[2]
+  uint8_t* sB = sm + 2 * kABytes;          // [kStages][7 digits x NC rows][32] canonical
+  int* pmax = reinterpret_cast<int*>(sB + kStages * kBBytes);  // [4][kT]
   uint64_t* bars = reinterpret_cast<uint64_t*>(pmax + 4 * kT);
-  uint64_t *full = bars, *empty = bars + 2, *bfull = bars + 4, *acc_full = bars + 6, *acc_empty = bars + 7,
-           *bempty = bars + 8;
-  uint32_t* slot = reinterpret_cast<uint32_t*>(bars + 10);
-  int* abort_flag = reinterpret_cast<int*>(slot + 1);
-  int* tile_abort = abort_flag + 1;  // the slicers' common copy of abort_flag at a tile's start
+  uint64_t *full = bars, *empty = bars + 2, *accf = bars + 4, *acce = bars + 6, *bfull = bars + 8,
+           *bempty = bars + 8 + kStages;
+  uint32_t* slot = reinterpret_cast<uint32_t*>(bars + 20);
+  volatile int* abort_flag = reinterpret_cast<int*>(slot + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int64_t ntiles = (rows + kT - 1) / kT;
   // with at most two data chunks per row, both stay in the two buffers for all
@@ -75,11 +86,13 @@ __global__ void __launch_bounds__(kSlicers + 32, 1) tc64_gemm(int64_t rows, int 
     for (int i = 0; i < 2; ++i) {
       tc::mbar_init(full + i, kSlicers / 32);  // one arrival per slicing warp
       tc::mbar_init(empty + i, 1);             // the products' commit
-      tc::mbar_init(bfull + i, 1);             // the bulk copy
+      tc::mbar_init(accf + i, 1);
+      tc::mbar_init(acce + i, kSlicers / 32);
     }
-    tc::mbar_init(acc_full, 1);
-    tc::mbar_init(acc_empty, kSlicers / 32);
-    for (int i = 0; i < 2; ++i) tc::mbar_init(bempty + i, 1);  // an operator stage's products completed
+    for (int i = 0; i < kStages; ++i) {
+      tc::mbar_init(bfull + i, 1);   // the bulk copy
+      tc::mbar_init(bempty + i, 1);  // the block's products completed
+    }
     *abort_flag = 0;
     tc::mbar_init_fence();
   }
@@ -89,40 +102,50 @@ __global__ void __launch_bounds__(kSlicers + 32, 1) tc64_gemm(int64_t rows, int 
   tc::fence_after();
   const uint32_t tb = *slot;
 
-  if (warp == kSlicers / 32) {
+  if (warp == kSlicers / 32 + 1) {
+    // ================= operator blocks
+    uint32_t g = 0;
+    for (int64_t tile = blockIdx.x; tile < ntiles && !tc::aborted(abort_flag); tile += gridDim.x)
+      for (int s = 0; s < NCH * KCH; ++s, ++g) {
+        const uint32_t b = g % kStages, use = g / kStages;
+        if (use > 0) tc::wait_or_abort(bempty + b, (use - 1) & 1u, abort_flag);
+        if (tc::aborted(abort_flag)) break;
+        if (lane == 0) {
+          tc::mbar_expect_tx(bfull + b, kBBytes);
+          tc::bulk_g2s(sB + b * kBBytes, Bops + size_t(s) * kBBytes, kBBytes, bfull + b);
+        }
+        __syncwarp();
+      }
+    // every copy has landed before the block ends
+    for (uint32_t k = g < kStages ? 0 : g - kStages; k < g; ++k)
+      tc::wait_or_abort(bfull + k % kStages, (k / kStages) & 1u, abort_flag);
+  } else if (warp == kSlicers / 32) {
     // ================= products
     uint32_t g = 0, pass = 0, it = 0;
     const uint64_t adesc0 = tc::smem_desc(tc::smem_addr(sA), 128, (kKC / 8) * 128);
     const uint64_t bdesc0 = tc::smem_desc(tc::smem_addr(sB), 128, (kKC / 8) * 128);
-    for (int64_t tile = blockIdx.x; tile < ntiles && !*abort_flag; tile += gridDim.x, ++it) {
+    for (int64_t tile = blockIdx.x; tile < ntiles && !tc::aborted(abort_flag); tile += gridDim.x, ++it) {
       for (int nc = 0; nc < NCH; ++nc, ++pass) {
-        // the accumulators are free once the previous pass has been drained
-        if (pass > 0 && !tc::mbar_wait(acc_empty, (pass - 1) & 1u)) *abort_flag = 1;
-        tc::fence_after();
+        // the accumulators are free once the pass that last used them has been drained
+        const uint32_t ab = pass % kAcc, ause = pass / kAcc;
+        if (ause > 0) tc::wait_or_abort(acce + ab, (ause - 1) & 1u, abort_flag);
         for (int kc = 0; kc < KCH; ++kc, ++g) {
-          const uint32_t bs = g & 1u;                 // operator stage
-          const uint32_t bd = resident ? kc : bs;     // data buffer
-          // the operator stage is free once chunk g - 2's products completed
-          if (g >= 2 && !tc::mbar_wait(bempty + bs, ((g - 2) >> 1) & 1u)) *abort_flag = 1;
-          if (lane == 0) {
-            tc::mbar_expect_tx(bfull + bs, kBBytes);
-            tc::bulk_g2s(sB + bs * kBBytes, Bops + size_t(nc * KCH + kc) * kBBytes, kBBytes, bfull + bs);
-          }
-          __syncwarp();
+          const uint32_t bs = g % kStages;                      // operator stage
+          const uint32_t bd = resident ? kc : (g & 1u);         // data buffer
           // the data chunk: sliced once per chunk, or (resident) once per tile for all passes
-          if (!resident && !tc::mbar_wait(full + bd, (g >> 1) & 1u)) *abort_flag = 1;
-          if (resident && nc == 0 && !tc::mbar_wait(full + bd, it & 1u)) *abort_flag = 1;
-          if (!tc::mbar_wait(bfull + bs, (g >> 1) & 1u)) *abort_flag = 1;
+          if (!resident) tc::wait_or_abort(full + bd, (g >> 1) & 1u, abort_flag);
+          else if (nc == 0) tc::wait_or_abort(full + bd, it & 1u, abort_flag);
+          tc::wait_or_abort(bfull + bs, (g / kStages) & 1u, abort_flag);
           tc::fence_after();
           if (lane == 0) {
-            const uint64_t ab = adesc0 + ((bd * kABytes) >> 4), bb = bdesc0 + ((bs * kBBytes) >> 4);
+            const uint64_t a0 = adesc0 + ((bd * kABytes) >> 4), b0 = bdesc0 + ((bs * kBBytes) >> 4);
 #pragma unroll
             for (int ks = 0; ks < kKC / 16; ++ks)
-              fx::issue_step<kKC * 2>(tb, ab + ((ks * 256) >> 4), kASlice, bb + ((ks * 256) >> 4), kNC,
+              fx::issue_step<kKC * 2>(tb + ab * kSums * NC, a0 + ((ks * 256) >> 4), kASlice, b0 + ((ks * 256) >> 4), NC,
                                       kc == 0 && ks == 0);
             tc::mma_commit(bempty + bs);
             if (!resident || nc == NCH - 1) tc::mma_commit(empty + bd);  // the data buffer is free
-            if (kc == KCH - 1) tc::mma_commit(acc_full);
+            if (kc == KCH - 1) tc::mma_commit(accf + ab);
           }
           __syncwarp();
         }
@@ -155,11 +178,6 @@ __global__ void __launch_bounds__(kSlicers + 32, 1) tc64_gemm(int64_t rows, int 
     int En = 0;
     double vn[8];  // the next chunk's values (loaded one chunk ahead)
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
-      // every slicer takes the same decision to stop (they meet at named barriers below)
-      asm volatile("bar.sync 1, %0;\n" ::"r"(kSlicers) : "memory");
-      if (tid == 0) *reinterpret_cast<volatile int*>(tile_abort) = *reinterpret_cast<volatile int*>(abort_flag);
-      asm volatile("bar.sync 1, %0;\n" ::"r"(kSlicers) : "memory");
-      if (*reinterpret_cast<volatile int*>(tile_abort)) break;
       const int64_t row = tile * kT + e;
       const bool live = row < rows;
       const double* xr = X + (live ? row : 0) * ldx;
@@ -180,9 +198,9 @@ __global__ void __launch_bounds__(kSlicers + 32, 1) tc64_gemm(int64_t rows, int 
             for (int t = 0; t < 8; ++t) em = max(em, max(fx::exp_bound(v[0][t]), fx::exp_bound(v[1][t])));
           }
         }
-        asm volatile("bar.sync 1, %0;\n" ::"r"(kSlicers) : "memory");  // pmax free (previous tile read it)
+        tc::bar_sync(1, kSlicers);  // pmax free (previous tile read it)
         pmax[q * kT + e] = em;
-        asm volatile("bar.sync 1, %0;\n" ::"r"(kSlicers) : "memory");
+        tc::bar_sync(1, kSlicers);
         E = max(max(pmax[e], pmax[kT + e]), max(pmax[2 * kT + e], pmax[3 * kT + e]));
         if (E == -1100) E = 0;
       }
@@ -212,40 +230,34 @@ __global__ void __launch_bounds__(kSlicers + 32, 1) tc64_gemm(int64_t rows, int 
           for (int t = 0; t < 8; ++t) x[t] = fx::fix<56>(v[t], E);
           // buffer b is free once the products that read it completed: chunk g - 2's, or
           // (resident) the previous tile's last pass
-          if (!resident && g >= 2 && !tc::mbar_wait(empty + b, ((g - 2) >> 1) & 1u)) *abort_flag = 1;
-          if (resident && it >= 1 && !tc::mbar_wait(empty + b, (it - 1) & 1u)) *abort_flag = 1;
+          if (!resident && g >= 2) tc::wait_or_abort(empty + b, ((g - 2) >> 1) & 1u, abort_flag);
+          if (resident && it >= 1) tc::wait_or_abort(empty + b, (it - 1) & 1u, abort_flag);
           fx::digits8(x, sA + b * kABytes + (e >> 3) * 512 + q * 128 + (e & 7) * 16, kASlice);
           tc::fence_async_smem();
           __syncwarp();
-          if (lane == 0) asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.shared::cta.b64 st, [%0];\n}\n" ::"r"(
-                                          tc::smem_addr(full + b))
-                                      : "memory");
+          if (lane == 0) tc::mbar_arrive(full + b);
         }
-        // drain: output columns [12q, 12q + 12) of this pass
-        if (!tc::mbar_wait(acc_full, pass & 1u)) *abort_flag = 1;
+        // drain: output columns [NC/4 q, NC/4 (q + 1)) of this pass
+        const uint32_t ab = pass % kAcc;
+        tc::wait_or_abort(accf + ab, (pass / kAcc) & 1u, abort_flag);
         tc::fence_after();
 #pragma unroll 1
-        for (int p = 0; p < 3; ++p) {
-          const int c0 = 12 * q + 4 * p;
+        for (int p = 0; p < NC / 16; ++p) {
+          const int c0 = NC / 4 * q + 4 * p;
+          __syncwarp();
+          if (nc * NC + c0 >= M) break;
           float acc[4][kSums];
 #pragma unroll
           for (int s = 0; s < kSums; ++s) {
             uint32_t vv[4];
-            tc::tmem_ld4(tb + lanebase + s * kNC + c0, vv);
+            tc::tmem_ld4(tb + lanebase + (ab * kSums + s) * NC + c0, vv);
 #pragma unroll
             for (int c = 0; c < 4; ++c) acc[c][s] = __uint_as_float(vv[c]);
           }
           tc::tmem_wait_ld();
-          if (p == 2) {  // the accumulators are read: release them to the next pass
-            tc::fence_before();
-            __syncwarp();
-            if (lane == 0) asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.shared::cta.b64 st, [%0];\n}\n" ::"r"(
-                                            tc::smem_addr(acc_empty))
-                                        : "memory");
-          }
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
-            const int col = nc * kNC + c0 + c;
+            const int col = nc * NC + c0 + c;
             if (live && col < M) {
               const double v = fx::to_double(fx::from_sums(acc[c]), __ldg(ea + col) + E - 56);
               if (accum) out[row * ldo + col] += v;
@@ -253,6 +265,9 @@ __global__ void __launch_bounds__(kSlicers + 32, 1) tc64_gemm(int64_t rows, int 
             }
           }
         }
+        tc::fence_before();
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(acce + ab);
       }
     }
   }
@@ -263,7 +278,6 @@ __global__ void __launch_bounds__(kSlicers + 32, 1) tc64_gemm(int64_t rows, int 
   if (warp == 0) tc::tmem_dealloc(tb, 512);
 }
 
-// ------------------------------------------------------------------ host side
 }  // namespace
 
 // A (M x K, row-major FP64) into the block layout of tc64_gemm; cudaErrorInvalidValue if
@@ -271,10 +285,12 @@ __global__ void __launch_bounds__(kSlicers + 32, 1) tc64_gemm(int64_t rows, int 
 cudaError_t tc64_op_create(const std::vector<double>& A, int M, int K, Tc64Op* op) {
   op->M = M;
   op->K = K;
-  op->NCH = (M + kNC - 1) / kNC;
+  const int nc = pass_columns(M, K), bytes = block_bytes(nc);
+  op->nc = nc;
+  op->NCH = (M + nc - 1) / nc;
   op->KCH = (K + kKC - 1) / kKC;
-  std::vector<uint8_t> img(size_t(op->NCH) * op->KCH * kBBytes, 0);
-  std::vector<int> ea(size_t(op->NCH) * kNC, 0);
+  std::vector<uint8_t> img(size_t(op->NCH) * op->KCH * bytes, 0);
+  std::vector<int> ea(size_t(op->NCH) * nc, 0);
   for (int r = 0; r < M; ++r) {
     double mx = 0.0, l1 = 0.0;
     for (int k = 0; k < K; ++k) {
@@ -289,9 +305,9 @@ cudaError_t tc64_op_create(const std::vector<double>& A, int M, int K, Tc64Op* o
       int d[kDigits];
       fx::digits_of(v, ea[r], d);
       for (int i = 0; i < 4; ++i) l1d[i] += std::abs(d[i]);
-      uint8_t* blk = img.data() + size_t(r / kNC * op->KCH + k / kKC) * kBBytes;
+      uint8_t* blk = img.data() + size_t(r / nc * op->KCH + k / kKC) * bytes;
       for (int i = 0; i < kDigits; ++i) {
-        const int R = i * kNC + r % kNC, c = k % kKC;
+        const int R = i * nc + r % nc, c = k % kKC;
         const uint16_t h = fx::fp16_int(d[i]);
         std::memcpy(blk + size_t(R / 8) * ((kKC / 8) * 128) + size_t(c / 8) * 128 + size_t(R % 8) * 16 + size_t(c % 8) * 2,
                     &h, 2);
@@ -329,7 +345,9 @@ cudaError_t tc64_gemm_launch(const Tc64Op& op, int64_t rows, const double* X, in
   {
     std::lock_guard<std::mutex> lk(table_mutex());
     if (!grid[dev & 63]) {
-      e = cudaFuncSetAttribute(tc64_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+      e = cudaFuncSetAttribute(tc64_gemm<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem(32));
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(tc64_gemm<48>, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem(48));
       int sms = 0;
       if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
       if (e != cudaSuccess) return e;
@@ -339,8 +357,12 @@ cudaError_t tc64_gemm_launch(const Tc64Op& op, int64_t rows, const double* X, in
   const int vec2 = (ldx % 2 == 0 && (reinterpret_cast<uintptr_t>(X) & 15u) == 0) ? 1 : 0;
   const int64_t tiles = (rows + kT - 1) / kT;
   const unsigned g = unsigned(std::min<int64_t>(tiles, grid[dev & 63]));
-  tc64_gemm<<<g, kSlicers + 32, kSmem, st>>>(rows, op.M, op.K, op.NCH, op.KCH, X, ldx, vec2, ex, op.blocks, op.ea, out,
-                                             ldo, accum);
+  if (op.nc == 32)
+    tc64_gemm<32><<<g, kSlicers + 64, gemm_smem(32), st>>>(rows, op.M, op.K, op.NCH, op.KCH, X, ldx, vec2, ex, op.blocks,
+                                                           op.ea, out, ldo, accum);
+  else
+    tc64_gemm<48><<<g, kSlicers + 64, gemm_smem(48), st>>>(rows, op.M, op.K, op.NCH, op.KCH, X, ldx, vec2, ex, op.blocks,
+                                                           op.ea, out, ldo, accum);
   note_launch();
   return cudaGetLastError();
 }

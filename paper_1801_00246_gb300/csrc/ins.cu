@@ -57,7 +57,7 @@ struct InsWorkspace {
   int npP = 0, colP[3] = {};  // projection blocks and their first columns in Y
   double* nrm = nullptr;      // [3][3][K]: per face n_x, n_y, sJ / J
   // point values of U^n, U^{n-1} and the velocity data, and of the advected fields; fluxes; projection
-  double *WU = nullptr, *WG = nullptr, *W = nullptr, *Y = nullptr, *R = nullptr;
+  double *WU = nullptr, *WG = nullptr, *gu = nullptr, *W = nullptr, *Y = nullptr, *R = nullptr;
   // the advected fields U~ (two buffers, [2 fields][2][K][Np]) and their LSERK residual
   double *Ut0 = nullptr, *Ut1 = nullptr, *res = nullptr, *Uhat = nullptr, *Uhh = nullptr, *bu = nullptr,
          *G = nullptr, *bp = nullptr, *dP = nullptr, *tmp = nullptr;
@@ -471,13 +471,14 @@ cudaError_t launch_advect(const dg_mesh* m, InsWorkspace* w, const double* Un, c
 //   Y = [ G.F at the volume points | (sJ/J) n.F* at the face points ]   same rows
 //   R = [Pr Ps -Lc] Y    same rows, Np each: the right-hand side
 // then the LSERK update; Ubar = ca U^n + cb U^{n-1} at the points from WU, the
-// interpolants of both, formed once a step. A face point's neighbour value is the
-// neighbour's own interpolant at the mirrored Gauss point.
+// interpolants of both, formed once a step and turned into what the fluxes take
+// (k_adv_metric): (U.grad r, U.grad s) at a volume point, (n.U, -) at a face point.
+// A face point's neighbour value is the neighbour's own interpolant at the
+// mirrored Gauss point (its n.U with the opposite sign).
 // At 8,192 elements of degree 8 a stage took 280 us, 117 us of it this kernel's
 // predecessor, which interpolated the face values itself on the FP64 pipe (nine
-// nodes of four fields of both sides a point): now 167 us, 69 us of it this kernel
-// (12 FP64 operations a volume point, about 30 a face point), and 271 us for two
-// fields at once.
+// nodes of four fields of both sides a point). Now the pipe, which still bounds it,
+// has 8 operations a volume point and about 15 a face point.
 
 // n_x, n_y, sJ / J of every face: [f][3][K]
 __global__ void k_adv_normals(int64_t K, const double* __restrict__ geo, double* __restrict__ nrm) {
@@ -495,11 +496,34 @@ __global__ void k_adv_normals(int64_t K, const double* __restrict__ geo, double*
 
 __host__ __device__ constexpr int pad2(int n) { return (n + 1) & ~1; }  // Y's rows start on 16 bytes
 
+// In place on point values [2][K][MW] of a velocity: at volume points (u, v) ->
+// (u.grad r, u.grad s), at face points u -> n.u (v is kept: the boundary data need it,
+// and for them u goes to `keep` [K][3 nc]).
+__global__ void k_adv_metric(int Nc, int nc, int64_t K, const double* __restrict__ geo, const double* __restrict__ nrm,
+                             double* __restrict__ W, double* __restrict__ keep) {
+  const int MW = Nc + 3 * nc;
+  const int64_t total = K * MW;
+  for (int64_t idx = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; idx < total;
+       idx += int64_t(gridDim.x) * blockDim.x) {
+    const int64_t e = idx / MW;
+    const int m = int(idx - e * MW);
+    const double u = W[idx], v = W[total + idx];
+    if (m < Nc) {
+      W[idx] = geo[4 * e] * u + geo[4 * e + 2] * v;
+      W[total + idx] = geo[4 * e + 1] * u + geo[4 * e + 3] * v;
+    } else {
+      const int f = (m - Nc) / nc;
+      W[idx] = nrm[(3 * f + 0) * K + e] * u + nrm[(3 * f + 1) * K + e] * v;
+      if (keep) keep[e * 3 * nc + m - Nc] = u;
+    }
+  }
+}
+
 // NF advected fields at once (one thread per cubature point of an element)
 template <int NF>
-__global__ void k_adv_flux(int Nc, int nc, int64_t K, const double* __restrict__ geo, const double* __restrict__ nrm,
-                           const int32_t* __restrict__ conn, const double* __restrict__ WU,
-                           const double* __restrict__ WG, double ca, double cb, const double* __restrict__ W,
+__global__ void k_adv_flux(int Nc, int nc, int64_t K, const double* __restrict__ nrm, const int32_t* __restrict__ conn,
+                           const double* __restrict__ WU, const double* __restrict__ WG,
+                           const double* __restrict__ gu, double ca, double cb, const double* __restrict__ W,
                            double* __restrict__ Y) {
   const int MW = Nc + 3 * nc, ldY = pad2(2 * Nc + 3 * nc);
   const int64_t total = K * MW, fsY = K * ldY;
@@ -511,34 +535,31 @@ __global__ void k_adv_flux(int Nc, int nc, int64_t K, const double* __restrict__
        idx += int64_t(gridDim.x) * blockDim.x) {
     const int64_t e = total < (int64_t(1) << 31) ? int64_t(uint32_t(idx) / uint32_t(MW)) : idx / MW;
     const int m = int(idx - e * MW);
-    const double u = ubar(0, idx), v = ubar(1, idx);
+    double w[2 * NF];
+#pragma unroll
+    for (int c = 0; c < 2 * NF; ++c) w[c] = __ldg(W + c * total + idx);
     if (m < Nc) {
-      const double2 gx = *reinterpret_cast<const double2*>(geo + 4 * e);      // r_x, s_x
-      const double2 gy = *reinterpret_cast<const double2*>(geo + 4 * e + 2);  // r_y, s_y
-      const double ur = gx.x * u + gy.x * v, us = gx.y * u + gy.y * v;
+      const double ur = ubar(0, idx), us = ubar(1, idx);
 #pragma unroll
       for (int c = 0; c < 2 * NF; ++c) {
-        const double w = __ldg(W + c * total + idx);
         double* y = Y + c * fsY + e * ldY + m;
-        y[0] = ur * w;
-        y[Nc] = us * w;
+        y[0] = ur * w[c];
+        y[Nc] = us * w[c];
       }
     } else {
       const int q = m - Nc, f = q / nc, k = q - f * nc;
       const int code = __ldg(conn + 3 * e + f);
       const int64_t in = code >= 0 ? int64_t(code >> 2) * MW + Nc + (code & 3) * nc + (nc - 1 - k) : idx;
       const bool data = code == -2;  // velocity Dirichlet: exterior state is the boundary datum (Neumann: the interior)
-      const double up = data ? __ldg(WG + idx) : (code >= 0 ? ubar(0, in) : u);
-      const double vp = data ? __ldg(WG + total + idx) : (code >= 0 ? ubar(1, in) : v);
-      const double nx = __ldg(nrm + (3 * f + 0) * K + e), ny = __ldg(nrm + (3 * f + 1) * K + e),
-                   sjj = __ldg(nrm + (3 * f + 2) * K + e);
-      const double unm = nx * u + ny * v, unp = nx * up + ny * vp;
-      const double lam = fmax(fabs(unm), fabs(unp));
+      const double unm = ubar(0, idx);
+      const double unp = data ? __ldg(WG + idx) : (code >= 0 ? -ubar(0, in) : unm);
+      const double sh = 0.5 * __ldg(nrm + (3 * f + 2) * K + e);
+      // F* = (n.u- w- + n.u+ w+) / 2 + lam (w- - w+) / 2
+      const double lam = fmax(fabs(unm), fabs(unp)), fm = sh * (unm + lam), fp = sh * (unp - lam);
 #pragma unroll
       for (int c = 0; c < 2 * NF; ++c) {
-        const double w = __ldg(W + c * total + idx);
-        const double wp = data ? __ldg(WG + (c & 1) * total + idx) : __ldg(W + c * total + in);
-        Y[c * fsY + e * ldY + 2 * Nc + q] = sjj * (0.5 * (unm * w + unp * wp) + 0.5 * lam * (w - wp));
+        const double wp = data ? ((c & 1) ? __ldg(WG + total + idx) : __ldg(gu + e * 3 * nc + q)) : __ldg(W + c * total + in);
+        Y[c * fsY + e * ldY + 2 * Nc + q] = fm * w[c] + fp * wp;
       }
     }
   }
@@ -624,6 +645,7 @@ cudaError_t setup_ins(dg_mesh* m) {
     ICK(al(&w->nrm, 9 * size_t(m->K)));
     ICK(al(&w->WU, 4 * nw));
     ICK(al(&w->WG, 2 * nw));
+    ICK(al(&w->gu, 3 * size_t(nc) * m->K));
     ICK(al(&w->W, 4 * nw));
     ICK(al(&w->Y, 4 * size_t(m->K) * pad2(KY)));
     ICK(al(&w->R, 4 * n1));
@@ -635,6 +657,15 @@ cudaError_t setup_ins(dg_mesh* m) {
   return cudaSuccess;
 }
 
+// A velocity field's point values in the form the fluxes take (keep: see k_adv_metric).
+cudaError_t point_values(const dg_mesh* m, InsWorkspace* w, const double* u, double* W, double* keep, cudaStream_t st) {
+  const AdvLayout& L = w->L;
+  ICK(tc64_gemm_launch(w->opI, 2 * m->K, u, L.Np, W, w->opI.M, st));
+  k_adv_metric<<<eg(m->K * w->opI.M), 256, 0, st>>>(L.Nc, L.nc, m->K, m->geo64, w->nrm, W, keep);
+  note_launch();
+  return cudaGetLastError();
+}
+
 // One LSERK stage of nf advected fields on the tensor cores (see k_adv_flux).
 cudaError_t advect_stage_tensor(const dg_mesh* m, InsWorkspace* w, int nf, double ca, double cb, const double* Ut_in,
                                 double* Ut_out, double a, double b, double dts, cudaStream_t st) {
@@ -642,8 +673,8 @@ cudaError_t advect_stage_tensor(const dg_mesh* m, InsWorkspace* w, int nf, doubl
   const int Np = L.Np, Nc = L.Nc, nc = L.nc, MW = Nc + 3 * nc;
   const int64_t K = m->K, rows = 2 * K * nf;
   ICK(tc64_gemm_launch(w->opI, rows, Ut_in, Np, w->W, MW, st));
-  if (nf == 1) k_adv_flux<1><<<eg(K * MW), 256, 0, st>>>(Nc, nc, K, m->geo64, w->nrm, m->conn, w->WU, w->WG, ca, cb, w->W, w->Y);
-  else k_adv_flux<2><<<eg(K * MW), 256, 0, st>>>(Nc, nc, K, m->geo64, w->nrm, m->conn, w->WU, w->WG, ca, cb, w->W, w->Y);
+  if (nf == 1) k_adv_flux<1><<<eg(K * MW), 256, 0, st>>>(Nc, nc, K, w->nrm, m->conn, w->WU, w->WG, w->gu, ca, cb, w->W, w->Y);
+  else k_adv_flux<2><<<eg(K * MW), 256, 0, st>>>(Nc, nc, K, w->nrm, m->conn, w->WU, w->WG, w->gu, ca, cb, w->W, w->Y);
   note_launch();
   for (int p = 0; p < w->npP; ++p)
     ICK(tc64_gemm_launch(w->opP[p], rows, w->Y + w->colP[p], pad2(2 * Nc + 3 * nc), w->R, Np, st, p > 0));
@@ -683,7 +714,7 @@ cudaError_t advect_substeps(const dg_mesh* m, InsWorkspace* w, const dg_ins_stat
           note_launch();
         }
         g = w->gts;
-        if (w->tensor) ICK(tc64_gemm_launch(w->opI, 2 * m->K, g, Np, w->WG, w->opI.M, st));
+        if (w->tensor) ICK(point_values(m, w, g, w->WG, w->gu, st));
       }
       if (w->tensor) {
         ICK(advect_stage_tensor(m, w, nf, ca, cb, *cur, nxt, kRkA[stg], kRkB[stg], dts, st));
@@ -707,9 +738,9 @@ cudaError_t advect_history(const dg_mesh* m, InsWorkspace* w, const dg_ins_state
   const bool first = s->step == 0;
   if (w->tensor) {
     const size_t nw = 2 * size_t(m->K) * w->opI.M;
-    ICK(tc64_gemm_launch(w->opI, 2 * m->K, s->U, Np, w->WU, w->opI.M, st));
-    if (!first) ICK(tc64_gemm_launch(w->opI, 2 * m->K, s->Uold, Np, w->WU + nw, w->opI.M, st));
-    if (!s->gU_hist) ICK(tc64_gemm_launch(w->opI, 2 * m->K, s->gU, Np, w->WG, w->opI.M, st));
+    ICK(point_values(m, w, s->U, w->WU, nullptr, st));
+    if (!first) ICK(point_values(m, w, s->Uold, w->WU + nw, nullptr, st));
+    if (!s->gU_hist) ICK(point_values(m, w, s->gU, w->WG, w->gu, st));
   }
   ICK(cudaMemsetAsync(w->res, 0, 2 * bytes, st));
   double* cur = w->Ut0;

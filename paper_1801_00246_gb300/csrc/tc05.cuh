@@ -116,6 +116,19 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, uint64_t
     if (__any_sync(0xffffffffu, globaltimer_ns() - t0 > limit_ns)) return false;
   }
 }
+// A wait that gave up sets the block's abort flag, and every later wait then
+// returns at once: all warps run to the end of their loops (their named
+// barriers stay matched) and the block ends.
+__device__ __forceinline__ bool aborted(volatile int* flag) { return __any_sync(0xffffffffu, *flag != 0); }
+__device__ __forceinline__ void wait_or_abort(uint64_t* b, uint32_t parity, volatile int* abort_flag) {
+  if (!aborted(abort_flag) && !mbar_wait(b, parity)) *abort_flag = 1;
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t* b) {
+  asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.shared::cta.b64 st, [%0];\n}\n" ::"r"(smem_addr(b)) : "memory");
+}
+__device__ __forceinline__ void bar_sync(int id, int threads) {
+  asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(threads) : "memory");
+}
 // arm the barrier for `bytes` of bulk-copy traffic (one arrival)
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* b, uint32_t bytes) {
   asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n}\n" ::"r"(
