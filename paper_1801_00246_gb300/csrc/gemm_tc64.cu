@@ -42,7 +42,10 @@ int pass_columns(int M, int K) { return K <= 2 * kKC || M <= 32 ? 32 : 48; }
 
 __device__ int g_tc64_err;
 
-// out[r][c] = sum_k A[c][k] X[r][k] for r < rows, c < M, k < Kd (A sliced in
+// out[r][c] = sum_k A[c][k] X[r][k] for r < rows, c < M, k < Kd; X row-major, or with
+// xcol, out with ocol (COLS only), column-major (ldx, ldo then lie between columns: a warp's 32
+// rows read and write 256 contiguous bytes a column, where rows of an odd length cost
+// 32 sectors an access) (A sliced in
 // blocks of NC rows x kKC columns: block (nc, kc) at (nc KCH + kc) block_bytes).
 //
 // Warp-specialised pipeline over a stream of data chunks (tile, output pass
@@ -59,13 +62,13 @@ __device__ int g_tc64_err;
 //    16,384 rows of 208 outputs, 45 deep, took 44 us).
 // No CTA-wide barrier in the steady state; every wait is bounded in time.
 constexpr int kSlicers = 512;  // threads of warps 0-15
-template <int NC>
+template <int NC, bool COLS>
 __global__ void __launch_bounds__(kSlicers + 64, 1) tc64_gemm(int64_t rows, int M, int Kd, int NCH, int KCH,
                                                               const double* __restrict__ X, int64_t ldx, int vec2,
-                                                              const int* __restrict__ ex_given,
+                                                              int xcol, const int* __restrict__ ex_given,
                                                               const uint8_t* __restrict__ Bops,
                                                               const int* __restrict__ ea, double* __restrict__ out,
-                                                              int64_t ldo, int accum) {
+                                                              int64_t ldo, int ocol, int accum) {
   extern __shared__ __align__(1024) uint8_t sm[];
   constexpr int kBBytes = block_bytes(NC);
   constexpr int kAcc = 2 * kSums * NC <= 512 ? 2 : 1;  // accumulator sets
@@ -158,7 +161,10 @@ __global__ void __launch_bounds__(kSlicers + 64, 1) tc64_gemm(int64_t rows, int 
     const uint32_t lanebase = uint32_t((warp & 3) * 32) << 16;
     uint32_t g = 0, pass = 0, it = 0;
     auto load8 = [&](const double* xr, bool live, int k0, double (&v)[8]) {
-      if (live && vec2 && k0 + 8 <= Kd) {
+      if (COLS && xcol) {
+#pragma unroll
+        for (int t = 0; t < 8; ++t) v[t] = (live && k0 + t < Kd) ? __ldg(xr + int64_t(k0 + t) * ldx) : 0.0;
+      } else if (live && vec2 && k0 + 8 <= Kd) {
         const double2* p2 = reinterpret_cast<const double2*>(xr + k0);
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
@@ -180,7 +186,7 @@ __global__ void __launch_bounds__(kSlicers + 64, 1) tc64_gemm(int64_t rows, int 
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
       const int64_t row = tile * kT + e;
       const bool live = row < rows;
-      const double* xr = X + (live ? row : 0) * ldx;
+      const double* xr = X + (live ? row : 0) * (COLS && xcol ? 1 : ldx);
       // scale exponent of the row: a bound |X[row][k]| < 2^E, given by the producer
       // of X or found here
       int E;
@@ -220,7 +226,7 @@ __global__ void __launch_bounds__(kSlicers + 64, 1) tc64_gemm(int64_t rows, int 
             } else if (ex_given && nc + 1 == NCH && tile + gridDim.x < ntiles) {
               const int64_t nrow = row + int64_t(gridDim.x) * kT;
               const bool nlive = nrow < rows;
-              load8(X + (nlive ? nrow : 0) * ldx, nlive, 8 * q, vn);
+              load8(X + (nlive ? nrow : 0) * (COLS && xcol ? 1 : ldx), nlive, 8 * q, vn);
               En = nlive ? __ldg(ex_given + nrow) : 0;
               have_next = true;
             }
@@ -260,8 +266,8 @@ __global__ void __launch_bounds__(kSlicers + 64, 1) tc64_gemm(int64_t rows, int 
             const int col = nc * NC + c0 + c;
             if (live && col < M) {
               const double v = fx::to_double(fx::from_sums(acc[c]), __ldg(ea + col) + E - 56);
-              if (accum) out[row * ldo + col] += v;
-              else out[row * ldo + col] = v;
+              double* o = out + (COLS && ocol ? col * ldo + row : row * ldo + col);
+              *o = accum ? *o + v : v;
             }
           }
         }
@@ -278,6 +284,12 @@ __global__ void __launch_bounds__(kSlicers + 64, 1) tc64_gemm(int64_t rows, int 
   if (warp == 0) tc::tmem_dealloc(tb, 512);
 }
 
+template <int NC>
+cudaError_t allow_smem() {
+  const auto a = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  const cudaError_t e = cudaFuncSetAttribute(tc64_gemm<NC, false>, a, gemm_smem(NC));
+  return e == cudaSuccess ? cudaFuncSetAttribute(tc64_gemm<NC, true>, a, gemm_smem(NC)) : e;
+}
 }  // namespace
 
 // A (M x K, row-major FP64) into the block layout of tc64_gemm; cudaErrorInvalidValue if
@@ -336,7 +348,7 @@ void tc64_op_free(Tc64Op* op) {
 }
 
 cudaError_t tc64_gemm_launch(const Tc64Op& op, int64_t rows, const double* X, int64_t ldx, double* out, int64_t ldo,
-                             cudaStream_t st, int accum, const int* ex) {
+                             cudaStream_t st, int accum, const int* ex, int xcol, int ocol) {
   if (rows <= 0) return cudaSuccess;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -345,9 +357,8 @@ cudaError_t tc64_gemm_launch(const Tc64Op& op, int64_t rows, const double* X, in
   {
     std::lock_guard<std::mutex> lk(table_mutex());
     if (!grid[dev & 63]) {
-      e = cudaFuncSetAttribute(tc64_gemm<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem(32));
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(tc64_gemm<48>, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem(48));
+      e = allow_smem<32>();
+      if (e == cudaSuccess) e = allow_smem<48>();
       int sms = 0;
       if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
       if (e != cudaSuccess) return e;
@@ -357,12 +368,14 @@ cudaError_t tc64_gemm_launch(const Tc64Op& op, int64_t rows, const double* X, in
   const int vec2 = (ldx % 2 == 0 && (reinterpret_cast<uintptr_t>(X) & 15u) == 0) ? 1 : 0;
   const int64_t tiles = (rows + kT - 1) / kT;
   const unsigned g = unsigned(std::min<int64_t>(tiles, grid[dev & 63]));
-  if (op.nc == 32)
-    tc64_gemm<32><<<g, kSlicers + 64, gemm_smem(32), st>>>(rows, op.M, op.K, op.NCH, op.KCH, X, ldx, vec2, ex, op.blocks,
-                                                           op.ea, out, ldo, accum);
-  else
-    tc64_gemm<48><<<g, kSlicers + 64, gemm_smem(48), st>>>(rows, op.M, op.K, op.NCH, op.KCH, X, ldx, vec2, ex, op.blocks,
-                                                           op.ea, out, ldo, accum);
+  // (the layouts of a product with a column-major side stay run-time choices: the
+  // specialised forms measured 8 ms slower in a flow step of 70 ms)
+  auto go = [&](auto kernel) {
+    kernel<<<g, kSlicers + 64, gemm_smem(op.nc), st>>>(rows, op.M, op.K, op.NCH, op.KCH, X, ldx, vec2, xcol, ex, op.blocks,
+                                                       op.ea, out, ldo, ocol, accum);
+  };
+  if (op.nc == 32) xcol || ocol ? go(tc64_gemm<32, true>) : go(tc64_gemm<32, false>);
+  else xcol || ocol ? go(tc64_gemm<48, true>) : go(tc64_gemm<48, false>);
   note_launch();
   return cudaGetLastError();
 }

@@ -58,7 +58,8 @@ struct InsWorkspace {
   double* nrm = nullptr;      // [3][3][K]: per face n_x, n_y, sJ / J
   // point values of U^n, U^{n-1} and the velocity data, and of the advected fields; fluxes; projection
   double *WU = nullptr, *WG = nullptr, *gu = nullptr, *W = nullptr, *Y = nullptr, *R = nullptr;
-  // the advected fields U~ (two buffers, [2 fields][2][K][Np]) and their LSERK residual
+  // the advected fields U~ (two buffers, [2 fields][2][K][Np], or on the tensor cores
+  // [Np][2 fields][2][K]) and their LSERK residual
   double *Ut0 = nullptr, *Ut1 = nullptr, *res = nullptr, *Uhat = nullptr, *Uhh = nullptr, *bu = nullptr,
          *G = nullptr, *bp = nullptr, *dP = nullptr, *tmp = nullptr;
   double *gts = nullptr, *zero = nullptr;  // time-dependent data: velocity data at a stage time; zeros
@@ -470,6 +471,9 @@ cudaError_t launch_advect(const dg_mesh* m, InsWorkspace* w, const double* Un, c
 //   W = I U~             rows (2 field + c) K + e, the Nc volume and 3 nc face points each
 //   Y = [ G.F at the volume points | (sJ/J) n.F* at the face points ]   same rows
 //   R = [Pr Ps -Lc] Y    same rows, Np each: the right-hand side
+// All of them, and U~ while it is advected, are column-major (entry i of row r at
+// [i][r]), so that every kernel's lanes are neighbouring elements at one point: each
+// access but the neighbour's is contiguous and no lane takes another branch.
 // then the LSERK update; Ubar = ca U^n + cb U^{n-1} at the points from WU, the
 // interpolants of both, formed once a step and turned into what the fluxes take
 // (k_adv_metric): (U.grad r, U.grad s) at a volume point, (n.U, -) at a face point.
@@ -494,85 +498,103 @@ __global__ void k_adv_normals(int64_t K, const double* __restrict__ geo, double*
   }
 }
 
-__host__ __device__ constexpr int pad2(int n) { return (n + 1) & ~1; }  // Y's rows start on 16 bytes
+// Rows [r][Np] of two components into columns [Np][ld] (back = 0) or out of them
+__global__ void k_adv_transpose(int Np, int64_t rows, int64_t ld, double* __restrict__ rowm, double* __restrict__ colm,
+                                int back) {
+  __shared__ double t[32][33];
+  const int64_t r0 = int64_t(blockIdx.x) * 32;
+  const int n0 = blockIdx.y * 32;
+  if (back) {
+    for (int k = threadIdx.y; k < 32; k += blockDim.y)
+      if (n0 + k < Np && r0 + threadIdx.x < rows) t[k][threadIdx.x] = colm[(n0 + k) * ld + r0 + threadIdx.x];
+    __syncthreads();
+    for (int k = threadIdx.y; k < 32; k += blockDim.y)
+      if (n0 + threadIdx.x < Np && r0 + k < rows) rowm[(r0 + k) * Np + n0 + threadIdx.x] = t[threadIdx.x][k];
+  } else {
+    for (int k = threadIdx.y; k < 32; k += blockDim.y)
+      if (n0 + threadIdx.x < Np && r0 + k < rows) t[k][threadIdx.x] = rowm[(r0 + k) * Np + n0 + threadIdx.x];
+    __syncthreads();
+    for (int k = threadIdx.y; k < 32; k += blockDim.y)
+      if (n0 + k < Np && r0 + threadIdx.x < rows) colm[(n0 + k) * ld + r0 + threadIdx.x] = t[threadIdx.x][k];
+  }
+}
 
-// In place on point values [2][K][MW] of a velocity: at volume points (u, v) ->
+// In place on point values [MW][2][K] of a velocity: at volume points (u, v) ->
 // (u.grad r, u.grad s), at face points u -> n.u (v is kept: the boundary data need it,
-// and for them u goes to `keep` [K][3 nc]).
+// and for them u goes to `keep` [3 nc][K]). The grid's second dimension is the point.
 __global__ void k_adv_metric(int Nc, int nc, int64_t K, const double* __restrict__ geo, const double* __restrict__ nrm,
                              double* __restrict__ W, double* __restrict__ keep) {
-  const int MW = Nc + 3 * nc;
-  const int64_t total = K * MW;
-  for (int64_t idx = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; idx < total;
-       idx += int64_t(gridDim.x) * blockDim.x) {
-    const int64_t e = idx / MW;
-    const int m = int(idx - e * MW);
-    const double u = W[idx], v = W[total + idx];
-    if (m < Nc) {
-      W[idx] = geo[4 * e] * u + geo[4 * e + 2] * v;
-      W[total + idx] = geo[4 * e + 1] * u + geo[4 * e + 3] * v;
-    } else {
-      const int f = (m - Nc) / nc;
-      W[idx] = nrm[(3 * f + 0) * K + e] * u + nrm[(3 * f + 1) * K + e] * v;
-      if (keep) keep[e * 3 * nc + m - Nc] = u;
-    }
+  const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  const int m = blockIdx.y;
+  if (e >= K) return;
+  double* w = W + 2 * K * m + e;
+  const double u = w[0], v = w[K];
+  if (m < Nc) {
+    w[0] = geo[4 * e] * u + geo[4 * e + 2] * v;
+    w[K] = geo[4 * e + 1] * u + geo[4 * e + 3] * v;
+  } else {
+    const int f = (m - Nc) / nc;
+    w[0] = nrm[(3 * f + 0) * K + e] * u + nrm[(3 * f + 1) * K + e] * v;
+    if (keep) keep[int64_t(m - Nc) * K + e] = u;
   }
 }
 
-// NF advected fields at once (one thread per cubature point of an element)
+// NF advected fields at once: one thread per element and cubature point (the grid's
+// second dimension); ld: rows between W's and Y's columns
 template <int NF>
-__global__ void k_adv_flux(int Nc, int nc, int64_t K, const double* __restrict__ nrm, const int32_t* __restrict__ conn,
-                           const double* __restrict__ WU, const double* __restrict__ WG,
-                           const double* __restrict__ gu, double ca, double cb, const double* __restrict__ W,
-                           double* __restrict__ Y) {
-  const int MW = Nc + 3 * nc, ldY = pad2(2 * Nc + 3 * nc);
-  const int64_t total = K * MW, fsY = K * ldY;
-  auto ubar = [&](int c, int64_t i) {
-    const double a = ca * __ldg(WU + c * total + i);
-    return cb != 0.0 ? a + cb * __ldg(WU + (2 + c) * total + i) : a;
+__global__ void __launch_bounds__(256) k_adv_flux(int Nc, int nc, int64_t K, int64_t ld, const double* __restrict__ nrm,
+                                                  const int32_t* __restrict__ conn, const double* __restrict__ WU,
+                                                  const double* __restrict__ WG, const double* __restrict__ gu,
+                                                  double ca, double cb, const double* __restrict__ W,
+                                                  double* __restrict__ Y) {
+  const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  const int m = blockIdx.y;
+  if (e >= K) return;
+  const int64_t old = int64_t(Nc + 3 * nc) * 2 * K;  // U^{n-1}'s values behind U^n's
+  auto ubar = [&](int64_t i) {
+    const double a = ca * __ldg(WU + i);
+    return cb != 0.0 ? a + cb * __ldg(WU + old + i) : a;
   };
-  for (int64_t idx = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; idx < total;
-       idx += int64_t(gridDim.x) * blockDim.x) {
-    const int64_t e = total < (int64_t(1) << 31) ? int64_t(uint32_t(idx) / uint32_t(MW)) : idx / MW;
-    const int m = int(idx - e * MW);
-    double w[2 * NF];
+  const double* w0 = W + m * ld + e;
+  double w[2 * NF];
 #pragma unroll
-    for (int c = 0; c < 2 * NF; ++c) w[c] = __ldg(W + c * total + idx);
-    if (m < Nc) {
-      const double ur = ubar(0, idx), us = ubar(1, idx);
+  for (int c = 0; c < 2 * NF; ++c) w[c] = __ldg(w0 + c * K);
+  if (m < Nc) {
+    const double ur = ubar(2 * K * m + e), us = ubar(2 * K * m + K + e);
 #pragma unroll
-      for (int c = 0; c < 2 * NF; ++c) {
-        double* y = Y + c * fsY + e * ldY + m;
-        y[0] = ur * w[c];
-        y[Nc] = us * w[c];
-      }
-    } else {
-      const int q = m - Nc, f = q / nc, k = q - f * nc;
-      const int code = __ldg(conn + 3 * e + f);
-      const int64_t in = code >= 0 ? int64_t(code >> 2) * MW + Nc + (code & 3) * nc + (nc - 1 - k) : idx;
-      const bool data = code == -2;  // velocity Dirichlet: exterior state is the boundary datum (Neumann: the interior)
-      const double unm = ubar(0, idx);
-      const double unp = data ? __ldg(WG + idx) : (code >= 0 ? -ubar(0, in) : unm);
-      const double sh = 0.5 * __ldg(nrm + (3 * f + 2) * K + e);
-      // F* = (n.u- w- + n.u+ w+) / 2 + lam (w- - w+) / 2
-      const double lam = fmax(fabs(unm), fabs(unp)), fm = sh * (unm + lam), fp = sh * (unp - lam);
+    for (int c = 0; c < 2 * NF; ++c) {
+      double* y = Y + m * ld + c * K + e;
+      y[0] = ur * w[c];
+      y[Nc * ld] = us * w[c];
+    }
+  } else {
+    const int q = m - Nc, f = q / nc, k = q - f * nc;
+    const int code = __ldg(conn + 3 * e + f);
+    const bool data = code == -2;  // velocity Dirichlet: exterior state is the boundary datum (Neumann: the interior)
+    const int64_t en = code >= 0 ? code >> 2 : e;
+    const int mn = code >= 0 ? Nc + (code & 3) * nc + (nc - 1 - k) : m;
+    const double unm = ubar(2 * K * m + e);
+    const double unp = data ? __ldg(WG + 2 * K * m + e) : (code >= 0 ? -ubar(2 * K * mn + en) : unm);
+    const double sh = 0.5 * __ldg(nrm + (3 * f + 2) * K + e);
+    // F* = (n.u- w- + n.u+ w+) / 2 + lam (w- - w+) / 2
+    const double lam = fmax(fabs(unm), fabs(unp)), fm = sh * (unm + lam), fp = sh * (unp - lam);
 #pragma unroll
-      for (int c = 0; c < 2 * NF; ++c) {
-        const double wp = data ? ((c & 1) ? __ldg(WG + total + idx) : __ldg(gu + e * 3 * nc + q)) : __ldg(W + c * total + in);
-        Y[c * fsY + e * ldY + 2 * Nc + q] = fm * w[c] + fp * wp;
-      }
+    for (int c = 0; c < 2 * NF; ++c) {
+      const double wp = data ? ((c & 1) ? __ldg(WG + 2 * K * m + K + e) : __ldg(gu + int64_t(q) * K + e))
+                             : __ldg(W + mn * ld + c * K + en);
+      Y[(2 * Nc + q) * ld + c * K + e] = fm * w[c] + fp * wp;
     }
   }
 }
 
-// res = a res + dts R; Ut_out = Ut_in + b res
-__global__ void k_adv_update(int64_t n, const double* __restrict__ R, double a, double dts, double b,
+// res = a res + dts R; Ut_out = Ut_in + b res, on columns of `rows` rows, ld apart
+__global__ void k_adv_update(int64_t rows, int64_t ld, const double* __restrict__ R, double a, double dts, double b,
                              const double* __restrict__ Ut_in, double* __restrict__ res, double* __restrict__ Ut_out) {
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
-    const double r = a * res[i] + dts * R[i];
-    res[i] = r;
-    Ut_out[i] = Ut_in[i] + b * r;
-  }
+  const int64_t r0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x, i = blockIdx.y * ld + r0;
+  if (r0 >= rows) return;
+  const double r = a * res[i] + dts * R[i];
+  res[i] = r;
+  Ut_out[i] = Ut_in[i] + b * r;
 }
 
 #define ICK(x)                         \
@@ -647,7 +669,7 @@ cudaError_t setup_ins(dg_mesh* m) {
     ICK(al(&w->WG, 2 * nw));
     ICK(al(&w->gu, 3 * size_t(nc) * m->K));
     ICK(al(&w->W, 4 * nw));
-    ICK(al(&w->Y, 4 * size_t(m->K) * pad2(KY)));
+    ICK(al(&w->Y, 4 * size_t(m->K) * KY));
     ICK(al(&w->R, 4 * n1));
     k_adv_normals<<<unsigned((m->K + 255) / 256), 256>>>(m->K, m->geo64, w->nrm);
     note_launch();
@@ -660,8 +682,9 @@ cudaError_t setup_ins(dg_mesh* m) {
 // A velocity field's point values in the form the fluxes take (keep: see k_adv_metric).
 cudaError_t point_values(const dg_mesh* m, InsWorkspace* w, const double* u, double* W, double* keep, cudaStream_t st) {
   const AdvLayout& L = w->L;
-  ICK(tc64_gemm_launch(w->opI, 2 * m->K, u, L.Np, W, w->opI.M, st));
-  k_adv_metric<<<eg(m->K * w->opI.M), 256, 0, st>>>(L.Nc, L.nc, m->K, m->geo64, w->nrm, W, keep);
+  ICK(tc64_gemm_launch(w->opI, 2 * m->K, u, L.Np, W, 2 * m->K, st, 0, nullptr, 0, 1));
+  k_adv_metric<<<dim3(unsigned((m->K + 255) / 256), unsigned(w->opI.M)), 256, 0, st>>>(L.Nc, L.nc, m->K, m->geo64, w->nrm,
+                                                                                  W, keep);
   note_launch();
   return cudaGetLastError();
 }
@@ -671,14 +694,16 @@ cudaError_t advect_stage_tensor(const dg_mesh* m, InsWorkspace* w, int nf, doubl
                                 double* Ut_out, double a, double b, double dts, cudaStream_t st) {
   const AdvLayout& L = w->L;
   const int Np = L.Np, Nc = L.Nc, nc = L.nc, MW = Nc + 3 * nc;
-  const int64_t K = m->K, rows = 2 * K * nf;
-  ICK(tc64_gemm_launch(w->opI, rows, Ut_in, Np, w->W, MW, st));
-  if (nf == 1) k_adv_flux<1><<<eg(K * MW), 256, 0, st>>>(Nc, nc, K, w->nrm, m->conn, w->WU, w->WG, w->gu, ca, cb, w->W, w->Y);
-  else k_adv_flux<2><<<eg(K * MW), 256, 0, st>>>(Nc, nc, K, w->nrm, m->conn, w->WU, w->WG, w->gu, ca, cb, w->W, w->Y);
+  const int64_t K = m->K, rows = 2 * K * nf, ld = 4 * K;
+  ICK(tc64_gemm_launch(w->opI, rows, Ut_in, ld, w->W, ld, st, 0, nullptr, 1, 1));
+  const dim3 g(unsigned((K + 255) / 256), unsigned(MW));
+  if (nf == 1) k_adv_flux<1><<<g, 256, 0, st>>>(Nc, nc, K, ld, w->nrm, m->conn, w->WU, w->WG, w->gu, ca, cb, w->W, w->Y);
+  else k_adv_flux<2><<<g, 256, 0, st>>>(Nc, nc, K, ld, w->nrm, m->conn, w->WU, w->WG, w->gu, ca, cb, w->W, w->Y);
   note_launch();
   for (int p = 0; p < w->npP; ++p)
-    ICK(tc64_gemm_launch(w->opP[p], rows, w->Y + w->colP[p], pad2(2 * Nc + 3 * nc), w->R, Np, st, p > 0));
-  k_adv_update<<<eg(rows * Np), 256, 0, st>>>(rows * Np, w->R, a, dts, b, Ut_in, w->res, Ut_out);
+    ICK(tc64_gemm_launch(w->opP[p], rows, w->Y + w->colP[p] * ld, ld, w->R, ld, st, p > 0, nullptr, 1, 1));
+  k_adv_update<<<dim3(unsigned((rows + 255) / 256), unsigned(Np)), 256, 0, st>>>(rows, ld, w->R, a, dts, b, Ut_in, w->res,
+                                                                            Ut_out);
   note_launch();
   return cudaGetLastError();
 }
@@ -744,18 +769,34 @@ cudaError_t advect_history(const dg_mesh* m, InsWorkspace* w, const dg_ins_state
   }
   ICK(cudaMemsetAsync(w->res, 0, 2 * bytes, st));
   double* cur = w->Ut0;
+  // the advected fields' place in `cur` (field f) and a plain field: columns for the tensor cores
+  const int64_t rows = 2 * m->K, ld = 4 * m->K;
+  const dim3 tg(unsigned((rows + 31) / 32), unsigned((Np + 31) / 32)), tb(32, 8);
+  auto put = [&](int f, double* field) -> cudaError_t {
+    if (!w->tensor) return cudaMemcpyAsync(cur + f * n2, field, bytes, cudaMemcpyDeviceToDevice, st);
+    k_adv_transpose<<<tg, tb, 0, st>>>(Np, rows, ld, field, cur + f * rows, 0);
+    note_launch();
+    return cudaGetLastError();
+  };
+  auto take = [&](int f, double* field) -> cudaError_t {
+    if (!w->tensor) return cudaMemcpyAsync(field, cur + f * n2, bytes, cudaMemcpyDeviceToDevice, st);
+    k_adv_transpose<<<tg, tb, 0, st>>>(Np, rows, ld, field, cur + f * rows, 1);
+    note_launch();
+    return cudaGetLastError();
+  };
   if (first) {
-    ICK(cudaMemcpyAsync(cur, s->U, bytes, cudaMemcpyDeviceToDevice, st));
+    ICK(put(0, s->U));
     ICK(advect_substeps(m, w, s, 1, tn, s->Ns, tn, false, &cur, st));
-    ICK(cudaMemcpyAsync(w->Uhat, cur, bytes, cudaMemcpyDeviceToDevice, st));
-    return cudaSuccess;
+    return take(0, w->Uhat);
   }
   // U^{n-1} to t^n by itself, then with U^n to t^{n+1}
-  ICK(cudaMemcpyAsync(cur, s->Uold, bytes, cudaMemcpyDeviceToDevice, st));
+  ICK(put(0, s->Uold));
   ICK(advect_substeps(m, w, s, 1, tn - s->dt, s->Ns, tn, true, &cur, st));
-  ICK(cudaMemcpyAsync(cur + n2, s->U, bytes, cudaMemcpyDeviceToDevice, st));
+  ICK(put(1, s->U));
   ICK(advect_substeps(m, w, s, 2, tn, s->Ns, tn, true, &cur, st));
-  axpby_kernel<<<eg(n2), 256, 0, st>>>(n2, 2.0, cur + n2, 0.0, w->Uhat, -0.5, cur);
+  ICK(take(1, w->tmp));
+  ICK(take(0, w->bu));
+  axpby_kernel<<<eg(n2), 256, 0, st>>>(n2, 2.0, w->tmp, 0.0, w->Uhat, -0.5, w->bu);
   note_launch();
   return cudaGetLastError();
 }
