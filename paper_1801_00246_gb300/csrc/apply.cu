@@ -367,7 +367,10 @@ cudaError_t launch_n(const dg_mesh* m, dg_prec prec, int B, double lambda, const
   const bool helm = lambda != 0.0;
   if (prec == DG_F64)
     return helm ? launch_t<N, double, true>(m, B, lambda, u, Au, st) : launch_t<N, double, false>(m, B, lambda, u, Au, st);
-  return helm ? launch_t<N, float, true>(m, B, lambda, u, Au, st) : launch_t<N, float, false>(m, B, lambda, u, Au, st);
+  if constexpr (N >= 9)  // wider tiles in registers there (apply_tile32.cu)
+    return launch_apply_tile32(m, N, B, lambda, static_cast<const float*>(u), static_cast<float*>(Au), st);
+  else
+    return helm ? launch_t<N, float, true>(m, B, lambda, u, Au, st) : launch_t<N, float, false>(m, B, lambda, u, Au, st);
 }
 
 }  // namespace

@@ -151,6 +151,9 @@ bool tensor_supported(int degree);  // the mma.sync tensor kernels (N <= 9)
 cudaError_t ensure_tensor_ops(dg_mesh* m, int degree, bool f64);
 bool tensor_ops_ready(int degree, bool f64);  // built on the current device (no build)
 cudaError_t tensor_pipe_error(int* flag);
+// the tile kernel's FP32 form of degrees 9 and 10 (apply_tile32.cu)
+cudaError_t launch_apply_tile32(const dg_mesh* m, int degree, int B, double lambda, const float* u, float* Au,
+                                cudaStream_t st);
 // FP32 apply on the tcgen05 tensor cores (apply_tc05.cu); needs 16-byte aligned u and Au
 bool tc05_usable(const void* u, const void* Au);
 cudaError_t launch_apply_tc05(dg_mesh* m, int degree, int B, double lambda, const float* u, float* Au,
