@@ -17,6 +17,7 @@
 #include <algorithm>
 
 #include "dg_internal.h"
+#include "fma2.cuh"
 
 namespace dgx {
 namespace {
@@ -48,47 +49,17 @@ struct Sz {
   static_assert(Np * kLdN <= 3 * Np * kLd + NFN * kLd, "the neighbours' values fit over u, w and F1");
 };
 
-__device__ __forceinline__ void load_g(float (&w)[kG], const float* p) {
-#pragma unroll
-  for (int q = 0; q < kG; q += 4) {
-    const float4 v = *reinterpret_cast<const float4*>(p + q);
-    w[q] = v.x, w[q + 1] = v.y, w[q + 2] = v.z, w[q + 3] = v.w;
-  }
-}
-// (x0, x1) += a (w0, w1), two lanes of the FP32 pipe in one instruction
-__device__ __forceinline__ void fma2(float& x0, float& x1, uint64_t a, float w0, float w1) {
-  uint64_t x, w;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(x0), "f"(x1));
-  asm("mov.b64 %0, {%1, %2};" : "=l"(w) : "f"(w0), "f"(w1));
-  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(x) : "l"(a), "l"(w));
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(x0), "=f"(x1) : "l"(x));
-}
-__device__ __forceinline__ uint64_t twice(float a) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(a));
-  return r;
-}
 // x[e] += a, y[e] += b times the values at p of a thread's elements
 __device__ __forceinline__ void fma_g(float (&x)[kG], float (&y)[kG], float a, float b, const float* p) {
   float w[kG];
-  load_g(w, p);
-  const uint64_t aa = twice(a), bb = twice(b);
-#pragma unroll
-  for (int e = 0; e < kG; e += 2) {
-    fma2(x[e], x[e + 1], aa, w[e], w[e + 1]);
-    fma2(y[e], y[e + 1], bb, w[e], w[e + 1]);
-  }
+  load_vec(w, p);
+  fma_vec(x, a, w);
+  fma_vec(y, b, w);
 }
 __device__ __forceinline__ void fma_g(float (&x)[kG], float a, const float* p) {
   float w[kG];
-  load_g(w, p);
-  const uint64_t aa = twice(a);
-#pragma unroll
-  for (int e = 0; e < kG; e += 2) fma2(x[e], x[e + 1], aa, w[e], w[e + 1]);
-}
-__device__ __forceinline__ void store_g(float* p, const float (&x)[kG]) {
-#pragma unroll
-  for (int q = 0; q < kG; q += 4) *reinterpret_cast<float4*>(p + q) = make_float4(x[q], x[q + 1], x[q + 2], x[q + 3]);
+  load_vec(w, p);
+  fma_vec(x, a, w);
 }
 
 template <int N, bool HELM>
@@ -232,8 +203,8 @@ __global__ void __launch_bounds__(Sz<N>::threads, 2)
         x[e] = grr * a[e] + grs * b[e];
         y[e] = grs * a[e] + gss * b[e];
       }
-      store_g(swr + i * kLd + g * kG, x);
-      store_g(sws + i * kLd + g * kG, y);
+      store_vec(swr + i * kLd + g * kG, x);
+      store_vec(sws + i * kLd + g * kG, y);
 #pragma unroll
       for (int f = 0; f < 3; ++f) {
         if (onf[f] < 0) continue;
@@ -242,7 +213,7 @@ __global__ void __launch_bounds__(Sz<N>::threads, 2)
           const int le = g * kG + e;
           x[e] = sg[(4 + 4 * f) * kE + le] * a[e] + sg[(5 + 4 * f) * kE + le] * b[e];
         }
-        store_g(sf + onf[f] * kLd + g * kG, x);
+        store_vec(sf + onf[f] * kLd + g * kG, x);
       }
     }
     __syncthreads();
@@ -320,7 +291,7 @@ __global__ void __launch_bounds__(Sz<N>::threads, 2)
         if (onf[f] >= 0) fma_g(acc, 1.f, sf + onf[f] * kLd + g * kG);
     }
     __syncthreads();
-    if (mine) store_g(swr + i * kLd + g * kG, acc);
+    if (mine) store_vec(swr + i * kLd + g * kG, acc);
     __syncthreads();
     float* o = Au + e0 * Np;
     for (int k = tid; k < ne * Np; k += T) {

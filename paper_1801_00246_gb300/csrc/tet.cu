@@ -39,6 +39,7 @@
 #include <vector>
 
 #include "dg_internal.h"
+#include "fma2.cuh"
 
 namespace dgx {
 namespace tet {
@@ -534,6 +535,328 @@ __global__ void __launch_bounds__(kTetThreads) tet_lift(int64_t K, int64_t nE, O
 }
 
 // ---------------------------------------------------------------------------
+// The same two kernels in FP32 at degrees 4 and 5, where the products dominate. What a
+// shared-memory read costs is the words it hands to the lanes, one address for all of
+// them or not: tet_lift's two elements per thread take about one word per multiply-add,
+// and shared memory delivers a quarter of what the FP32 pipe takes. Here a thread has
+// four rows of an operator and two elements (12 words for 32 multiply-adds in the mass
+// product, 18 for 24 in the last), in tet32_grad one row and eight elements of three
+// operators (11 for 24), two multiply-adds to an instruction. Fields are [node][element]
+// in shared memory; w passes between the kernels as [tile][3 Np][elements]; the traces
+// stay [element][face node], as neighbours read them. A block's elements are as many as
+// give each of its 128 threads one item; the operators leave room for 2 to 6 blocks per
+// SM. Helmholtz, N = 4, 58,956 elements: 219 -> 145 us; N = 5, 29,478: 203 -> 154 (eight
+// elements and one row throughout: 185 and 218; 256 threads with four: 231).
+// At degrees 1 to 3 the loads and barriers dominate and tet_grad / tet_lift stay
+// (N = 3, 29,478 elements: 42 us against 54).
+constexpr int kT32 = 128;
+constexpr int kG32 = 8;
+constexpr int kMaxTile32 = 64;
+template <int N>
+struct Tet32 {
+  static constexpr int Np = (N + 1) * (N + 2) * (N + 3) / 6, Nfp = (N + 1) * (N + 2) / 2, NF = 4 * Nfp;
+  static constexpr int fit = kT32 * kG32 / Np / kG32 * kG32;
+  static constexpr int E = fit < kMaxTile32 ? fit : kMaxTile32;  // elements per tile
+  static constexpr int P4 = (Np + 3) / 4 * 4, F4 = (Nfp + 3) / 4 * 4;  // operator rows in fours
+  static constexpr int LD = E + 4;               // row pitch: 16-byte rows, 4-way conflicts in the transposes
+  static constexpr int ZR = 3 * Np > 2 * NF ? 3 * Np : 2 * NF;
+  static constexpr int grad_words = (4 * Np + kGeo) * LD + E + 3 * Np * Np;
+  static constexpr int lift_words(bool helm) {
+    return ((helm ? 4 : 3) * Np + ZR + 2 * NF + kGeo) * LD + E + 4 * Np * P4 + 4 * Nfp * F4;
+  }
+  static_assert(Np * (E / kG32) <= kT32 && E % kG32 == 0 && E <= kT32, "one node item per thread");
+  static_assert(P4 / 4 * (E / 2) <= kT32, "one item of four nodes and two elements per thread");
+};
+
+// the tile's mesh elements (rows past the batch repeat the first) and their geometry [word][element]
+template <int E, int LD>
+__device__ __forceinline__ void tet32_geometry(int64_t e0, int nv, int64_t K, const float* __restrict__ geo, int* sel,
+                                               float* sg) {
+  if (threadIdx.x < E) sel[threadIdx.x] = int(tet_elem(e0, int(threadIdx.x) < nv ? int(threadIdx.x) : 0, K));
+  __syncthreads();
+#pragma unroll 4
+  for (int q = threadIdx.x; q < E * kGeo; q += kT32) {
+    const int g = q / kGeo, v = q - g * kGeo;
+    sg[v * LD + g] = __ldg(geo + int64_t(sel[g]) * kGeo + v);
+  }
+}
+
+template <int N>
+__global__ void __launch_bounds__(kT32) tet32_grad(int64_t K, int64_t nE, OpsLayout L, const float* __restrict__ ops,
+                                                   const int* __restrict__ fmask, const float* __restrict__ geo,
+                                                   const float* __restrict__ u, float* __restrict__ w,
+                                                   float2* __restrict__ tr) {
+  using D = Tet32<N>;
+  constexpr int Np = D::Np, NF = D::NF, E = D::E, LD = D::LD;
+  extern __shared__ __align__(16) unsigned char tet_smem[];
+  float* su = reinterpret_cast<float*>(tet_smem);  // [Np][LD]
+  float* sub = su + Np * LD;                       // [3 Np][LD]
+  float* sg = sub + 3 * Np * LD;                   // [kGeo][LD]
+  int* sel = reinterpret_cast<int*>(sg + kGeo * LD);
+  float* sDT = reinterpret_cast<float*>(sel + E);  // [3][m][i] = D_b[i][m]
+#pragma unroll
+  for (int b = 0; b < 3; ++b) {
+#pragma unroll 5
+    for (int r = threadIdx.x; r < Np * Np; r += kT32) {
+      const int i = r / Np, m = r - i * Np;
+      sDT[b * Np * Np + m * Np + i] = __ldg(ops + L.D[b] + r);
+    }
+  }
+  const int grp = threadIdx.x / Np, i = threadIdx.x - grp * Np, g0 = grp * kG32;
+  const bool mine = g0 < E;
+  const int64_t stride = int64_t(gridDim.x) * E, strideK = stride % K;
+  int64_t e0 = (int64_t(blockIdx.x) * E) % K;  // be0 mod K, advanced with be0
+  for (int64_t be0 = int64_t(blockIdx.x) * E; be0 < nE; be0 += stride, e0 = e0 + strideK < K ? e0 + strideK : e0 + strideK - K) {
+    const int nv = int(nE - be0 < E ? nE - be0 : E);
+    __syncthreads();
+#pragma unroll 8
+    for (int q = threadIdx.x; q < E * Np; q += kT32) {
+      const int g = q / Np;
+      su[(q - g * Np) * LD + g] = g < nv ? __ldg(u + be0 * Np + q) : 0.f;
+    }
+    tet32_geometry<E, LD>(e0, nv, K, geo, sel, sg);
+    __syncthreads();
+    if (mine) {
+      float a[3][kG32] = {};
+#pragma unroll 5
+      for (int m = 0; m < Np; ++m) {
+        float v[kG32];
+        dgx::load_vec(v, su + m * LD + g0);
+#pragma unroll
+        for (int b = 0; b < 3; ++b) dgx::fma_vec(a[b], sDT[b * Np * Np + m * Np + i], v);
+      }
+      float* wo = w + be0 * 3 * Np;  // the tile's [3 Np][E]
+      constexpr int kRow[3][3] = {{1, 2, 3}, {2, 4, 5}, {3, 5, 6}};  // G in the geometry words
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        float x[kG32];
+#pragma unroll
+        for (int e = 0; e < kG32; ++e) {
+          const float* G = sg + g0 + e;
+          x[e] = G[kRow[b][0] * LD] * a[0][e] + G[kRow[b][1] * LD] * a[1][e] + G[kRow[b][2] * LD] * a[2][e];
+        }
+        dgx::store_vec(sub + (b * Np + i) * LD + g0, a[b]);
+        dgx::store_vec(wo + (b * Np + i) * E + g0, x);
+      }
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int q = threadIdx.x; q < nv * NF; q += kT32) {
+      const int g = q / NF, fj = q - g * NF, f = fj / D::Nfp, k = __ldg(fmask + fj);
+      const float* nr = sg + (7 + 8 * f) * LD + g;
+      const float* ub = sub + k * LD + g;
+      tr[be0 * NF + q] = make_float2(su[k * LD + g], nr[0] * ub[0] + nr[LD] * ub[Np * LD] + nr[2 * LD] * ub[2 * Np * LD]);
+    }
+  }
+}
+
+template <int N, bool HELM>
+__global__ void __launch_bounds__(kT32, 3) tet32_lift(int64_t K, int64_t nE, OpsLayout L, const float* __restrict__ ops,
+                                                   const int* __restrict__ nfs, const float* __restrict__ geo,
+                                                   const int* __restrict__ conn, const int* __restrict__ mapJ,
+                                                   float lambda, const float* __restrict__ u,
+                                                   const float* __restrict__ w, const float2* __restrict__ tr,
+                                                   float* __restrict__ Au) {
+  using D = Tet32<N>;
+  constexpr int Np = D::Np, Nfp = D::Nfp, NF = D::NF, E = D::E, LD = D::LD, P4 = D::P4, F4 = D::F4;
+  extern __shared__ __align__(16) unsigned char tet_smem[];
+  float* sw = reinterpret_cast<float*>(tet_smem);  // [3 Np][LD]
+  float* sz = sw + 3 * Np * LD;                    // F1 and F2 [2 NF][LD], then z [3 Np][LD]
+  float* sJm = sz + D::ZR * LD;                    // [NF][LD]
+  float* sAv = sJm + NF * LD;                      // [NF][LD]: average + tau jump
+  float* sg = sAv + NF * LD;                       // [kGeo][LD]
+  float* su = sg + kGeo * LD;                      // [Np][LD]
+  int* sel = reinterpret_cast<int*>(su + (HELM ? Np * LD : 0));
+  float* sD = reinterpret_cast<float*>(sel + E);   // [3][m][P4] = D_b[m][i], zero past Np
+  float* sM = sD + 3 * Np * P4;                    // [m][P4]
+  float* sMf = sM + Np * P4;                       // [4][l][F4]
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {
+    const float* src = ops + (b < 3 ? L.D[b < 3 ? b : 0] : L.M);
+#pragma unroll 5
+    for (int q = threadIdx.x; q < Np * P4; q += kT32) {
+      const int m = q / P4, i = q - m * P4;
+      sD[b * Np * P4 + q] = i < Np ? __ldg(src + m * Np + i) : 0.f;
+    }
+  }
+#pragma unroll
+  for (int f = 0; f < 4; ++f)
+    for (int q = threadIdx.x; q < Nfp * F4; q += kT32) {
+      const int l = q / F4, j = q - l * F4;
+      sMf[f * Nfp * F4 + q] = j < Nfp ? __ldg(ops + L.Mf[f] + l * Nfp + j) : 0.f;
+    }
+  const int pair = threadIdx.x / (P4 / 4), i0 = 4 * (threadIdx.x - pair * (P4 / 4)), g0 = 2 * pair;
+  const bool mine = g0 < E;
+  const int64_t stride = int64_t(gridDim.x) * E, strideK = stride % K;
+  int64_t e0 = (int64_t(blockIdx.x) * E) % K;  // be0 mod K, advanced with be0
+  for (int64_t be0 = int64_t(blockIdx.x) * E; be0 < nE; be0 += stride, e0 = e0 + strideK < K ? e0 + strideK : e0 + strideK - K) {
+    const int nv = int(nE - be0 < E ? nE - be0 : E);
+    __syncthreads();
+    tet32_geometry<E, LD>(e0, nv, K, geo, sel, sg);
+    const float4* wi = reinterpret_cast<const float4*>(w + be0 * 3 * Np);
+#pragma unroll 5
+    for (int q = threadIdx.x; q < 3 * Np * E / 4; q += kT32) {
+      const int r = q / (E / 4);
+      *reinterpret_cast<float4*>(sw + r * LD + 4 * (q - r * (E / 4))) = __ldg(wi + q);
+    }
+    if (HELM) {
+#pragma unroll 8
+      for (int q = threadIdx.x; q < E * Np; q += kT32) {
+        const int g = q / Np;
+        su[(q - g * Np) * LD + g] = g < nv ? __ldg(u + be0 * Np + q) : 0.f;
+      }
+    }
+    constexpr int kB = 6;  // face nodes in flight per thread: their loads are a chain (neighbour, then its trace)
+    for (int q0 = threadIdx.x; q0 < E * NF; q0 += kB * kT32) {  // jumps and averages
+      int c[kB], mj[kB];
+      float2 own[kB], nb[kB];
+      float tau[kB];
+#pragma unroll
+      for (int t = 0; t < kB; ++t) {
+        const int q = q0 + t * kT32 < nv * NF ? q0 + t * kT32 : 0, g = q / NF, fj = q - g * NF, f = fj / Nfp;
+        const int64_t e = sel[g];
+        c[t] = __ldg(conn + 4 * e + f);
+        mj[t] = __ldg(mapJ + e * NF + fj);
+        own[t] = __ldg(tr + be0 * NF + q);
+        tau[t] = __ldg(geo + e * kGeo + 14 + 8 * f);
+      }
+#pragma unroll
+      for (int t = 0; t < kB; ++t) {
+        const int q = q0 + t * kT32 < nv * NF ? q0 + t * kT32 : 0, g = q / NF;
+        nb[t] = __ldg(tr + (c[t] >= 0 ? (be0 + g - sel[g] + c[t]) * NF + mj[t] : be0 * NF + q));
+      }
+#pragma unroll
+      for (int t = 0; t < kB; ++t) {
+        const int q = q0 + t * kT32, g = q / NF, fj = q - g * NF;
+        float jm = 0.f, av = 0.f;
+        if (c[t] >= 0) {
+          jm = nb[t].x - own[t].x;
+          av = 0.5f * (own[t].y - nb[t].y);  // the neighbour's trace carries its own (opposite) normal
+        } else if (c[t] == -2) {             // Dirichlet ghost: u+ = -u-, grad u+ = grad u-
+          jm = -2.f * own[t].x;
+          av = own[t].y;
+        }
+        if (q < E * NF) {  // (past the batch: any value of the tile, whose results are not stored)
+          sJm[fj * LD + g] = jm;
+          sAv[fj * LD + g] = av + tau[t] * jm;
+        }
+      }
+    }
+    __syncthreads();
+    constexpr int FR = F4 / 4;
+    for (int q = threadIdx.x; q < 4 * FR * (E / 2); q += kT32) {  // face-mass products: four rows, two elements
+      const int h0 = 2 * (q / (4 * FR)), r = q % (4 * FR), f = r / FR, j0 = 4 * (r - f * FR);
+      float m1[4][2] = {}, m2[4][2] = {};
+#pragma unroll 5
+      for (int l = 0; l < Nfp; ++l) {
+        float mf[4];
+        dgx::load_vec(mf, sMf + (f * Nfp + l) * F4 + j0);
+        const float2 a = *reinterpret_cast<const float2*>(sAv + (f * Nfp + l) * LD + h0);
+        const float2 b = *reinterpret_cast<const float2*>(sJm + (f * Nfp + l) * LD + h0);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const uint64_t mm = dgx::twice(mf[k]);
+          dgx::fma2(m1[k][0], m1[k][1], mm, a.x, a.y);
+          dgx::fma2(m2[k][0], m2[k][1], mm, b.x, b.y);
+        }
+      }
+      const float2 sJ = *reinterpret_cast<const float2*>(sg + (13 + 8 * f) * LD + h0);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (j0 + k >= Nfp) continue;
+        float* o = sz + (f * Nfp + j0 + k) * LD + h0;
+        *reinterpret_cast<float2*>(o) = make_float2(-sJ.x * m1[k][0], -sJ.y * m1[k][1]);
+        *reinterpret_cast<float2*>(o + NF * LD) = make_float2(0.5f * sJ.x * m2[k][0], 0.5f * sJ.y * m2[k][1]);
+      }
+    }
+    __syncthreads();
+    float z[3][4][2] = {}, extra[4][2] = {};
+    if (mine) {
+      float h[4][2] = {};
+#pragma unroll 5
+      for (int m = 0; m < Np; ++m) {
+        float mv[4];
+        dgx::load_vec(mv, sM + m * P4 + i0);
+        float2 v[4];
+#pragma unroll
+        for (int b = 0; b < 3; ++b) v[b] = *reinterpret_cast<const float2*>(sw + (b * Np + m) * LD + g0);
+        if (HELM) v[3] = *reinterpret_cast<const float2*>(su + m * LD + g0);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const uint64_t mm = dgx::twice(mv[k]);
+#pragma unroll
+          for (int b = 0; b < 3; ++b) dgx::fma2(z[b][k][0], z[b][k][1], mm, v[b].x, v[b].y);
+          if (HELM) dgx::fma2(h[k][0], h[k][1], mm, v[3].x, v[3].y);
+        }
+      }
+      const float2 J = *reinterpret_cast<const float2*>(sg + g0);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (i0 + k >= Np) continue;
+        float y[3][2] = {};
+#pragma unroll
+        for (int s = 0; s < 3; ++s) {
+          const int at = __ldg(nfs + 3 * (i0 + k) + s);  // face node at this node
+          if (at < 0) continue;
+          const float2 F1 = *reinterpret_cast<const float2*>(sz + at * LD + g0);
+          const float2 F2 = *reinterpret_cast<const float2*>(sz + (NF + at) * LD + g0);
+          const float* nr = sg + (7 + 8 * (at / Nfp)) * LD + g0;
+#pragma unroll
+          for (int b = 0; b < 3; ++b) {
+            y[b][0] += nr[b * LD] * F2.x;
+            y[b][1] += nr[b * LD + 1] * F2.y;
+          }
+          extra[k][0] += F1.x;
+          extra[k][1] += F1.y;
+        }
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+          z[b][k][0] = J.x * z[b][k][0] + y[b][0];
+          z[b][k][1] = J.y * z[b][k][1] + y[b][1];
+        }
+        if (HELM) {
+          extra[k][0] += lambda * J.x * h[k][0];
+          extra[k][1] += lambda * J.y * h[k][1];
+        }
+      }
+    }
+    __syncthreads();
+    if (mine) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (i0 + k >= Np) continue;
+#pragma unroll
+        for (int b = 0; b < 3; ++b)
+          *reinterpret_cast<float2*>(sz + (b * Np + i0 + k) * LD + g0) = make_float2(z[b][k][0], z[b][k][1]);
+      }
+    }
+    __syncthreads();
+    if (mine) {
+      float o[3][4][2] = {};
+#pragma unroll 5
+      for (int m = 0; m < Np; ++m) {
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+          float d[4];
+          dgx::load_vec(d, sD + (b * Np + m) * P4 + i0);
+          const float2 v = *reinterpret_cast<const float2*>(sz + (b * Np + m) * LD + g0);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) dgx::fma2(o[b][k][0], o[b][k][1], dgx::twice(d[k]), v.x, v.y);
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (i0 + k >= Np) continue;
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+          if (g0 + e < nv)
+            Au[(be0 + g0 + e) * Np + i0 + k] = (o[0][k][e] + o[1][k][e] + o[2][k][e]) + extra[k][e];
+      }
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
 // FP64 apply with its dense products on the tensor cores (exactly sliced FP64
 // GEMMs, out[r] = A X[r]): UB = [Dr; Ds; Dt] u, FM_f = diag(Mf_f, Mf_f) [avg +
 // tau jump | jump] per local face f, MW = M [J w_0; J w_1; J w_2; lambda J u] and
@@ -835,18 +1158,39 @@ struct TetKernelInfo {
 };
 
 template <typename Kern>
-cudaError_t tet_prepare(Kern k, size_t smem, TetKernelInfo& info, int dev, int* occ) {
+cudaError_t tet_prepare(Kern k, size_t smem, TetKernelInfo& info, int dev, int* occ, int threads = kTetThreads) {
   const uint64_t bit = uint64_t(1) << (dev & 63);
   if (!(info.ready.load() & bit)) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     int o = 0;
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k, kTetThreads, smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k, threads, smem);
     if (e != cudaSuccess) return e;
     info.occ.store(o > 0 ? o : 1);
     info.ready.fetch_or(bit);
   }
   *occ = info.occ.load();
   return cudaSuccess;
+}
+
+template <int N, bool HELM>
+cudaError_t tet32_apply_n(const dg_tet_mesh* m, int64_t nE, int dev, int sms, float lambda, const float* u, float* Au,
+                          float* w, float2* tr, cudaStream_t st) {
+  using D = Tet32<N>;
+  static TetKernelInfo info_g, info_l;
+  constexpr size_t sg = D::grad_words * sizeof(float), sl = D::lift_words(HELM) * sizeof(float);
+  int og = 1, ol = 1;
+  cudaError_t e = tet_prepare(tet32_grad<N>, sg, info_g, dev, &og, kT32);
+  if (e == cudaSuccess) e = tet_prepare(tet32_lift<N, HELM>, sl, info_l, dev, &ol, kT32);
+  if (e != cudaSuccess) return e;
+  const int64_t tiles = (nE + D::E - 1) / D::E;
+  const unsigned gg = unsigned(std::min<int64_t>(tiles, int64_t(sms) * og));
+  const unsigned gl = unsigned(std::min<int64_t>(tiles, int64_t(sms) * ol));
+  tet32_grad<N><<<gg, kT32, sg, st>>>(m->K, nE, m->L, m->ops32, m->fmask, m->geo32, u, w, tr);
+  note_launch();
+  tet32_lift<N, HELM><<<gl, kT32, sl, st>>>(m->K, nE, m->L, m->ops32, m->nfs, m->geo32, m->conn, m->mapJ, lambda, u, w,
+                                            tr, Au);
+  note_launch();
+  return cudaGetLastError();
 }
 
 template <typename T, int N, bool HELM>
@@ -862,6 +1206,13 @@ cudaError_t tet_apply_n(const dg_tet_mesh* m, int64_t nE, T lambda, const T* ops
   if (e != cudaSuccess) return e;
   // one resident wave of blocks, each loading the operators once and striding over element batches
   const int64_t batches = (nE + TetDims<N>::EB - 1) / TetDims<N>::EB;
+  if constexpr (sizeof(T) == 4 && N >= 4) {
+    // FP32 beyond one wave of tet_lift: the register-blocked form, whose tiles are larger and
+    // take longer each (one wave of them 35 us at N = 4, 39 at N = 5, one of tet_lift 28) but
+    // serve more elements: N = 4, 10,368 elements 58 -> 44 us; N = 5, 4,374 elements 52 -> 46.
+    if (batches > int64_t(sms) * ol)
+      return tet32_apply_n<N, HELM>(m, nE, dev, sms, lambda, u, Au, w, reinterpret_cast<float2*>(tr), st);
+  }
   const unsigned gg = unsigned(std::min<int64_t>(batches, int64_t(sms) * og));
   const unsigned gl = unsigned(std::min<int64_t>(batches, int64_t(sms) * ol));
   tet_grad<T, N><<<gg, kTetThreads, sg, st>>>(m->K, nE, m->L, ops, m->fmask, geo, u, w, tr);
@@ -938,7 +1289,9 @@ cudaError_t tet_apply_launch(const dg_tet_mesh* m, int B, double lambda, const T
   const T* ops = f64 ? reinterpret_cast<const T*>(m->ops64) : reinterpret_cast<const T*>(m->ops32);
   const T* geo = f64 ? reinterpret_cast<const T*>(m->geo64) : reinterpret_cast<const T*>(m->geo32);
   const int64_t nE = int64_t(B) * m->K;
-  const size_t need = size_t(nE) * size_t(3 * m->Np + 8 * m->Nfp) * sizeof(T);
+  // w, for FP32 in whole tiles (of at most kMaxTile32 elements), then the traces on 16 bytes
+  const size_t nW = (size_t(f64 ? nE : nE + kMaxTile32 - 1) * size_t(3 * m->Np) + 3) & ~size_t(3);
+  const size_t need = (nW + size_t(nE) * size_t(8 * m->Nfp)) * sizeof(T);
   if (m->ascr_bytes < need) {
     cudaFree(m->ascr);
     m->ascr = nullptr;
@@ -948,7 +1301,7 @@ cudaError_t tet_apply_launch(const dg_tet_mesh* m, int B, double lambda, const T
     m->ascr_bytes = need;
   }
   T* w = static_cast<T*>(m->ascr);
-  T* tr = w + nE * 3 * m->Np;
+  T* tr = w + nW;
   const T lam = T(lambda);
   const bool helm = lambda != 0.0;
   switch (m->N) {
