@@ -66,10 +66,15 @@ struct Tc {
   static constexpr int N2 = rup16(Np);  // output rows
   static constexpr int RQ = N2 / 4;     // output rows per thread of an element
   static constexpr int KQ = K1 / 2;     // u values per volume quarter in the gradient product's input
-  // tensor-memory columns of tc_apply
-  static constexpr int oA1 = 0, oD1 = K1, oAV = oD1 + N1, oAF = oAV + KYV, oDV = oAF + KYF, oDF = oDV + N2,
+  // tensor-memory columns of tc_apply (the volume columns of Y take the place of u's pieces,
+  // which the gradient product has read by then)
+  static constexpr int oA1 = 0, oAV = 0, oD1 = K1 > KYV ? K1 : KYV, oAF = oD1 + N1, oDV = oAF + KYF, oDF = oDV + N2,
                        TCOLS = oDF + N2;
   static_assert(TCOLS <= 512, "tensor memory");
+  // tc_apply blocks per SM: one tile's steps form a chain, so a second block runs in the
+  // first one's waits where half the tensor memory holds a tile's columns (N <= 5).
+  // 524,288 triangles with tc_face: N = 4 124 -> 94 us, N = 5 131 -> 102 us.
+  static constexpr int kPerSm = TCOLS <= 256 ? 2 : 1;
   static_assert(KQ % 8 == 0 || KQ % 4 == 0, "volume quarter input columns");
   // operator image (bytes): tc_apply part [B1 hi | B1 lo | BV hi | BV lo | BF2 hi | BF2 lo |
   // isc1 | iscV | iscF2], tc_face part [BF hi | BF lo | iscF]
@@ -362,7 +367,7 @@ __device__ __forceinline__ void face_quarter(float (&y)[YN], const float2* __res
 // accumulators, volume and face columns, each with its own scale, so each
 // pair issues its own products as soon as its columns are in tensor memory.
 template <int N, bool HELM>
-__global__ void __launch_bounds__(512, 1) tc_apply(int64_t K, int64_t nE, const float* __restrict__ gx,
+__global__ void __launch_bounds__(512, Tc<N>::kPerSm) tc_apply(int64_t K, int64_t nE, const float* __restrict__ gx,
                                                    const int32_t* __restrict__ conn,
                                                    const float2* __restrict__ FN, int64_t ldc,
                                                    const float* __restrict__ u, const uint8_t* __restrict__ opsA,
@@ -392,7 +397,7 @@ __global__ void __launch_bounds__(512, 1) tc_apply(int64_t K, int64_t nE, const 
     *abort_flag = 0;
     tc::mbar_init_fence();
   }
-  if (warp == 0) tc::tmem_alloc(slot, 512);
+  if (warp == 0) tc::tmem_alloc(slot, 512 / S::kPerSm);
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
@@ -638,7 +643,7 @@ __global__ void __launch_bounds__(512, 1) tc_apply(int64_t K, int64_t nE, const 
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
-  if (warp == 0) tc::tmem_dealloc(tb, 512);
+  if (warp == 0) tc::tmem_dealloc(tb, 512 / S::kPerSm);
 }
 
 // ------------------------------------------------------------------------- host side
@@ -778,7 +783,7 @@ cudaError_t launch_n(dg_mesh* m, int B, double lambda, const float* u, float* Au
       // memory (128 of 512 columns each)
       const int per = std::max(1, std::min(4, smem_sm / (S::smF + 1024)));
       grid_face[dev] = sms * per;
-      grid_apply[dev] = sms;
+      grid_apply[dev] = sms * S::kPerSm;
       o = built;
     }
     ops = &o;
