@@ -45,9 +45,9 @@ PMG_DEGREES = [8, 4, 2, 1]
 CHEB = 3           # Chebyshev-Jacobi smoothing degree per pre/post smoothing
 COARSE_PASSES = 1  # degree-1 coarse solve: one AMG-preconditioned CG pass (a scaled AMG V-cycle)
 # DRAM bytes per FP64 apply at N=8 from the latest ncu capture of the current
-# default kernels (tcgen05: gradient product 0.806 GB, face fill 0.938 GB, output
-# product 0.888 GB); None while the kernels differ from that capture
-TENSOR_APPLY_TRAFFIC = 2.632e9
+# default kernels (tcgen05: boundary derivatives 0.479 GB, output product 0.522 GB);
+# None while the kernels differ from that capture
+TENSOR_APPLY_TRAFFIC = 1.001e9
 
 
 # apply kernels by DG_KERNEL_* value
@@ -55,8 +55,8 @@ KERNEL_NAMES = {1: "tile (FP64/FP32 pipe)", 2: "gemm (FP32 register GEMMs)",
                 3: "tensor (mma.sync BF16 slice products: gradient product, then fused fill + output product)",
                 4: "ept (element per thread)", 5: "tensor_pipe",
                 6: "tc05 (tcgen05 FP16-piece products, tensor-memory operands: face kernel, then fused apply)",
-                7: "tc64 (tcgen05 exactly sliced FP64 products: gradient product, float-float pointwise stage, "
-                   "output product)"}
+                7: "tc64 (tcgen05 exactly sliced FP64 products: boundary derivatives, then pointwise stage in "
+                   "64-bit fixed point and output product)"}
 
 
 def peaks():
@@ -404,11 +404,12 @@ def run_ours(args, world, rank, local):
     value = job_gdofs(world, K, Np, ax_ms_max)
     fp64_ms = ax["poisson_f64"]["ms"]
     achieved = K * flops / (fp64_ms * 1e-3) / 1e9
-    # BF16 MMA flops the tensor-core FP64 apply issues per launch at N=8 (Poisson):
-    # 36 slice products x 2 flops x padded (rows x depth) of its two products (the
-    # tcgen05 kernel pads the depth to 32-column chunks, the mma.sync one to 16)
+    # 16-bit MMA flops the tensor-core FP64 apply issues per launch at N=8 (Poisson):
+    # slice products x 2 flops x padded (rows x depth) of its two products (tcgen05: 34
+    # FP16 products, boundary derivatives 64 x 48 and 5 chunks of 48 columns; mma.sync:
+    # 36 BF16 products, depth padded to 16)
     k64 = mesh.kernel(N, P.DG_F64, 0)
-    tc_flops = 36 * 2 * ((96 * 64 + 48 * 192) if k64 == P.KERNEL_TC64 else (96 * 48 + 48 * 176)) * K
+    tc_flops = 2 * (34 * (64 * 48 + 48 * 240) if k64 == P.KERNEL_TC64 else 36 * (96 * 48 + 48 * 176)) * K
     algo_gbs = K * bytes64 / (fp64_ms * 1e-3) / 1e9
     line = {
         "metric": METRIC, "value": value, "unit": "GDOF/s", "n_gpus": world, "steps": args.steps,
@@ -448,7 +449,7 @@ def run_ours(args, world, rank, local):
                      "peak_src": pk["hbm_src"] + " HBM copy bandwidth (MEASURED_PEAKS.json)",
                      "fp64_equiv_tflops": achieved / 1e3,
                      "fp64_pipe_peak_tflops": pk["fp64_gflops"] / 1e3,
-                     # the FP64 emulation's own work (BF16 slice products on padded tiles), kept
+                     # the FP64 emulation's own work (16-bit slice products on padded tiles), kept
                      # apart from frac: it is work the method does not need
                      "emulation_bf16_tflops": tc_flops / (fp64_ms * 1e-3) / 1e12,
                      "emulation_bf16_frac": tc_flops / (fp64_ms * 1e-3) / 1e12 / pk["bf16_tflops"]},

@@ -33,6 +33,8 @@
 // amplifies), and the digit products left out weigh 2^-60 of the largest. Against
 // 64-bit arithmetic the relative error of an apply is 0.9e-15 (N = 3) to 1.2e-14
 // (N = 10) on random fields, 1.5 times the FP64-pipe kernel's.
+// 524,288 triangles, N = 8: 1714 us and 2.6 GB of traffic with the pointwise stage
+// in float-float between two generic products and X in memory; 776 us and 1.0 GB now.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -128,7 +130,10 @@ struct TraceArgs {
 // columns each), so one block's slicing runs under the other's products. The
 // tile's rows arrive by one bulk copy into the space that then takes their
 // digits (each thread reads its values before the first digit is written), so
-// the row-major u is read with full sectors.
+// the row-major u is read with full sectors. 524,288 triangles, N = 8: 223 us (70
+// of it the 0.48 GB at the copy rate), bound by the slicing and the drain, whose
+// 64-bit integer work the two blocks overlap with each other's waits; the product
+// of all gradient rows that it replaces took 808 us.
 template <int KS>
 __global__ void __launch_bounds__(288, KS <= 3 ? 2 : 1) t64_trace(const TraceArgs a) {
   extern __shared__ __align__(1024) uint8_t sm[];
@@ -376,6 +381,12 @@ __host__ __device__ constexpr int out_smem(int nc) {
 // its neighbours' exponents, the coefficients at that scale and the shifts that
 // bring both sides of a face to a common one (done by every thread that forms
 // columns, this took a third of the kernel's instructions).
+// 524,288 triangles, N = 8: 539 us, in place of 234 (face terms) and 667 (product).
+// Nothing is near its limit: without the loads about 485, without the stores 495, without
+// the products 390, with none of them 275 and as an empty pipeline 170 us; a chunk's
+// forming, slicing and products follow each other and only two chunks fit in shared
+// memory. Handing over every 16 columns in place of a chunk gave 520 at N = 8 but
+// 6 % more at N = 5 and 9 % at N = 6.
 template <int NC>
 __global__ void __launch_bounds__(kOutThreads, 1) t64_output(const OutArgs a) {
   extern __shared__ __align__(1024) uint8_t sm[];

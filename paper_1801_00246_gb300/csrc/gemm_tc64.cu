@@ -60,6 +60,9 @@ __device__ int g_tc64_err;
 //  * warp 17 keeps a ring of operator blocks filled by bulk copies (loaded by
 //    warp 16 only when a chunk needed them, their latency was in every chunk:
 //    16,384 rows of 208 outputs, 45 deep, took 44 us).
+// Four products of a tetrahedral apply (196,608 elements, N = 3): 920 us with eight
+// 7-bit digits in BF16 (36 products, each its own instruction, and a float-float
+// recombination) -> 563 us, bound by the slicing and the drain of thin tiles.
 // No CTA-wide barrier in the steady state; every wait is bounded in time.
 constexpr int kSlicers = 512;  // threads of warps 0-15
 template <int NC, bool COLS>
