@@ -20,6 +20,7 @@
 // tensor cores, around an FP64 kernel for the fluxes at those points; U^n and
 // U^{n-1} are interpolated once a step, and once U^{n-1} has reached t^n both
 // history fields advance together (they meet the same Ubar at the same times).
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <string>
@@ -56,8 +57,13 @@ struct InsWorkspace {
   Tc64Op opI, opP[3];
   int npP = 0, colP[3] = {};  // projection blocks and their first columns in Y
   double* nrm = nullptr;      // [3][3][K]: per face n_x, n_y, sJ / J
-  // point values of U^n, U^{n-1} and the velocity data, and of the advected fields; fluxes; projection
-  double *WU = nullptr, *WG = nullptr, *gu = nullptr, *W = nullptr, *Y = nullptr, *R = nullptr;
+  // velocity-Dirichlet faces: 3 e + f of each, each face's place among them [3 K], and
+  // the velocity data at their points
+  int64_t nD = 0;
+  int32_t *dface = nullptr, *dslot = nullptr;
+  double* gd = nullptr;       // [n.U, U_x, U_y][nc][nD]
+  // point values of U^n and U^{n-1}, and of the advected fields; fluxes; projection
+  double *WU = nullptr, *W = nullptr, *Y = nullptr, *R = nullptr;
   // the advected fields U~ (two buffers, [2 fields][2][K][Np], or on the tensor cores
   // [Np][2 fields][2][K]) and their LSERK residual
   double *Ut0 = nullptr, *Ut1 = nullptr, *res = nullptr, *Uhat = nullptr, *Uhh = nullptr, *bu = nullptr,
@@ -478,7 +484,8 @@ cudaError_t launch_advect(const dg_mesh* m, InsWorkspace* w, const double* Un, c
 // interpolants of both, formed once a step and turned into what the fluxes take
 // (k_adv_metric): (U.grad r, U.grad s) at a volume point, (n.U, -) at a face point.
 // A face point's neighbour value is the neighbour's own interpolant at the
-// mirrored Gauss point (its n.U with the opposite sign).
+// mirrored Gauss point (its n.U with the opposite sign); on a velocity-Dirichlet face
+// it is the boundary datum, interpolated from that face's nodes alone (k_adv_data).
 // At 8,192 elements of degree 8 a stage took 280 us, 117 us of it this kernel's
 // predecessor, which interpolated the face values itself on the FP64 pipe (nine
 // nodes of four fields of both sides a point). Now the pipe, which still bounds it,
@@ -520,10 +527,9 @@ __global__ void k_adv_transpose(int Np, int64_t rows, int64_t ld, double* __rest
 }
 
 // In place on point values [MW][2][K] of a velocity: at volume points (u, v) ->
-// (u.grad r, u.grad s), at face points u -> n.u (v is kept: the boundary data need it,
-// and for them u goes to `keep` [3 nc][K]). The grid's second dimension is the point.
+// (u.grad r, u.grad s), at face points u -> n.u. The grid's second dimension is the point.
 __global__ void k_adv_metric(int Nc, int nc, int64_t K, const double* __restrict__ geo, const double* __restrict__ nrm,
-                             double* __restrict__ W, double* __restrict__ keep) {
+                             double* __restrict__ W) {
   const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   const int m = blockIdx.y;
   if (e >= K) return;
@@ -535,18 +541,40 @@ __global__ void k_adv_metric(int Nc, int nc, int64_t K, const double* __restrict
   } else {
     const int f = (m - Nc) / nc;
     w[0] = nrm[(3 * f + 0) * K + e] * u + nrm[(3 * f + 1) * K + e] * v;
-    if (keep) keep[int64_t(m - Nc) * K + e] = u;
   }
+}
+
+// The velocity data g [2][K][Np] at the points of the Dirichlet faces: gd
+// [n.U, U_x, U_y][nc][nD]. Reads the faces' own nodes only: the data are defined
+// there, the other nodes of g may hold anything.
+__global__ void k_adv_data(int N, int nc, int64_t K, int64_t nD, const int32_t* __restrict__ dface,
+                           const double* __restrict__ nrm, const double* __restrict__ I1, const double* __restrict__ g,
+                           double* __restrict__ gd) {
+  const int64_t d = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  const int k = blockIdx.y, Np = (N + 1) * (N + 2) / 2;
+  if (d >= nD) return;
+  const int64_t e = dface[d] / 3;
+  const int f = dface[d] - int(3 * e);
+  double u = 0.0, v = 0.0;
+  for (int a = 0; a <= N; ++a) {
+    const double c = I1[k * (N + 1) + a];
+    const int64_t i = e * Np + fnode_i(N, f, a);
+    u += c * g[i];
+    v += c * g[K * Np + i];
+  }
+  gd[k * nD + d] = nrm[3 * f * K + e] * u + nrm[(3 * f + 1) * K + e] * v;
+  gd[(nc + k) * nD + d] = u;
+  gd[(2 * nc + k) * nD + d] = v;
 }
 
 // NF advected fields at once: one thread per element and cubature point (the grid's
 // second dimension); ld: rows between W's and Y's columns
 template <int NF>
 __global__ void __launch_bounds__(256) k_adv_flux(int Nc, int nc, int64_t K, int64_t ld, const double* __restrict__ nrm,
-                                                  const int32_t* __restrict__ conn, const double* __restrict__ WU,
-                                                  const double* __restrict__ WG, const double* __restrict__ gu,
-                                                  double ca, double cb, const double* __restrict__ W,
-                                                  double* __restrict__ Y) {
+                                                  const int32_t* __restrict__ conn, const int32_t* __restrict__ dslot,
+                                                  int64_t nD, const double* __restrict__ gd,
+                                                  const double* __restrict__ WU, double ca, double cb,
+                                                  const double* __restrict__ W, double* __restrict__ Y) {
   const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   const int m = blockIdx.y;
   if (e >= K) return;
@@ -573,15 +601,15 @@ __global__ void __launch_bounds__(256) k_adv_flux(int Nc, int nc, int64_t K, int
     const bool data = code == -2;  // velocity Dirichlet: exterior state is the boundary datum (Neumann: the interior)
     const int64_t en = code >= 0 ? code >> 2 : e;
     const int mn = code >= 0 ? Nc + (code & 3) * nc + (nc - 1 - k) : m;
+    const double* g = gd + (data ? k * nD + __ldg(dslot + 3 * e + f) : 0);
     const double unm = ubar(2 * K * m + e);
-    const double unp = data ? __ldg(WG + 2 * K * m + e) : (code >= 0 ? -ubar(2 * K * mn + en) : unm);
+    const double unp = data ? __ldg(g) : (code >= 0 ? -ubar(2 * K * mn + en) : unm);
     const double sh = 0.5 * __ldg(nrm + (3 * f + 2) * K + e);
     // F* = (n.u- w- + n.u+ w+) / 2 + lam (w- - w+) / 2
     const double lam = fmax(fabs(unm), fabs(unp)), fm = sh * (unm + lam), fp = sh * (unp - lam);
 #pragma unroll
     for (int c = 0; c < 2 * NF; ++c) {
-      const double wp = data ? ((c & 1) ? __ldg(WG + 2 * K * m + K + e) : __ldg(gu + int64_t(q) * K + e))
-                             : __ldg(W + mn * ld + c * K + en);
+      const double wp = data ? __ldg(g + (1 + (c & 1)) * nc * nD) : __ldg(W + mn * ld + c * K + en);
       Y[(2 * Nc + q) * ld + c * K + e] = fm * w[c] + fp * wp;
     }
   }
@@ -666,8 +694,21 @@ cudaError_t setup_ins(dg_mesh* m) {
     const size_t nw = size_t(m->K) * MW;
     ICK(al(&w->nrm, 9 * size_t(m->K)));
     ICK(al(&w->WU, 4 * nw));
-    ICK(al(&w->WG, 2 * nw));
-    ICK(al(&w->gu, 3 * size_t(nc) * m->K));
+    std::vector<int32_t> face, slot(3 * size_t(m->K), -1);
+    for (size_t i = 0; i < slot.size(); ++i)
+      if (m->conn_h[i] == -2) {
+        slot[i] = int32_t(face.size());
+        face.push_back(int32_t(i));
+      }
+    w->nD = int64_t(face.size());
+    auto put = [&](int32_t** d, const std::vector<int32_t>& v) -> cudaError_t {
+      cudaError_t e = cudaMalloc(reinterpret_cast<void**>(d), std::max<size_t>(v.size(), 1) * sizeof(int32_t));
+      if (e == cudaSuccess) w->allocs.push_back(*d);
+      return e == cudaSuccess ? cudaMemcpy(*d, v.data(), v.size() * sizeof(int32_t), cudaMemcpyHostToDevice) : e;
+    };
+    ICK(put(&w->dface, face));
+    ICK(put(&w->dslot, slot));
+    ICK(al(&w->gd, 3 * size_t(nc) * std::max<size_t>(face.size(), 1)));
     ICK(al(&w->W, 4 * nw));
     ICK(al(&w->Y, 4 * size_t(m->K) * KY));
     ICK(al(&w->R, 4 * n1));
@@ -679,12 +720,22 @@ cudaError_t setup_ins(dg_mesh* m) {
   return cudaSuccess;
 }
 
-// A velocity field's point values in the form the fluxes take (keep: see k_adv_metric).
-cudaError_t point_values(const dg_mesh* m, InsWorkspace* w, const double* u, double* W, double* keep, cudaStream_t st) {
+// A velocity field's point values in the form the fluxes take.
+cudaError_t point_values(const dg_mesh* m, InsWorkspace* w, const double* u, double* W, cudaStream_t st) {
   const AdvLayout& L = w->L;
   ICK(tc64_gemm_launch(w->opI, 2 * m->K, u, L.Np, W, 2 * m->K, st, 0, nullptr, 0, 1));
   k_adv_metric<<<dim3(unsigned((m->K + 255) / 256), unsigned(w->opI.M)), 256, 0, st>>>(L.Nc, L.nc, m->K, m->geo64, w->nrm,
-                                                                                  W, keep);
+                                                                                  W);
+  note_launch();
+  return cudaGetLastError();
+}
+
+// The velocity data at the points of the Dirichlet faces.
+cudaError_t boundary_values(const dg_mesh* m, InsWorkspace* w, const double* g, cudaStream_t st) {
+  if (w->nD == 0) return cudaSuccess;
+  const AdvLayout& L = w->L;
+  k_adv_data<<<dim3(unsigned((w->nD + 127) / 128), unsigned(L.nc)), 128, 0, st>>>(m->N, L.nc, m->K, w->nD, w->dface, w->nrm,
+                                                                              w->ops + L.I1, g, w->gd);
   note_launch();
   return cudaGetLastError();
 }
@@ -697,8 +748,10 @@ cudaError_t advect_stage_tensor(const dg_mesh* m, InsWorkspace* w, int nf, doubl
   const int64_t K = m->K, rows = 2 * K * nf, ld = 4 * K;
   ICK(tc64_gemm_launch(w->opI, rows, Ut_in, ld, w->W, ld, st, 0, nullptr, 1, 1));
   const dim3 g(unsigned((K + 255) / 256), unsigned(MW));
-  if (nf == 1) k_adv_flux<1><<<g, 256, 0, st>>>(Nc, nc, K, ld, w->nrm, m->conn, w->WU, w->WG, w->gu, ca, cb, w->W, w->Y);
-  else k_adv_flux<2><<<g, 256, 0, st>>>(Nc, nc, K, ld, w->nrm, m->conn, w->WU, w->WG, w->gu, ca, cb, w->W, w->Y);
+  auto flux = [&](auto kernel) {
+    kernel<<<g, 256, 0, st>>>(Nc, nc, K, ld, w->nrm, m->conn, w->dslot, w->nD, w->gd, w->WU, ca, cb, w->W, w->Y);
+  };
+  nf == 1 ? flux(k_adv_flux<1>) : flux(k_adv_flux<2>);
   note_launch();
   for (int p = 0; p < w->npP; ++p)
     ICK(tc64_gemm_launch(w->opP[p], rows, w->Y + w->colP[p] * ld, ld, w->R, ld, st, p > 0, nullptr, 1, 1));
@@ -739,7 +792,7 @@ cudaError_t advect_substeps(const dg_mesh* m, InsWorkspace* w, const dg_ins_stat
           note_launch();
         }
         g = w->gts;
-        if (w->tensor) ICK(point_values(m, w, g, w->WG, w->gu, st));
+        if (w->tensor) ICK(boundary_values(m, w, g, st));
       }
       if (w->tensor) {
         ICK(advect_stage_tensor(m, w, nf, ca, cb, *cur, nxt, kRkA[stg], kRkB[stg], dts, st));
@@ -763,9 +816,9 @@ cudaError_t advect_history(const dg_mesh* m, InsWorkspace* w, const dg_ins_state
   const bool first = s->step == 0;
   if (w->tensor) {
     const size_t nw = 2 * size_t(m->K) * w->opI.M;
-    ICK(point_values(m, w, s->U, w->WU, nullptr, st));
-    if (!first) ICK(point_values(m, w, s->Uold, w->WU + nw, nullptr, st));
-    if (!s->gU_hist) ICK(point_values(m, w, s->gU, w->WG, w->gu, st));
+    ICK(point_values(m, w, s->U, w->WU, st));
+    if (!first) ICK(point_values(m, w, s->Uold, w->WU + nw, st));
+    if (!s->gU_hist) ICK(boundary_values(m, w, s->gU, st));
   }
   ICK(cudaMemsetAsync(w->res, 0, 2 * bytes, st));
   double* cur = w->Ut0;
