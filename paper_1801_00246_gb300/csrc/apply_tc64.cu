@@ -42,6 +42,7 @@
 
 #include "dg_internal.h"
 #include "fix64.cuh"
+#include "tables64.h"
 #include "tc05.cuh"
 
 namespace dgx {
@@ -570,7 +571,7 @@ __global__ void __launch_bounds__(kOutThreads, 1) t64_output(const OutArgs a) {
 #pragma unroll
             for (int c = 0; c < 4; ++c)
               if (col + c < a.M) {
-                const double v = fx::to_double(fx::from_sums(acc[c]), __ldg(a.ea + col + c) + E - 56);
+                const double v = fx::sums_to_double(acc[c], __ldg(a.ea + col + c) + E - 56);
                 o[c] = E == kBadScale ? fx::double_of(0x7ff8000000000000ll) : v;
               }
           }
@@ -697,23 +698,21 @@ __global__ void __launch_bounds__(kOutThreads, 1) t64_output(const OutArgs a) {
 }
 
 // ------------------------------------------------------------------ host side
-// An operator block image: rows scaled to integers below 2^56 (one exponent
-// per row, or one for all), cut into digits (fix64.cuh), digit i of row r at
-// stacked row i nc + r, in 16-column steps of the canonical layout.
-// A(r, k) for r < M <= nc, k < K (columns past K are zero; K a multiple of 16 on
-// the way out), ea[r] the row exponents to use.
+// An operator block image: the integers A(r, k) (a row's entries 2^{56 - its exponent}),
+// r < M <= nc, k < K, cut into digits (fix64.cuh), digit i of row r at stacked row
+// i nc + r, in 16-column steps of the canonical layout (columns past K are zero).
 template <typename F>
-void slice_block(const F& A, int M, int nc, int K, const int* ea, std::vector<uint8_t>& img) {
+void slice_block(const F& A, int M, int nc, int K, std::vector<uint8_t>& img) {
   const int steps = (K + 15) / 16;
   const size_t step_bytes = size_t(kDigits) * nc * 32;
   const size_t base = img.size();
   img.resize(base + steps * step_bytes, 0);
   for (int r = 0; r < M; ++r)
     for (int k = 0; k < K; ++k) {
-      const double v = A(r, k);
-      if (v == 0.0) continue;
+      const long long x = A(r, k);
+      if (x == 0) continue;
       int d[kDigits];
-      fx::digits_of(v, ea[r], d);
+      fx::digits_of(x, d);
       uint8_t* blk = img.data() + base + size_t(k / 16) * step_bytes;
       for (int i = 0; i < kDigits; ++i) {
         const int R = i * nc + r, c = k % 16;
@@ -745,14 +744,9 @@ cudaError_t upload(const void* p, size_t n, void** d) {
   if (e == cudaSuccess) e = cudaMemcpy(*d, p, n, cudaMemcpyHostToDevice);
   return e;
 }
-int floor_log2(double x) {
-  int e = 0;
-  std::frexp(x, &e);
-  return e - 1;
-}
 
 cudaError_t build_t64(const RefElem& R, Tc64Apply& o) {
-  const int N = R.N, Np = R.Np, Nfp = R.Nfp, nface = 3 * Nfp;
+  const int N = R.N, Np = R.Np;
   // boundary derivatives: rows 2b, 2b + 1 = d/dr, d/ds at the b-th node counter-clockwise
   auto trace = [&](int r, int k) {
     const int b = r / 2, n = face_node(N, b / N, b % N);
@@ -771,88 +765,32 @@ cudaError_t build_t64(const RefElem& R, Tc64Apply& o) {
   o.passes = (6 * N + kTraceN - 1) / kTraceN;
   o.ks = (Np + 15) / 16;
   std::vector<uint8_t> img;
-  const std::vector<int> eat(kTraceN, o.trace_ea);
   for (int p = 0; p < o.passes; ++p)
-    slice_block([&](int r, int k) { return k < Np ? trace(p * kTraceN + r, k) : 0.0; },
-                std::min(kTraceN, 6 * N - p * kTraceN), kTraceN, 16 * o.ks, eat.data(), img);
+    slice_block([&](int r, int k) { return k < Np ? std::llround(std::ldexp(trace(p * kTraceN + r, k), 56 - o.trace_ea)) : 0ll; },
+                std::min(kTraceN, 6 * N - p * kTraceN), kTraceN, 16 * o.ks, img);
   cudaError_t e = upload(img.data(), img.size(), reinterpret_cast<void**>(&o.trace));
-  // the output operator, its three volume blocks in extended precision
-  std::vector<double> S[3], Df[2], Ef(size_t(Np) * nface, 0.0);
-  for (auto& s : S) s.assign(size_t(Np) * Np, 0.0);
-  for (auto& d : Df) d.assign(size_t(Np) * nface, 0.0);
-  double ms = 0.0, md = 0.0, me = 0.0, mm = 0.0;
-  for (int i = 0; i < Np; ++i) {
-    for (int n = 0; n < Np; ++n) {
-      long double rr = 0, rs = 0, ss = 0;
-      for (int k = 0; k < Np; ++k) {
-        const long double br = R.Br[size_t(i) * Np + k], bs = R.Bs[size_t(i) * Np + k];
-        const long double dr = R.Dr[size_t(k) * Np + n], ds = R.Ds[size_t(k) * Np + n];
-        rr += br * dr;
-        rs += br * ds + bs * dr;
-        ss += bs * ds;
-      }
-      S[0][size_t(i) * Np + n] = double(rr);
-      S[1][size_t(i) * Np + n] = double(rs);
-      S[2][size_t(i) * Np + n] = double(ss);
-      for (const auto& s : S) ms = std::max(ms, std::fabs(s[size_t(i) * Np + n]));
-      mm = std::max(mm, std::fabs(R.M[size_t(i) * Np + n]));
-    }
-    for (int f = 0; f < 3; ++f)
-      for (int l = 0; l < Nfp; ++l) {
-        double dr = 0.0, ds = 0.0, ef = 0.0;
-        for (int j = 0; j < Nfp; ++j) {
-          const int k = face_node(N, f, j);
-          const double mf = R.Mf[size_t(j) * Nfp + l];
-          dr += R.Dr[size_t(k) * Np + i] * mf;
-          ds += R.Ds[size_t(k) * Np + i] * mf;
-          if (k == i) ef += mf;
-        }
-        Df[0][size_t(i) * nface + f * Nfp + l] = dr;
-        Df[1][size_t(i) * nface + f * Nfp + l] = ds;
-        Ef[size_t(i) * nface + f * Nfp + l] = ef;
-        md = std::max(md, std::max(std::fabs(dr), std::fabs(ds)));
-        me = std::max(me, std::fabs(ef));
-      }
-  }
-  // powers of two that bring every block's largest entry to the volume block's
-  o.k1 = floor_log2(ms / me);
-  o.k2 = floor_log2(ms / md);
-  o.km = floor_log2(ms / mm);
+  OutTable tables[2];
+  build_out_tables(R, tables);
   for (int helm = 0; helm < 2; ++helm) {
     OutSet& w = o.out[helm];
-    w.gvol = (Np + 7) / 8;
-    w.gface = w.gvol + (nface + 7) / 8;
-    w.chunks = (w.gface + (helm ? (Np + 23) / 24 : 0) + 1) / 2;
+    const OutTable& t = tables[helm];
+    o.k1 = t.k1;
+    o.k2 = t.k2;
+    o.km = t.km;
+    w.gvol = t.gvol;
+    w.gface = t.gface;
+    w.chunks = t.chunks;
     w.parts = Np > 64 ? 2 : 1;
     const int M = (Np + w.parts - 1) / w.parts;
     w.nc = (M + 15) & ~15;
-    auto entry = [&](int i, int k) -> double {  // column k = (3 chunk + kind) 16 + item of the chunk
-      const int c = (k / 16) % 3, g = k / 48 * 2 + k % 16 / 8, t = k % 8;
-      if (g < w.gvol) return 8 * g + t < Np ? S[c][size_t(i) * Np + 8 * g + t] : 0.0;
-      if (g < w.gface) {
-        const int l = 8 * (g - w.gvol) + t;
-        if (l >= nface) return 0.0;
-        const size_t at = size_t(i) * nface + l;
-        return c == 2 ? std::ldexp(Ef[at], o.k1) : std::ldexp(Df[c][at], o.k2);
-      }
-      const int n = 24 * (g - w.gface) + 3 * t + c;
-      return helm && n < Np ? std::ldexp(R.M[size_t(i) * Np + n], o.km) : 0.0;
-    };
     for (int q = 0; q < w.parts; ++q) {
       OutOp& p = w.part[q];
       p.c0 = q * M;
       p.M = std::min(M, Np - p.c0);
       std::vector<int> ea(w.nc, 0);
-      for (int r = 0; r < p.M; ++r) {
-        double m = 0.0, s = 0.0;
-        for (int k = 0; k < 48 * w.chunks; ++k) {
-          m = std::max(m, std::fabs(entry(p.c0 + r, k)));
-          s += std::fabs(entry(p.c0 + r, k));
-        }
-        ea[r] = fx::row_exp(m, s);
-      }
+      std::copy(t.ea.begin() + p.c0, t.ea.begin() + p.c0 + p.M, ea.begin());
       std::vector<uint8_t> im;
-      slice_block([&](int r, int k) { return entry(p.c0 + r, k); }, p.M, w.nc, 48 * w.chunks, ea.data(), im);
+      slice_block([&](int r, int k) { return t.x[size_t(p.c0 + r) * t.cols + k]; }, p.M, w.nc, t.cols, im);
       if (e == cudaSuccess) e = upload(im.data(), im.size(), reinterpret_cast<void**>(&p.ops));
       if (e == cudaSuccess) e = upload(ea.data(), ea.size() * sizeof(int), reinterpret_cast<void**>(&p.ea));
     }

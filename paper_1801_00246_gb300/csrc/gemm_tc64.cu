@@ -318,7 +318,7 @@ cudaError_t tc64_op_create(const std::vector<double>& A, int M, int K, Tc64Op* o
       const double v = A[size_t(r) * K + k];
       if (v == 0.0 || !std::isfinite(v)) continue;
       int d[kDigits];
-      fx::digits_of(v, ea[r], d);
+      fx::digits_of(std::llround(std::ldexp(v, 56 - ea[r])), d);
       for (int i = 0; i < 4; ++i) l1d[i] += std::abs(d[i]);
       uint8_t* blk = img.data() + size_t(r / nc * op->KCH + k / kKC) * bytes;
       for (int i = 0; i < kDigits; ++i) {
