@@ -701,18 +701,21 @@ __global__ void __launch_bounds__(kOutThreads, 1) t64_output(const OutArgs a) {
 // An operator block image: the integers A(r, k) (a row's entries 2^{56 - its exponent}),
 // r < M <= nc, k < K, cut into digits (fix64.cuh), digit i of row r at stacked row
 // i nc + r, in 16-column steps of the canonical layout (columns past K are zero).
+// False if a row's digit sums could leave the integers that FP32 holds.
 template <typename F>
-void slice_block(const F& A, int M, int nc, int K, std::vector<uint8_t>& img) {
+bool slice_block(const F& A, int M, int nc, int K, std::vector<uint8_t>& img) {
   const int steps = (K + 15) / 16;
   const size_t step_bytes = size_t(kDigits) * nc * 32;
   const size_t base = img.size();
   img.resize(base + steps * step_bytes, 0);
-  for (int r = 0; r < M; ++r)
+  for (int r = 0; r < M; ++r) {
+    fx::ExactSums sums;
     for (int k = 0; k < K; ++k) {
       const long long x = A(r, k);
       if (x == 0) continue;
       int d[kDigits];
       fx::digits_of(x, d);
+      sums.add(d);
       uint8_t* blk = img.data() + base + size_t(k / 16) * step_bytes;
       for (int i = 0; i < kDigits; ++i) {
         const int R = i * nc + r, c = k % 16;
@@ -720,6 +723,9 @@ void slice_block(const F& A, int M, int nc, int K, std::vector<uint8_t>& img) {
         std::memcpy(blk + size_t(R / 8) * 256 + (c / 8) * 128 + (R % 8) * 16 + (c % 8) * 2, &h, 2);
       }
     }
+    if (!sums.exact()) return false;
+  }
+  return true;
 }
 
 struct OutOp {
@@ -765,10 +771,12 @@ cudaError_t build_t64(const RefElem& R, Tc64Apply& o) {
   o.passes = (6 * N + kTraceN - 1) / kTraceN;
   o.ks = (Np + 15) / 16;
   std::vector<uint8_t> img;
+  bool exact = true;
   for (int p = 0; p < o.passes; ++p)
-    slice_block([&](int r, int k) { return k < Np ? std::llround(std::ldexp(trace(p * kTraceN + r, k), 56 - o.trace_ea)) : 0ll; },
-                std::min(kTraceN, 6 * N - p * kTraceN), kTraceN, 16 * o.ks, img);
-  cudaError_t e = upload(img.data(), img.size(), reinterpret_cast<void**>(&o.trace));
+    exact &= slice_block([&](int r, int k) { return k < Np ? std::llround(std::ldexp(trace(p * kTraceN + r, k), 56 - o.trace_ea)) : 0ll; },
+                         std::min(kTraceN, 6 * N - p * kTraceN), kTraceN, 16 * o.ks, img);
+  cudaError_t e = exact ? cudaSuccess : cudaErrorInvalidValue;
+  if (exact) e = upload(img.data(), img.size(), reinterpret_cast<void**>(&o.trace));
   OutTable tables[2];
   build_out_tables(R, tables);
   for (int helm = 0; helm < 2; ++helm) {
@@ -790,7 +798,8 @@ cudaError_t build_t64(const RefElem& R, Tc64Apply& o) {
       std::vector<int> ea(w.nc, 0);
       std::copy(t.ea.begin() + p.c0, t.ea.begin() + p.c0 + p.M, ea.begin());
       std::vector<uint8_t> im;
-      slice_block([&](int r, int k) { return t.x[size_t(p.c0 + r) * t.cols + k]; }, p.M, w.nc, t.cols, im);
+      if (!slice_block([&](int r, int k) { return t.x[size_t(p.c0 + r) * t.cols + k]; }, p.M, w.nc, t.cols, im))
+        return cudaErrorInvalidValue;
       if (e == cudaSuccess) e = upload(im.data(), im.size(), reinterpret_cast<void**>(&p.ops));
       if (e == cudaSuccess) e = upload(ea.data(), ea.size() * sizeof(int), reinterpret_cast<void**>(&p.ea));
     }

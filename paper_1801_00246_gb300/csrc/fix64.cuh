@@ -258,5 +258,26 @@ inline void digits_of(long long x, int (&out)[kDigits]) {
   }
 }
 
+// An operator row's digits, for the bound on its products' digit sums. Sums 0 .. 4
+// have to be integers below 2^24, which FP32 holds exactly, whatever the data (whose
+// leading digit is at most 257 in size, the others 128). Sum 5 weighs one unit of the
+// result, 2^-56 of its bound, 6 and 7 less: where digits of one sign in every place take
+// them past 2^24 (1.12 of it at degree 9, 1.28 at degree 10) a step's rounding is one
+// unit of the result or less.
+struct ExactSums {
+  double l1[5] = {};
+  void add(const int (&d)[kDigits]) {
+    for (int i = 0; i < 5; ++i) l1[i] += d[i] < 0 ? -d[i] : d[i];
+  }
+  bool exact() const {
+    for (int s = 0; s < 5; ++s) {
+      double most = 257.0 * l1[s];
+      for (int i = 0; i < s; ++i) most += 128.0 * l1[i];
+      if (most >= 16777216.0) return false;
+    }
+    return true;
+  }
+};
+
 }  // namespace fx
 }  // namespace dgx

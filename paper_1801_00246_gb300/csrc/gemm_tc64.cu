@@ -296,7 +296,7 @@ cudaError_t allow_smem() {
 }  // namespace
 
 // A (M x K, row-major FP64) into the block layout of tc64_gemm; cudaErrorInvalidValue if
-// its sums are too long to stay exact (beyond some 400 terms).
+// its sums are too long to stay exact (beyond some 350 terms).
 cudaError_t tc64_op_create(const std::vector<double>& A, int M, int K, Tc64Op* op) {
   op->M = M;
   op->K = K;
@@ -313,13 +313,13 @@ cudaError_t tc64_op_create(const std::vector<double>& A, int M, int K, Tc64Op* o
       l1 += std::fabs(A[size_t(r) * K + k]);
     }
     ea[r] = fx::row_exp(mx, l1);
-    double l1d[4] = {};  // absolute sums of the row's four leading digits
+    fx::ExactSums sums;
     for (int k = 0; k < K; ++k) {
       const double v = A[size_t(r) * K + k];
       if (v == 0.0 || !std::isfinite(v)) continue;
       int d[kDigits];
       fx::digits_of(std::llround(std::ldexp(v, 56 - ea[r])), d);
-      for (int i = 0; i < 4; ++i) l1d[i] += std::abs(d[i]);
+      sums.add(d);
       uint8_t* blk = img.data() + size_t(r / nc * op->KCH + k / kKC) * bytes;
       for (int i = 0; i < kDigits; ++i) {
         const int R = i * nc + r % nc, c = k % kKC;
@@ -328,13 +328,7 @@ cudaError_t tc64_op_create(const std::vector<double>& A, int M, int K, Tc64Op* o
                     &h, 2);
       }
     }
-    // The sums that carry the result (s <= 3) have to stay integers below 2^24, which
-    // FP32 holds exactly, whatever the data: its leading digit is at most 257, the others 128.
-    for (int s4 = 0; s4 < 4; ++s4) {
-      double most = 257.0 * l1d[s4];
-      for (int i = 0; i < s4; ++i) most += 128.0 * l1d[i];
-      if (most >= 16777216.0) return cudaErrorInvalidValue;
-    }
+    if (!sums.exact()) return cudaErrorInvalidValue;
   }
   cudaError_t e = cudaMalloc(&op->blocks, img.size());
   if (e == cudaSuccess) e = cudaMemcpy(op->blocks, img.data(), img.size(), cudaMemcpyHostToDevice);

@@ -52,7 +52,7 @@ struct InsWorkspace {
   double* ops = nullptr;
   // tensor-core advection (degree >= 3): interpolation to the Nc volume and 3 nc
   // face cubature points, and the projection [Pr Ps -Lc] as one sliced operator, or
-  // as its three blocks where a sum over all of them would not be exact
+  // as two (N >= 9) where a sum over all columns would not be exact
   bool tensor = false;
   Tc64Op opI, opP[3];
   int npP = 0, colP[3] = {};  // projection blocks and their first columns in Y
@@ -676,21 +676,24 @@ cudaError_t setup_ins(dg_mesh* m) {
                                        : (k < 2 * Nc ? h[L.Ps + size_t(i) * Nc + k - Nc]
                                                      : -h[L.Lc + size_t(i) * 3 * nc + k - 2 * Nc]);
     ICK(tc64_op_create(I, MW, Np, &w->opI));
-    const cudaError_t one = tc64_op_create(P, Np, KY, &w->opP[0]);
-    w->npP = 1;
-    if (one != cudaSuccess) {  // too deep for exact sums: block by block
-      if (one != cudaErrorInvalidValue) return one;
-      const int col[4] = {0, Nc, 2 * Nc, KY};
-      w->npP = 3;
-      for (int b = 0; b < 3; ++b) {
-        const int n = col[b + 1] - col[b];
+    // the fewest blocks of columns whose sums stay exact: one up to N = 8 (whose fifth
+    // sum reaches 0.99 of the limit), two at N = 9 and 10
+    cudaError_t made = cudaErrorInvalidValue;
+    for (int blocks = 1; blocks <= 3 && made == cudaErrorInvalidValue; ++blocks) {
+      for (Tc64Op& op : w->opP) tc64_op_free(&op);
+      const int width = ((KY + blocks - 1) / blocks + 31) & ~31;
+      made = cudaSuccess;
+      w->npP = blocks;
+      for (int b = 0; b < blocks && made == cudaSuccess; ++b) {
+        const int c0 = b * width, n = std::min(width, KY - c0);
         std::vector<double> Pb(size_t(Np) * n);
         for (int i = 0; i < Np; ++i)
-          for (int k = 0; k < n; ++k) Pb[size_t(i) * n + k] = P[size_t(i) * KY + col[b] + k];
-        ICK(tc64_op_create(Pb, Np, n, &w->opP[b]));
-        w->colP[b] = col[b];
+          for (int k = 0; k < n; ++k) Pb[size_t(i) * n + k] = P[size_t(i) * KY + c0 + k];
+        made = tc64_op_create(Pb, Np, n, &w->opP[b]);
+        w->colP[b] = c0;
       }
     }
+    ICK(made);
     const size_t nw = size_t(m->K) * MW;
     ICK(al(&w->nrm, 9 * size_t(m->K)));
     ICK(al(&w->WU, 4 * nw));
