@@ -298,8 +298,12 @@ typedef struct {
  * time through t^{n-1}, t^n, t^{n+1} (quadratic; linear between t^n and
  * t^{n+1} at step 0), the Helmholtz solve and D take gU at t^{n+1}, G P^n takes
  * gP_n, and the increment takes gP - gP_n on pressure-Dirichlet faces.
- * Workspace is allocated on the first call and kept with mesh_u. Returns the
- * status of a failing solve. */
+ * Workspace is allocated on the first call and kept with mesh_u: 27 K Np
+ * doubles, and from degree 3, with c = (3N + 2) / 2 (integer) cubature points a
+ * direction, (8 c (c + 3) + 9) K + 4 (c (2 c + 3) + Np) min(K, 32768) more (the
+ * second term at most, in equal chunks of the mesh): at degree 8 about 4,600
+ * doubles per triangle up to 32,768 triangles and 2,900 for each one beyond; the
+ * solves' own workspace comes on top. Returns the status of a failing solve. */
 dg_status dg_ins_step(dg_mesh* mesh_u, dg_mesh* mesh_p, dg_ins_state* state, int nsteps, void* stream);
 
 /* Jacobi-preconditioned CG on A(lambda) x = b that allocates nothing.
