@@ -646,10 +646,7 @@ __global__ void k_adv_update(int64_t K, int64_t e0, int64_t n, int64_t ldr, cons
 // kernel (65,536 rows are 3.4 waves of the product's tiles).
 constexpr int64_t kAdvChunk = 32768;
 
-cudaError_t setup_ins(dg_mesh* m) {
-  if (m->ins) return cudaSuccess;
-  InsWorkspace* w = new InsWorkspace();
-  m->ins = w;
+cudaError_t fill_ins(dg_mesh* m, InsWorkspace* w) {
   w->K = m->K;
   w->N = m->N;
   const std::vector<double> h = build_adv_ops(m->ref[m->N], w->L);
@@ -738,6 +735,19 @@ cudaError_t setup_ins(dg_mesh* m) {
     w->tensor = true;
   }
   return cudaSuccess;
+}
+
+// The mesh's workspace, built on the first call. One that could not be built whole is
+// given back: the next call starts afresh.
+cudaError_t setup_ins(dg_mesh* m) {
+  if (m->ins) return cudaSuccess;
+  m->ins = new InsWorkspace();
+  const cudaError_t e = fill_ins(m, m->ins);
+  if (e != cudaSuccess) {
+    free_ins_workspace(m);
+    cudaGetLastError();  // reported by this call, not by a later launch's check
+  }
+  return e;
 }
 
 // A velocity field's point values in the form the fluxes take.

@@ -113,7 +113,8 @@ namespace {
 template <typename T>
 cudaError_t walloc(Workspace* w, T** p, size_t count) {
   cudaError_t e = cudaMalloc(reinterpret_cast<void**>(p), count * sizeof(T) + 16);
-  if (e == cudaSuccess) w->allocs.push_back(*p);
+  if (e != cudaSuccess) *p = nullptr;
+  else w->allocs.push_back(*p);
   if (e == cudaSuccess) e = poison(*p, count * sizeof(T) + 16, POISON_SOLVER);
   return e;
 }
@@ -719,26 +720,13 @@ cudaError_t ensure_transfer(dg_mesh* m, int Nf, int Nc) {
   return cudaSuccess;
 }
 
-cudaError_t setup_workspace(Ctx& c) {
+cudaError_t fill_workspace(Ctx& c, Workspace* w) {
   dg_mesh* m = c.m;
   const dg_solver_opts* o = c.o;
-  Workspace* w = m->ws;
   const bool pmg = o->precond == DG_PREC_PMG;
-  std::string key = std::to_string(c.B) + "/" + std::to_string(pmg) + "/" + std::to_string(o->mixed);
-  if (pmg)
-    for (int l = 0; l < o->nlevels; ++l) key += "," + std::to_string(o->degrees[l]);
-  auto it = m->ws_cache.find(key);
-  if (it != m->ws_cache.end()) {
-    m->ws = it->second;
-    return cudaSuccess;
-  }
-  w = new Workspace();
-  m->ws_cache[key] = w;
-  m->ws = w;
   w->B = c.B;
   w->K = m->K;
   w->N = m->N;
-  w->pmg_key = key;
   const int64_t n = int64_t(m->K) * npd(m->N);
   const size_t nt = size_t(n) * c.B;
   CK(walloc(w, &w->r, nt));
@@ -789,6 +777,33 @@ cudaError_t setup_workspace(Ctx& c) {
     CK(walloc(w, &w->cscal, size_t(c.B) * kNS));
     CK(walloc(w, &w->cpartial, size_t(c.B) * kRedBlocks * 2));
   }
+  return cudaSuccess;
+}
+
+// The workspace of these options, built on their first use. One that could not be
+// built whole is given back: the next call starts afresh.
+cudaError_t setup_workspace(Ctx& c) {
+  dg_mesh* m = c.m;
+  const dg_solver_opts* o = c.o;
+  const bool pmg = o->precond == DG_PREC_PMG;
+  std::string key = std::to_string(c.B) + "/" + std::to_string(pmg) + "/" + std::to_string(o->mixed);
+  if (pmg)
+    for (int l = 0; l < o->nlevels; ++l) key += "," + std::to_string(o->degrees[l]);
+  auto it = m->ws_cache.find(key);
+  if (it != m->ws_cache.end()) {
+    m->ws = it->second;
+    return cudaSuccess;
+  }
+  Workspace* w = new Workspace();
+  const cudaError_t e = fill_workspace(c, w);
+  if (e != cudaSuccess) {
+    free_one(w);
+    cudaGetLastError();  // reported by this call, not by a later launch's check
+    return e;
+  }
+  w->pmg_key = key;
+  m->ws_cache[key] = w;
+  m->ws = w;
   return cudaSuccess;
 }
 
@@ -861,6 +876,7 @@ cudaError_t ensure_amg(Ctx& c, int degree) {
   if (c.g) return cudaErrorStreamCaptureUnsupported;
   amg_free(w->amg);
   w->amg = nullptr;
+  w->amg_key.clear();  // one that fails halfway answers to no key
   CK(amg_build(c.m, degree, c.lambda, c.B, &w->amg, c.st));
   w->amg_key = key;
   ++w->amg_gen;
@@ -1321,13 +1337,13 @@ cudaError_t capture_solve(Ctx& c, const std::string& key) {
 cudaError_t pcg_graph(Ctx& c, const double* b, double* x, int& it, int& coarse_iters) {
   Workspace* w = c.w;
   const size_t nt = size_t(c.m->K) * npd(c.m->N) * c.B;
-  if (!w->gb) {
-    CK(walloc(w, &w->gb, nt));
-    CK(walloc(w, &w->gx, nt));
-    CK(walloc(w, &w->gctr, size_t(G_NCTR)));
-    CK(cudaMallocHost(&w->h_gctr, sizeof(unsigned long long) * G_NCTR));
-    for (cudaStream_t& s : w->cap) CK(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
-  }
+  // (each by itself: a call that failed at one of them is taken up there)
+  if (!w->gb) CK(walloc(w, &w->gb, nt));
+  if (!w->gx) CK(walloc(w, &w->gx, nt));
+  if (!w->gctr) CK(walloc(w, &w->gctr, size_t(G_NCTR)));
+  if (!w->h_gctr) CK(cudaMallocHost(&w->h_gctr, sizeof(unsigned long long) * G_NCTR));
+  for (cudaStream_t& s : w->cap)
+    if (!s) CK(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
   if (!w->gexec || w->gkey != graph_key(c)) {
     CK(warm_applies(c));
     CK(cudaStreamSynchronize(c.st));
