@@ -59,7 +59,7 @@ constexpr int kChunkBytes = kDigits * kChunkSlice;     // 84 KB
 constexpr int kTraceN = 32;                            // output columns (16 boundary nodes) per pass of t64_trace
 constexpr int kTraceStep = kDigits * kTraceN * 16 * 2; // operator block of one pass and 16 columns
 constexpr int trace_smem(int ks) {
-  return kDigits * kT * ks * 32 + (ks != 3 ? 2 : 1) * ks * kTraceStep + 6 * kT * 4 + 6 * 8;
+  return kDigits * kT * ks * 32 + (ks != 3 ? 2 : 1) * ks * kTraceStep + 6 * kT * 4 + 7 * 8;
 }
 constexpr int kCoefs = 12;    // Grr, Grs, Gss | per face nr sJ, ns sJ | per face -sJ tau0
 
@@ -68,8 +68,8 @@ __device__ int g_t64_err;
 using tc::aborted;
 using tc::bar_sync;
 using tc::mbar_arrive;
-__device__ __forceinline__ void wait(uint64_t* b, uint32_t parity, volatile int* abort_flag) {
-  tc::wait_or_abort(b, parity, abort_flag);
+__device__ __forceinline__ bool wait(uint64_t* b, uint32_t parity, volatile int* abort_flag) {
+  return tc::wait_or_abort(b, parity, abort_flag);
 }
 __device__ __forceinline__ int64_t elem_of(int64_t row, int64_t K) { return row < K ? row : row % K; }
 
@@ -144,8 +144,9 @@ __global__ void __launch_bounds__(288, KS <= 3 ? 2 : 1) t64_trace(const TraceArg
   uint8_t* sB = sm + kDigits * kSlice;
   int* pmax = reinterpret_cast<int*>(sB + (kResident ? 2 : 1) * kPass);  // [2 halves][exponent of v, of u, bits of q][kT]
   uint64_t* bars = reinterpret_cast<uint64_t*>(pmax + 6 * kT);
-  uint64_t *ufull = bars, *full = bars + 1, *accf = bars + 2, *acce = bars + 3, *bfull = bars + 4;
-  uint32_t* slot = reinterpret_cast<uint32_t*>(bars + 5);
+  uint64_t *ufull = bars, *full = bars + 1, *accf = bars + 2, *acce = bars + 3, *bfull = bars + 4,
+           *done = bars + 5;
+  uint32_t* slot = reinterpret_cast<uint32_t*>(bars + 6);
   volatile int* abort_flag = reinterpret_cast<int*>(slot + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int N = a.N, Np = (N + 1) * (N + 2) / 2;
@@ -156,6 +157,7 @@ __global__ void __launch_bounds__(288, KS <= 3 ? 2 : 1) t64_trace(const TraceArg
     tc::mbar_init(accf, 1);
     tc::mbar_init(acce, 8);
     tc::mbar_init(bfull, 1);
+    tc::mbar_init(done, 1);
     *abort_flag = 0;
     tc::mbar_init_fence();
   }
@@ -174,7 +176,7 @@ __global__ void __launch_bounds__(288, KS <= 3 ? 2 : 1) t64_trace(const TraceArg
   if (warp == 8) {
     const uint64_t ad = tc::smem_desc(tc::smem_addr(sm), 128, KS * 256);
     const uint64_t bd = tc::smem_desc(tc::smem_addr(sB), 128, 256);
-    uint32_t loads = 0, it = 0, pc = 0;
+    uint32_t loads = 0, bulks = 0, it = 0, pc = 0;
     auto load_ops = [&](int pass0, int n) {
       if (lane == 0) {
         tc::mbar_expect_tx(bfull, n * kPass);
@@ -188,6 +190,7 @@ __global__ void __launch_bounds__(288, KS <= 3 ? 2 : 1) t64_trace(const TraceArg
         tc::mbar_expect_tx(ufull, bytes);
         tc::bulk_g2s(sm, a.u + tile * kT * Np, bytes, ufull);
       }
+      bulks += bytes != 0;
     };
     load_ops(0, kResident ? a.passes : 1);
     if (int64_t(blockIdx.x) < ntiles) load_u(blockIdx.x);
@@ -207,14 +210,18 @@ __global__ void __launch_bounds__(288, KS <= 3 ? 2 : 1) t64_trace(const TraceArg
         __syncwarp();
         const bool last = p + 1 == a.passes;
         if (!kResident || last) {  // the products are done: their operands' space is free
-          wait(accf, pc & 1u, abort_flag);
+          if (!wait(accf, pc & 1u, abort_flag)) continue;
           if (!kResident && a.passes > 1 && (!last || tile + gridDim.x < ntiles)) load_ops(last ? 0 : p + 1, 1);
           if (last && tile + gridDim.x < ntiles) load_u(tile + gridDim.x);
         }
       }
     }
     // nothing is left in flight when the block ends
-    wait(bfull, (loads - 1) & 1u, abort_flag);
+    tc::wait_done(bfull, (loads - 1) & 1u, abort_flag);
+    if (bulks > 0) tc::wait_done(ufull, (bulks - 1) & 1u, abort_flag);
+    if (lane == 0) tc::mma_commit(done);
+    __syncwarp();
+    tc::wait_done(done, 0, abort_flag);
   } else {
     const int e = (warp & 3) * 32 + lane, half = warp >> 2;
     const uint32_t lanebase = uint32_t((warp & 3) * 32) << 16;
@@ -402,7 +409,7 @@ __global__ void __launch_bounds__(kOutThreads, 1) t64_output(const OutArgs a) {
   long long* lut = reinterpret_cast<long long*>(sinfo + kSets * 7 * kT);   // [3][N + 1]: offset of face f's j-th node in Iu
   uint64_t* bars = reinterpret_cast<uint64_t*>(lut + kLut);
   uint64_t *full = bars, *empty = bars + 2, *accf = bars + 4, *acce = bars + 6, *sfull = bars + 8, *sempty = bars + 10,
-           *bfull = bars + 12, *bempty = bars + 12 + kStages;
+           *bfull = bars + 12, *bempty = bars + 12 + kStages, *done = bars + 12 + 2 * kStages;
   uint32_t* slot = reinterpret_cast<uint32_t*>(bars + 24);
   volatile int* abort_flag = reinterpret_cast<int*>(slot + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -421,6 +428,7 @@ __global__ void __launch_bounds__(kOutThreads, 1) t64_output(const OutArgs a) {
       tc::mbar_init(bfull + i, 1);
       tc::mbar_init(bempty + i, 1);
     }
+    tc::mbar_init(done, 1);
     *abort_flag = 0;
     tc::mbar_init_fence();
   }
@@ -447,7 +455,7 @@ __global__ void __launch_bounds__(kOutThreads, 1) t64_output(const OutArgs a) {
       }
     // every copy has landed before the block ends
     for (uint32_t k = n < kStages ? 0 : n - kStages; k < n; ++k)
-      wait(bfull + k % kStages, (k / kStages) & 1u, abort_flag);
+      tc::wait_done(bfull + k % kStages, (k / kStages) & 1u, abort_flag);
   } else if (warp == 16) {
     // ================= products
     const uint64_t ad = tc::smem_desc(tc::smem_addr(sm), 128, 6 * 128);
@@ -473,6 +481,9 @@ __global__ void __launch_bounds__(kOutThreads, 1) t64_output(const OutArgs a) {
         }
       }
     }
+    if (lane == 0) tc::mma_commit(done);
+    __syncwarp();
+    tc::wait_done(done, 0, abort_flag);
   } else if (warp >= 18) {
     // ================= scales
     uint32_t it = 0;

@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(kSlicers + 64, 1) tc64_gemm(int64_t rows, int 
   int* pmax = reinterpret_cast<int*>(sB + kStages * kBBytes);  // [4][kT]
   uint64_t* bars = reinterpret_cast<uint64_t*>(pmax + 4 * kT);
   uint64_t *full = bars, *empty = bars + 2, *accf = bars + 4, *acce = bars + 6, *bfull = bars + 8,
-           *bempty = bars + 8 + kStages;
+           *bempty = bars + 8 + kStages, *done = bars + 8 + 2 * kStages;
   uint32_t* slot = reinterpret_cast<uint32_t*>(bars + 20);
   volatile int* abort_flag = reinterpret_cast<int*>(slot + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -99,6 +99,7 @@ __global__ void __launch_bounds__(kSlicers + 64, 1) tc64_gemm(int64_t rows, int 
       tc::mbar_init(bfull + i, 1);   // the bulk copy
       tc::mbar_init(bempty + i, 1);  // the block's products completed
     }
+    tc::mbar_init(done, 1);
     *abort_flag = 0;
     tc::mbar_init_fence();
   }
@@ -124,7 +125,7 @@ __global__ void __launch_bounds__(kSlicers + 64, 1) tc64_gemm(int64_t rows, int 
       }
     // every copy has landed before the block ends
     for (uint32_t k = g < kStages ? 0 : g - kStages; k < g; ++k)
-      tc::wait_or_abort(bfull + k % kStages, (k / kStages) & 1u, abort_flag);
+      tc::wait_done(bfull + k % kStages, (k / kStages) & 1u, abort_flag);
   } else if (warp == kSlicers / 32) {
     // ================= products
     uint32_t g = 0, pass = 0, it = 0;
@@ -157,6 +158,9 @@ __global__ void __launch_bounds__(kSlicers + 64, 1) tc64_gemm(int64_t rows, int 
         }
       }
     }
+    if (lane == 0) tc::mma_commit(done);
+    __syncwarp();
+    tc::wait_done(done, 0, abort_flag);
   } else {
     // ================= slicing and epilogue
     const int e = (warp & 3) * 32 + lane;

@@ -120,8 +120,17 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, uint64_t
 // returns at once: all warps run to the end of their loops (their named
 // barriers stay matched) and the block ends.
 __device__ __forceinline__ bool aborted(volatile int* flag) { return __any_sync(0xffffffffu, *flag != 0); }
-__device__ __forceinline__ void wait_or_abort(uint64_t* b, uint32_t parity, volatile int* abort_flag) {
-  if (!aborted(abort_flag) && !mbar_wait(b, parity)) *abort_flag = 1;
+// (False if it gave up, here or before.)
+__device__ __forceinline__ bool wait_or_abort(uint64_t* b, uint32_t parity, volatile int* abort_flag) {
+  if (aborted(abort_flag)) return false;
+  if (mbar_wait(b, parity)) return true;
+  *abort_flag = 1;
+  return false;
+}
+// Before a block ends: its last copies and products have to be done also when a wait
+// gave up, or they would reach memory that is another block's by then (bounded too).
+__device__ __forceinline__ void wait_done(uint64_t* b, uint32_t parity, volatile int* abort_flag) {
+  if (!mbar_wait(b, parity)) *abort_flag = 1;
 }
 __device__ __forceinline__ void mbar_arrive(uint64_t* b) {
   asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.shared::cta.b64 st, [%0];\n}\n" ::"r"(smem_addr(b)) : "memory");
