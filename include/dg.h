@@ -62,7 +62,7 @@ typedef enum {
 
 /* DG_F64: FP64 in/out with the mesh's FP64 kernel (DG_KERNEL_* below; built-in:
  *         from degree 3 up the dense products run on the FP16 tensor cores with
- *         exact integer slicing, relative error ~1e-15 of |A||u|; that path scales
+ *         exact integer slicing (accuracy: DG_KERNEL_TC64 below); that path scales
  *         each element's data by a power of two and rebuilds results from their
  *         exponent bits, so it takes finite fields whose nonzero element
  *         magnitudes lie between about 1e-250 and 1e250);
@@ -95,8 +95,15 @@ typedef struct dg_mesh dg_mesh; /* opaque; owned by the library until dg_mesh_de
  *   DG_KERNEL_TC64:   FP64 only: both products on the Blackwell tensor cores (tcgen05,
  *                     exact integer slicing, 7 digits of 8 bits, accumulators in tensor
  *                     memory) and the pointwise stage in 64-bit fixed point, each element's
- *                     data at its own power-of-two scale; all degrees. An element with an
- *                     infinity or a NaN, and its neighbours, give NaN.
+ *                     data at its own power-of-two scale; all degrees. Error against
+ *                     exact arithmetic on jittered meshes, N = 1..10: below 5e-15 of
+ *                     |A||u| in the 2-norm and 4e-14 of (|A||u|)_i entry by entry. An
+ *                     element's scale is set by itself and its neighbours: next to
+ *                     elements 2^60 larger an entry's error reaches 3e-13 of (|A||u|)_i
+ *                     (the tile kernel's 2e-13). The entries of an element sum to its
+ *                     flux, what one element loses its neighbours gain, up to the
+ *                     rounding of the entries. An element with an infinity or a NaN, and
+ *                     its neighbours, give NaN.
  *                     Handles finite fields whose magnitudes stay within the double range
  *                     at every stage (about 1e-250..1e250, as DG_KERNEL_TENSOR). */
 enum { DG_KERNEL_AUTO = 0, DG_KERNEL_TILE = 1, DG_KERNEL_GEMM = 2, DG_KERNEL_TENSOR = 3, DG_KERNEL_EPT = 4,
@@ -322,7 +329,9 @@ dg_status dg_ins_step(dg_mesh* mesh_u, dg_mesh* mesh_p, dg_ins_state* state, int
  * (4 B + 1) K Np words for the CG vectors and the Jacobi inverse, a few per
  * right-hand side, and the apply's scratch: B K (2 Np + 15 (N + 1)) words
  * (B K (3 Np + 15 (N + 1)) with lambda != 0) for the tcgen05 FP64 kernel,
- * the default from degree 3, or 2 B K Np (3 B K Np) for the mma.sync ones.
+ * the default from degree 3 (it uses B K (Np + 3 (N + 1) + 3) of them; the
+ * requirement, and with it what is rejected, stays as published), or 2 B K Np
+ * (3 B K Np) for the mma.sync ones.
  * At B = 1 and N = 8 that is about K <= 9,200 triangles (lambda = 0) or
  * 8,400; larger problems are rejected with DG_ERR_ARG before any device
  * work. The

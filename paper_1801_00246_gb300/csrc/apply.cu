@@ -387,9 +387,11 @@ DG_TE_DECL(9)
 // tensor cores with exact integer slicing (apply_tensor.cu; FP64 and FP32), or one element per
 // thread (apply_ept.cu). DG_F64_DFMA forces the tile kernel in FP64.
 
-// Built-in kernel per degree and precision (the measured winners on the
-// 524,288-triangle workload; dg_autotune replaces them per mesh). Above degree
-// 8 the tcgen05 FP32 kernel's operands no longer fit in tensor memory.
+// Built-in kernel per degree and precision (dg_autotune replaces them per mesh): the
+// measured winners on the 524,288-triangle workload, but for FP64 at degree 2, where
+// the tcgen05 kernel now takes 263 us against the element-per-thread kernel's 617
+// (degree 1: 203 against 195), and by 2 % FP32 at degree 3. Above degree 8 the tcgen05
+// FP32 kernel's operands no longer fit in tensor memory.
 int default_kernel(int degree, bool f64) {
   if (f64) return degree >= 3 ? DG_KERNEL_TC64 : DG_KERNEL_EPT;
   if (degree <= 3) return DG_KERNEL_EPT;

@@ -32,9 +32,12 @@
 // (a bias that all elements share would be a smooth source, which a solve
 // amplifies), and the digit products left out weigh 2^-60 of the largest. Against
 // 64-bit arithmetic the relative error of an apply is 0.9e-15 (N = 3) to 1.2e-14
-// (N = 10) on random fields, 1.5 times the FP64-pipe kernel's.
+// (N = 10) on random fields, 1.5 times the FP64-pipe kernel's. What an apply yields
+// summed over an element (its flux balance) matters more to a solve than any entry:
+// the operator's columns sum to what the basis says exactly (tables64.cpp), so a
+// column's rounding drops out of that sum.
 // 524,288 triangles, N = 8: 1714 us and 2.6 GB of traffic with the pointwise stage
-// in float-float between two generic products and X in memory; 776 us and 1.0 GB now.
+// in float-float between two generic products and X in memory; 780 us and 1.0 GB now.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -79,7 +82,7 @@ __device__ __forceinline__ int node_of(int N, int f, int j) {  // local node of 
 }
 
 // Per-element coefficients in fixed point, one exponent for each kind (|c| < 2^e):
-// word i of element e at tab[i K + e], exponents in ex (G, n sJ, sJ tau0, J).
+// word i of element e at tab[i K + e], exponents in ex (G, n sJ, sJ tau0).
 __global__ void k_fix_geometry(int64_t K, const double* __restrict__ gx, int2* __restrict__ tab,
                                short4* __restrict__ ex) {
   const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -101,7 +104,7 @@ __global__ void k_fix_geometry(int64_t K, const double* __restrict__ gx, int2* _
     const Split s = fx::split(fx::fix<62>(c[i], i < 3 ? eg : (i < 9 ? ec : et)));
     tab[int64_t(i) * K + e] = make_int2(s.h, s.l);
   }
-  ex[e] = make_short4(short(eg), short(ec), short(et), short(fx::exp_bound(g[0])));
+  ex[e] = make_short4(short(eg), short(ec), short(et), 0);
 }
 
 __device__ __forceinline__ Split coef(const int2* p) {

@@ -577,7 +577,7 @@ template <typename T, int NPC>
 void launch_transfer_n(int Npf, int64_t nE, const T* P, const T* a, const T* b, T* out, cudaStream_t st) {
   auto bytes = [&](int E) { return (size_t(E) * Npf + size_t(Npf) * pad4(NPC)) * sizeof(T); };
   int E = 128;
-  while (E > 32 && (bytes(E) > 48 * 1024 || nE / E < 304)) E /= 2;  // (two blocks per SM where the mesh allows)
+  while (E > 32 && (bytes(E) > 48 * 1024 || nE / E < 2 * 152)) E /= 2;  // (two blocks on each of the 152 SMs where the mesh allows)
   const unsigned g = unsigned((nE + E - 1) / E);
   if (b) k_sub_restrict<T, NPC><<<g, E, bytes(E), st>>>(Npf, nE, P, a, b, out);
   else k_prolong<T, NPC><<<g, E, bytes(E), st>>>(Npf, nE, P, a, out);
