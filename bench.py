@@ -45,9 +45,9 @@ PMG_DEGREES = [8, 4, 2, 1]
 CHEB = 3           # Chebyshev-Jacobi smoothing degree per pre/post smoothing
 COARSE_PASSES = 1  # degree-1 coarse solve: one AMG-preconditioned CG pass (a scaled AMG V-cycle)
 # DRAM bytes per FP64 apply at N=8 from the latest ncu capture of the current
-# default kernels (tcgen05: boundary derivatives 0.479 GB, output product 0.522 GB);
+# default kernels (tcgen05: boundary derivatives 0.479 GB, output product 0.530 GB);
 # None while the kernels differ from that capture
-TENSOR_APPLY_TRAFFIC = 1.001e9
+TENSOR_APPLY_TRAFFIC = 1.010e9
 
 
 # apply kernels by DG_KERNEL_* value

@@ -392,7 +392,7 @@ __host__ __device__ constexpr int out_smem(int nc) {
 // its neighbours' exponents, the coefficients at that scale and the shifts that
 // bring both sides of a face to a common one (done by every thread that forms
 // columns, this took a third of the kernel's instructions).
-// 524,288 triangles, N = 8: 539 us, in place of 234 (face terms) and 667 (product).
+// 524,288 triangles, N = 8: 553 us, in place of 234 (face terms) and 667 (product).
 // Nothing is near its limit: without the loads about 485, without the stores 495, without
 // the products 390, with none of them 275 and as an empty pipeline 170 us; a chunk's
 // forming, slicing and products follow each other and only two chunks fit in shared
