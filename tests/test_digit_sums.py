@@ -3,8 +3,6 @@ result could leave the integers that FP32 holds exactly, whatever the data."""
 import os
 import subprocess
 
-import pytest
-
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 PKG = os.path.join(ROOT, "paper_1801_00246_gb300")
 # A row of n entries between 1/2 and 3/4: its exponent is that of its absolute sum less 6,

@@ -5,8 +5,6 @@ no entry is further from the product in doubles than the rounding of either."""
 import os
 import subprocess
 
-import pytest
-
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CSRC = os.path.join(ROOT, "paper_1801_00246_gb300", "csrc")
 SOURCE = r"""
